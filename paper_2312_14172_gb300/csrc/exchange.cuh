@@ -1,0 +1,221 @@
+// exchange.cuh -- device pieces of the momentum exchange (Eq. hlbm:mea,
+// Sec. 3.2) of one particle from the populations alone, on the library's
+// blocked storage.
+#pragma once
+#include "lbm_common.cuh"
+
+namespace hlbm {
+
+constexpr int XCH_MAX_T = 256;  // threads per block: 128 or 256
+
+// The bounding box [floor(X - r_c), ceil(X + r_c)] of a particle (clipped at
+// walls and to a slab's owned planes) and, per plane of the block, its rows
+// that meet the circumscribed sphere (+-1 cell of margin), flattened: row r
+// of plane j covers the flat cells [start[j][r], start[j][r + 1]) from
+// unwrapped x = lo[0] + xa[j][r] on.
+struct ExchangeBox {
+  int lo[3], ext[3];
+  float x0, rc2;
+  float dy[MAX_PLANES], dz[MAX_PLANES];
+  unsigned short start[MAX_PLANES][MAX_PLANES + 2];
+  signed char xa[MAX_PLANES][MAX_PLANES];
+};
+
+// Fills the box for planes [q0, q0 + nq); called by all threads of the block
+// (it synchronises).  The only FP64 arithmetic of the walk, and done once
+// per block, a lane per axis, row or plane: an FP64 instruction holds a
+// GB300 SM's narrow pipe for 16 cycles per warp however few lanes run.
+__device__ __forceinline__ void exchange_box(const PartArgs& a, int p, const BoxDesc& bd, int q0, int nq,
+                                             ExchangeBox& b) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const double* Xp = a.P + (long long)PF_X * a.cap + p;
+  if (tid < 3) {
+    const int n = tid == 0 ? bd.nx : (tid == 1 ? bd.ny : bd.nz);
+    const double X = Xp[(long long)tid * a.cap], rc = a.P[(long long)PF_RC * a.cap + p];
+    int l = 0, h = -1;
+    if (X > -1.0e6 && X < 1.0e6) {  // no interior cells otherwise (the update flags it)
+      l = (int)floor(X - rc);
+      h = (int)ceil(X + rc);
+      if ((bd.bc >> tid) & 1) {
+        const bool cut = tid == 2 && (bd.bc & BC_CUT_Z);  // owned planes only
+        l = max(l, cut ? bd.own_lo : 0);
+        h = min(h, cut ? bd.own_hi - 1 : n - 1);
+      }
+    } else {
+      atomicOr(a.status, ST_UNSTABLE);
+    }
+    b.lo[tid] = l;
+    b.ext[tid] = min(max(h - l + 1, 0), MAX_PLANES);
+    if (tid == 0) {
+      b.x0 = (float)X;
+      b.rc2 = (float)(rc * rc) * 1.0001f + 1e-3f;
+    }
+  }
+  __syncthreads();
+  {
+    const int j = tid & (MAX_PLANES - 1);  // warps 0, 1: rows; 2, 3: planes
+    if (tid < 2 * MAX_PLANES) {
+      const int ax = tid < MAX_PLANES ? 1 : 2;
+      const float d = (float)((double)(b.lo[ax] + j) - Xp[(long long)ax * a.cap]);
+      (ax == 1 ? b.dy : b.dz)[j] = d;
+    }
+  }
+  __syncthreads();
+  for (int j = warp; j < nq; j += blockDim.x >> 5) {
+    if (q0 + j >= b.ext[2]) break;
+    int len[2], xa[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int iy = lane + 32 * u;
+      const float dy = b.dy[iy], dz = b.dz[q0 + j];
+      len[u] = xa[u] = 0;
+      const float d2 = __fmaf_rn(dz, dz, __fmul_rn(dy, dy));
+      if (iy < b.ext[1] && d2 < b.rc2) {
+        const float s = sqrtf(b.rc2 - d2);
+        const int x = max(b.lo[0], (int)floorf(b.x0 - s) - 1);
+        const int xb = min(b.lo[0] + b.ext[0] - 1, (int)ceilf(b.x0 + s) + 1);
+        len[u] = max(xb - x + 1, 0);
+        xa[u] = min(max(x - b.lo[0], 0), MAX_PLANES - 1);
+      }
+    }
+    int s0 = len[0], s1 = len[1];
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int t0 = __shfl_up_sync(0xffffffffu, s0, off);
+      const int t1 = __shfl_up_sync(0xffffffffu, s1, off);
+      if (lane >= off) { s0 += t0; s1 += t1; }
+    }
+    s1 += __shfl_sync(0xffffffffu, s0, 31);
+    b.start[j][lane] = (unsigned short)(s0 - len[0]);
+    b.start[j][lane + 32] = (unsigned short)(s1 - len[1]);
+    b.xa[j][lane] = (signed char)xa[0];
+    b.xa[j][lane + 32] = (signed char)xa[1];
+    if (lane == 31) b.start[j][MAX_PLANES] = (unsigned short)s1;
+  }
+  __syncthreads();
+}
+
+// Sum over the links of an interior cell (used form of Eq. hlbm:mea):
+//   sum_i (c_i - u_p) f_i(x) + (c_i + u_p) f_ibar(x - c_i)
+// = sum_i c_i (in_i + out_i) - u_p sum_i (in_i - out_i), in_i = f_i(x), out_i
+// = f_ibar(x - c_i).  This is the printed per-cell sum with the opposite
+// sign: on post-streaming populations the printed sum is what the cell hands
+// to the fluid, and the particle feels the reverse.  In both AA parities the
+// pair of slots is {slot i of x, slot ibar of x - c_i}; only which of the two
+// is the arrival differs.  A link to a node beyond a wall carries no fluid
+// and is left out; on deviations d = f - w that leaves -2 c_i w_i per omitted
+// link, because the weights of all 18 links sum to zero.  All 36 loads are
+// independent of one another and of any branch.
+template <typename S, int PAR, bool W>
+__device__ __forceinline__ void exchange_links(const S* f, const BoxDesc& bd, int x, int y, int z, float scale,
+                                               float inv_s, float (&F)[3], float& mgain) {
+  const RowBlocks rb = row_blocks<W>(bd, x, y, 1);
+  int zb[3];
+  slice_blocks<W>(bd, z, zb);
+  const S* own = cell_ptr(f, zb[1] + rb.yb[1] + rb.xb, rb.xin);
+  float va[Q], vb[Q];
+  unsigned walls = 0;  // bit i: x - c_i lies beyond a wall
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    const int by = rb.yb[1 - cy(i)], bz = zb[1 - cz(i)];
+    const bool wall = W && (by < 0 || bz < 0 || (cx(i) > 0 && rb.wl) || (cx(i) < 0 && rb.wr));
+    const int dx = cx(i) > 0 ? rb.dl : (cx(i) < 0 ? rb.dr : 0);
+    const S* nb = wall ? own : cell_ptr(f, bz + by + rb.xb, rb.xin) + dx;
+    if (wall) walls |= 1u << i;
+    va[i] = Pop<S>::ld_raw(own + i * VB);
+    vb[i] = Pop<S>::ld_raw(nb + opp(i) * VB);
+  }
+  // in stored units; the scale is a power of two
+  F[0] = F[1] = F[2] = 0.0f;
+  mgain = 0.0f;
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    const float in = PAR == 0 ? va[i] : vb[i], out = PAR == 0 ? vb[i] : va[i];
+    float sum = in + out, dif = in - out;
+    if (W && ((walls >> i) & 1u)) {
+      sum = Pop<S>::SCALED ? -2.0f * (float)wq(i) * scale : -2.0f * (float)wq(i);
+      dif = 0.0f;
+    }
+    if (cx(i)) F[0] += (float)cx(i) * sum;
+    if (cy(i)) F[1] += (float)cy(i) * sum;
+    if (cz(i)) F[2] += (float)cz(i) * sum;
+    mgain += dif;
+  }
+  if (Pop<S>::SCALED) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) F[j] = __fmul_rn(F[j], inv_s);
+    mgain = __fmul_rn(mgain, inv_s);
+  }
+}
+
+// One warp's share of one group of planes [j0, j1) of the block's box: flat
+// cells 32 vw + lane, + 128, ... of each plane, as if four warps (vw = 0 .. 3)
+// walked the group together; per-thread sums (F, T) in FP32 over the cells
+// and then the planes, added over the warp by shuffles.  The split and the
+// order are part of the result (a force to the last bit): warps may take the
+// shares in any order.
+template <typename S, int PAR, bool WALLS, bool GRIDS>
+__device__ __forceinline__ void exchange_share(const PartArgs& a, const Rec& R, const BoxDesc& bd,
+                                               const ExchangeBox& b, int q0, int j0, int j1, int vw, float (&v)[6]) {
+  const S* f = reinterpret_cast<const S*>(a.f);
+  const int lane = threadIdx.x & 31;
+  const GridSet gs = GRIDS ? a.grids : GridSet{};
+  bool any = false;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) v[k] = 0.0f;
+  for (int j = j0; j < j1; ++j) {
+    const int zu = b.lo[2] + q0 + j;
+    const int z = zu < 0 ? zu + bd.nz : (zu >= bd.nz ? zu - bd.nz : zu);
+    const int total = b.start[j][MAX_PLANES];
+    float s[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int q = 32 * vw + lane; q < total; q += 128) {
+      int r = 0;  // the row holding flat index q: the last one starting at or before it
+#pragma unroll
+      for (int step = 32; step > 0; step >>= 1)
+        if (b.start[j][r + step] <= q) r += step;
+      const int xu = b.lo[0] + b.xa[j][r] + (q - b.start[j][r]);
+      const int yu = b.lo[1] + r;
+      const int x = xu < 0 ? xu + bd.nx : (xu >= bd.nx ? xu - bd.nx : xu);
+      const int y = yu < 0 ? yu + bd.ny : (yu >= bd.ny ? yu - bd.ny : yu);
+      float rr[3];
+      const bool in = (unsigned)x < (unsigned)bd.nx && (unsigned)y < (unsigned)bd.ny &&
+                      (unsigned)z < (unsigned)bd.nz && inside_fp32(R, bd, x, y, z, rr, gs);
+      auto cell = [&](auto wtag) {
+        float Fc[3], mg;
+        exchange_links<S, PAR, decltype(wtag)::value>(f, bd, x, y, z, a.scale, a.inv_scale, Fc, mg);
+        const float upx = R.u[0] + (R.w[1] * rr[2] - R.w[2] * rr[1]);
+        const float upy = R.u[1] + (R.w[2] * rr[0] - R.w[0] * rr[2]);
+        const float upz = R.u[2] + (R.w[0] * rr[1] - R.w[1] * rr[0]);
+        Fc[0] -= upx * mg;
+        Fc[1] -= upy * mg;
+        Fc[2] -= upz * mg;
+        s[0] += Fc[0];
+        s[1] += Fc[1];
+        s[2] += Fc[2];
+        s[3] += rr[1] * Fc[2] - rr[2] * Fc[1];
+        s[4] += rr[2] * Fc[0] - rr[0] * Fc[2];
+        s[5] += rr[0] * Fc[1] - rr[1] * Fc[0];
+      };
+      if (WALLS) {
+        // only cells next to a wall take the wall selects
+        const bool edge = ((bd.bc & 1) && (x == 0 || x == bd.nx - 1)) || ((bd.bc & 2) && (y == 0 || y == bd.ny - 1)) ||
+                          ((bd.bc & 4) && (z == 0 || z == bd.nz - 1));
+        if (in && edge) cell(std::integral_constant<bool, WALLS>{});
+        if (in && !edge) cell(std::integral_constant<bool, false>{});
+      } else if (in) {
+        cell(std::integral_constant<bool, false>{});
+      }
+      any = any || in;
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) v[k] += s[k];
+  }
+  if (__any_sync(0xffffffffu, any)) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+  }
+}
+
+}  // namespace hlbm

@@ -39,7 +39,7 @@ struct Layout {
   long long nblocks = 0, ncell = 0, ntiles = 0, stage_cells = 0;
   int cap = 0, bin_cap = 0;
   size_t off_f, off_boxes, off_P, off_shape, off_box, off_rec, off_part, off_acc, off_chp, off_chq,
-      off_pc0, off_pnc, off_done, off_lcnt, off_lidx, off_lmom, off_cnt[2], off_ids[2], off_status,
+      off_pc0, off_pnc, off_ppl, off_done, off_lcnt, off_lidx, off_lmom, off_cnt[2], off_ids[2], off_status,
       off_stage, off_gdesc, off_gvals, total;
   long long grid_floats = 0;
   long long ilist_cap = 0;
@@ -106,6 +106,7 @@ bool make_layout(int nb, const hlbm_box* boxes, const hlbm_params* prm, Layout& 
   L.off_chq = o; o = align_up(o + sizeof(int) * MAX_PLANES * (size_t)L.cap);
   L.off_pc0 = o; o = align_up(o + sizeof(int) * (size_t)L.cap);
   L.off_pnc = o; o = align_up(o + sizeof(int) * (size_t)L.cap);
+  L.off_ppl = o; o = align_up(o + sizeof(int) * (size_t)L.cap);
   L.off_done = o; o = align_up(o + sizeof(int) * (size_t)L.cap);
   // interior-cell list for the momentum exchange from moments, in
   // ILIST_STRIPES stripes: together room for half of all cells (more than
@@ -153,6 +154,7 @@ struct hlbm_ctx {
   int* chunk_q = nullptr;
   int* p_chunk0 = nullptr;
   int* p_nchunk = nullptr;
+  int* p_planes = nullptr;
   int* done = nullptr;
   int* ilist_count = nullptr;
   int2* ilist_idx = nullptr;
@@ -163,8 +165,9 @@ struct hlbm_ctx {
   // with, still in L2); larger lattices gain nothing and keep one order
   bool reverse_odd = false;
   int nchunks = 0;
-  std::vector<int> h_nchunk;  // bounding-box planes per particle
-  int mea_planes = 1;         // bounding-box planes per momentum-exchange block
+  std::vector<int> h_planes;    // bounding-box planes per particle
+  int mea_group = 1;            // planes whose cells are summed together
+  int mea_threads = 128;        // threads per momentum-exchange block
   int mea_mode = HLBM_MEA_KERNEL;
   int* cnt[2] = {nullptr, nullptr};
   int* ids[2] = {nullptr, nullptr};
@@ -286,7 +289,9 @@ static PartArgs part_args(const hlbm_ctx* h, int parity) {
   a.p_chunk0 = h->p_chunk0;
   a.p_nchunk = h->p_nchunk;
   a.nchunks = h->nchunks;
-  a.mea_planes = h->mea_planes;
+  a.p_planes = h->p_planes;
+  a.mea_group = h->mea_group;
+  a.mea_threads = h->mea_threads;
   a.partial = h->partial;
   a.done = h->done;
   a.acc = h->acc;
@@ -327,7 +332,7 @@ static cudaError_t enqueue_step(hlbm_ctx* h, int parity, bool moments, cudaStrea
     pa.from_acc = moments ? 1 : 0;
     if (moments) {
       if ((e = launch_mea_moments(la, h->prm.precision, parity, h->walls, h->nsm, s)) != cudaSuccess) return e;
-    } else if ((e = launch_mea(pa, h->prm.precision, parity, s)) != cudaSuccess) {
+    } else if ((e = launch_mea(pa, h->prm.precision, parity, h->walls, s)) != cudaSuccess) {
       return e;
     }
     if ((e = launch_contact(pa, s)) != cudaSuccess) return e;
@@ -484,6 +489,7 @@ int hlbm_init_batch(hlbm_handle* out, int nboxes, const hlbm_box* boxes, const h
   h->chunk_q = (int*)(h->buf + h->L.off_chq);
   h->p_chunk0 = (int*)(h->buf + h->L.off_pc0);
   h->p_nchunk = (int*)(h->buf + h->L.off_pnc);
+  h->p_planes = (int*)(h->buf + h->L.off_ppl);
   h->done = (int*)(h->buf + h->L.off_done);
   h->ilist_count = (int*)(h->buf + h->L.off_lcnt);
   h->ilist_idx = h->L.ilist_cap > 0 ? (int2*)(h->buf + h->L.off_lidx) : nullptr;
@@ -797,6 +803,48 @@ int hlbm_add_grid(hlbm_handle h, int nx, int ny, int nz, double spacing, const f
   return HLBM_OK;
 }
 
+// The order and the blocks of the bounding-box momentum exchange.
+// mea_group, the planes whose cells a group of four warps sums together, is
+// part of the result (to the last bit of a force): one plane up to four
+// resident waves of one-plane blocks, then up to three.  The blocks are not:
+// few particles are split over several blocks of 256 threads to shorten one
+// particle's latency, many take one block of 128 threads each, where no
+// block waits for another's sum (us, 256 threads and 6 planes against 128
+// and 24: 200 spheres FP32 35 / 57, 2000 ellipsoids and cuboids 249 / 170,
+// 50 000 spheres FP16 2869 / 1470).
+static int plan_exchange(hlbm_ctx* h) {
+  const int nsm = h->nsm > 0 ? h->nsm : 152;
+  long long planes = 0;
+  for (int p : h->h_planes) planes += p;
+  const int G = (int)std::min(3LL, std::max(1LL, planes / (4LL * nsm * 8)));
+  h->mea_group = G;
+  const bool few = h->np < 4 * nsm;
+  h->mea_threads = few ? 256 : 128;
+  const int per = few ? 6 : 24;
+  std::vector<int> cp, cq, c0(h->np), cn(h->np), pl(h->np);
+  for (int p = 0; p < h->np; ++p) {
+    // whole groups per block, about `per` planes
+    const int groups = (h->h_planes[p] + G - 1) / G;
+    const int parts = std::max(1, (h->h_planes[p] + per - 1) / per);
+    const int gp = (groups + parts - 1) / parts;
+    pl[p] = gp * G;
+    cn[p] = (groups + gp - 1) / gp;
+    c0[p] = (int)cp.size();
+    for (int k = 0; k < cn[p]; ++k) {
+      cp.push_back(p);
+      cq.push_back(k * pl[p]);
+    }
+  }
+  h->nchunks = (int)cp.size();
+  CK(cudaMemcpyAsync(h->chunk_p, cp.data(), sizeof(int) * cp.size(), cudaMemcpyHostToDevice, h->stream));
+  CK(cudaMemcpyAsync(h->chunk_q, cq.data(), sizeof(int) * cq.size(), cudaMemcpyHostToDevice, h->stream));
+  CK(cudaMemcpyAsync(h->p_chunk0, c0.data(), sizeof(int) * c0.size(), cudaMemcpyHostToDevice, h->stream));
+  CK(cudaMemcpyAsync(h->p_nchunk, cn.data(), sizeof(int) * cn.size(), cudaMemcpyHostToDevice, h->stream));
+  CK(cudaMemcpyAsync(h->p_planes, pl.data(), sizeof(int) * pl.size(), cudaMemcpyHostToDevice, h->stream));
+  CK(cudaStreamSynchronize(h->stream));
+  return HLBM_OK;
+}
+
 int hlbm_add_particles(hlbm_handle h, int n, const int* box_id, const int* shape,
                        const double* shape_params, const double* X, const double* U,
                        const double* omega, const double* quat, const double* rho_p) {
@@ -901,34 +949,9 @@ int hlbm_add_particles(hlbm_handle h, int n, const int* box_id, const int* shape
   h->hst_valid = false;
   h->h_shape.insert(h->h_shape.end(), sh.begin(), sh.end());
   h->h_box.insert(h->h_box.end(), bx.begin(), bx.end());
-  h->h_nchunk.insert(h->h_nchunk.end(), nch.begin(), nch.end());
-  {
-    // one momentum-exchange block per particle and run of mea_planes
-    // bounding-box planes: one plane while the blocks of one plane each fill
-    // the GPU at most four times (the walk is latency-bound and a block's
-    // fixed cost is then spread over few waves), up to three for many
-    // particles, where each block's fixed cost counts in every wave
-    long long planes = 0;
-    for (int q = 0; q < h->np; ++q) planes += h->h_nchunk[q];
-    const long long resident = (long long)(h->nsm > 0 ? h->nsm : 152) * MEA_MINBLOCKS;
-    h->mea_planes = (int)std::min(3LL, std::max(1LL, planes / (4 * resident)));
-    const int G = h->mea_planes;
-    std::vector<int> cp, cq, c0(h->np), cn(h->np);
-    for (int q = 0; q < h->np; ++q) {
-      c0[q] = (int)cp.size();
-      cn[q] = (h->h_nchunk[q] + G - 1) / G;
-      for (int k = 0; k < cn[q]; ++k) {
-        cp.push_back(q);
-        cq.push_back(k * G);
-      }
-    }
-    h->nchunks = (int)cp.size();
-    CK(cudaMemcpyAsync(h->chunk_p, cp.data(), sizeof(int) * cp.size(), cudaMemcpyHostToDevice, h->stream));
-    CK(cudaMemcpyAsync(h->chunk_q, cq.data(), sizeof(int) * cq.size(), cudaMemcpyHostToDevice, h->stream));
-    CK(cudaMemcpyAsync(h->p_chunk0, c0.data(), sizeof(int) * c0.size(), cudaMemcpyHostToDevice, h->stream));
-    CK(cudaMemcpyAsync(h->p_nchunk, cn.data(), sizeof(int) * cn.size(), cudaMemcpyHostToDevice, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-  }
+  h->h_planes.insert(h->h_planes.end(), nch.begin(), nch.end());
+  rc = plan_exchange(h);
+  if (rc != HLBM_OK) return rc;
   CK(launch_records(part_args(h, 0), h->stream));
   CK(cudaStreamSynchronize(h->stream));
   drop_graphs(h);
@@ -1093,7 +1116,7 @@ int hlbm_step_forces(hlbm_handle h, double* F, double* T) {
         T[3 * k + j] = (double)acc[6 * (size_t)k + 3 + j] * unit;
       }
   } else {
-    CK(launch_mea(part_args(h, parity), h->prm.precision, parity, h->stream));
+    CK(launch_mea(part_args(h, parity), h->prm.precision, parity, h->walls, h->stream));
     std::vector<double> rows((size_t)6 * n);
     CK(cudaMemcpy2DAsync(rows.data(), sizeof(double) * n, h->P + (size_t)PF_F * h->L.cap, sizeof(double) * h->L.cap,
                          sizeof(double) * n, 6, cudaMemcpyDeviceToHost, h->stream));
@@ -1464,7 +1487,7 @@ int hlbm_kernel_times(hlbm_handle h, int nsteps, float ms[3]) {
     const bool fused = h->moments_valid && h->np > 0;
     pa.from_acc = fused ? 1 : 0;
     cudaEventRecord(ev[0], h->stream);
-    if (h->np > 0 && !fused) launch_mea(pa, h->prm.precision, parity, h->stream);
+    if (h->np > 0 && !fused) launch_mea(pa, h->prm.precision, parity, h->walls, h->stream);
     if (h->np > 0 && fused) launch_mea_moments(lbm_args(h, parity), h->prm.precision, parity, h->walls, h->nsm, h->stream);
     cudaEventRecord(ev[1], h->stream);
     if (h->np > 0) launch_contact(pa, h->stream);

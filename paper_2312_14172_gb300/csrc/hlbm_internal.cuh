@@ -97,13 +97,6 @@ __device__ __forceinline__ void cell_coords(const BoxDesc& bd, unsigned c, int& 
 // cells of the owned planes [own_lo, own_hi) enter the momentum exchange.
 constexpr int BC_CUT_Z = 8;
 
-// resident blocks per SM of the bounding-box momentum exchange (64
-// registers): the walk is latency-bound, and more resident blocks beat the
-// spills this costs
-#ifndef HLBM_MEA_MINBLOCKS
-#define HLBM_MEA_MINBLOCKS 8
-#endif
-constexpr int MEA_MINBLOCKS = HLBM_MEA_MINBLOCKS;
 __host__ __device__ __forceinline__ bool owned_plane(const BoxDesc& bd, int z) {
   return !(bd.bc & BC_CUT_Z) || (z >= bd.own_lo && z < bd.own_hi);
 }
@@ -131,9 +124,8 @@ enum {
   PF_COUNT = 43
 };
 
-// the momentum-exchange kernel gives every z-plane of a particle's bounding
-// box its own thread block; a particle spans at most this many planes
-// (circumscribed radius <= 30 cells)
+// a particle's bounding box spans at most this many planes (circumscribed
+// radius <= 30 cells)
 constexpr int MAX_PLANES = 64;
 
 // stripes of the list of interior cells (a power of two)
@@ -383,14 +375,16 @@ struct PartArgs {
   // momentum exchange input
   const void* f;            // populations, blocked layout
   float scale, inv_scale;
-  // momentum-exchange kernel: one block per (particle, bounding-box plane)
+  // momentum-exchange kernel: one block per particle and run of planes
   const int* chunk_p;       // [chunks] particle of the block
-  const int* chunk_q;       // [chunks] plane of the block
+  const int* chunk_q;       // [chunks] first plane of the block
   const int* p_chunk0;      // [cap] first block of a particle
   const int* p_nchunk;      // [cap] blocks of a particle
+  const int* p_planes;      // [cap] bounding-box planes per block of a particle
+  int mea_group;            // planes whose cells are summed together
   int nchunks;
-  int mea_planes;           // bounding-box planes per momentum-exchange block
-  double* partial;          // [chunks][6] FP64 partial force/torque sums
+  int mea_threads;          // threads per momentum-exchange block
+  double* partial;          // [cap][MAX_PLANES][6] FP64 sums of the groups of planes
   int* done;                // [cap] blocks finished per particle (reset to 0)
   // the same sums added up by the moments-mode momentum exchange from the
   // moments the previous collision recorded
@@ -489,7 +483,7 @@ cudaError_t launch_collide_pair(const LbmArgs& a, int precision, int parity, boo
 // interior cells (a.rec must describe the particle state of this step)
 cudaError_t launch_mea_moments(const LbmArgs& a, int precision, int parity, bool walls, int nsm,
                                cudaStream_t s);
-cudaError_t launch_mea(const PartArgs& a, int precision, int parity, cudaStream_t s);
+cudaError_t launch_mea(const PartArgs& a, int precision, int parity, bool walls, cudaStream_t s);
 cudaError_t launch_update(const PartArgs& a, cudaStream_t s);
 // contact force and torque of every particle into PF_FC / PF_TC (only when
 // a.contact_k > 0)

@@ -1,6 +1,6 @@
-// mea_common.cuh -- device pieces of the bounding-box momentum exchange
-// shared by the kernels that compute Eq. hlbm:mea (Sec. 3.2) from the
-// populations alone.
+// mea_common.cuh -- device pieces of the momentum exchange of Eq. hlbm:mea
+// (Sec. 3.2) on a caller's populations in the plain structure of arrays, and
+// the rotation matrix the particle kernels share with it.
 #pragma once
 #include "hlbm_internal.cuh"
 
@@ -43,8 +43,7 @@ __device__ __forceinline__ void rotation_rn(const double q[4], double R[9]) {
 // omitted link, because the weights of all 18 links sum to zero.  In both AA
 // parities the pair of slots is {slot i of x, slot ibar of x - c_i}; only
 // which of the two is the arrival differs.  Slot i of the cell whose slot 0
-// is element e lies at f + i * P + e: P is the plane stride of a plain
-// structure of arrays, or VB in the blocked layout (nb from make_nbr_blocked).
+// is element e lies at f + i * P + e, P the plane stride.
 template <typename S, int PAR, typename NB>
 __device__ __forceinline__ void mea_cell(const S* f, long long P, const NB& nb, long long c,
                                          float inv_s, float F[3], float& mgain) {
@@ -92,11 +91,10 @@ __device__ __forceinline__ void row_range(int iy, int ext1, int lo0, int ext0, i
 // Per-thread sums (F, T) over the cells of plane iz of the bounding box
 // [floor(X - r_c), ceil(X + r_c)] of one particle whose centre is finite.
 // All threads of the block call it (it synchronises); s_start holds
-// MAX_PLANES + 1 ints, s_xa MAX_PLANES.  BLOCKED: f is the library's
-// blocked storage (plane unused); otherwise f holds the box alone as a plain
+// MAX_PLANES + 1 ints, s_xa MAX_PLANES.  f holds one box as a plain
 // structure of arrays with `plane` values per slot, cell (x, y, z) at
 // (z * ny + y) * nx + x.
-template <typename S, int PAR, bool BLOCKED>
+template <typename S, int PAR>
 __device__ __forceinline__ void mea_plane_sums(const Rec& R, const BoxDesc& bd, const double X[3],
                                                double rc, int iz, const S* f, long long plane,
                                                float inv_scale, int* s_start, int* s_xa,
@@ -159,13 +157,8 @@ __device__ __forceinline__ void mea_plane_sums(const Rec& R, const BoxDesc& bd, 
       float rr[3];
       if (!inside_fp32(R, bd, x, y, z, rr, gs)) continue;
       float Fc[3], mg;
-      if constexpr (BLOCKED) {
-        mea_cell<S, PAR>(f, (long long)VB, make_nbr_blocked(bd, x, y, z), elem_of(bd, x, y, z), inv_scale,
-                         Fc, mg);
-      } else {
-        mea_cell<S, PAR>(f, plane, make_nbr<true>(bd, x, y, z), (long long)((z * bd.ny + y) * bd.nx + x),
-                         inv_scale, Fc, mg);
-      }
+      mea_cell<S, PAR>(f, plane, make_nbr<true>(bd, x, y, z), (long long)((z * bd.ny + y) * bd.nx + x), inv_scale,
+                       Fc, mg);
       const float upx = R.u[0] + (R.w[1] * rr[2] - R.w[2] * rr[1]);
       const float upy = R.u[1] + (R.w[2] * rr[0] - R.w[0] * rr[2]);
       const float upz = R.u[2] + (R.w[0] * rr[1] - R.w[1] * rr[0]);

@@ -137,8 +137,8 @@ __global__ void noalloc_setup_kernel(NoAllocArgs a) {
 
 // the bounding-box momentum exchange, one block per (particle, plane); the
 // last block of a particle adds the planes' FP64 partials in plane order and
-// writes the caller's output; eight resident blocks per SM, as the
-// bounding-box momentum exchange of the library
+// writes the caller's output; eight resident blocks per SM (64 registers):
+// the walk is latency-bound, and more resident blocks beat the spills
 template <typename S, int PAR>
 __global__ void __launch_bounds__(128, 8) noalloc_mea_kernel(NoAllocArgs a) {
   const int p = blockIdx.x, iz = blockIdx.y;
@@ -155,8 +155,8 @@ __global__ void __launch_bounds__(128, 8) noalloc_mea_kernel(NoAllocArgs a) {
   double X[3];
   for (int j = 0; j < 3; ++j) X[j] = na_x(a)[3 * p + j];
   float v[6];
-  mea_plane_sums<S, PAR, false>(R, a.bd, X, na_rc(a)[p], iz, reinterpret_cast<const S*>(a.f), a.plane,
-                         a.inv_scale, s_start, s_xa, v);
+  mea_plane_sums<S, PAR>(R, a.bd, X, na_rc(a)[p], iz, reinterpret_cast<const S*>(a.f), a.plane, a.inv_scale,
+                         s_start, s_xa, v);
 #pragma unroll
   for (int k = 0; k < 6; ++k)
 #pragma unroll
