@@ -53,8 +53,8 @@ extern "C" {
 #define HLBM_ERR_CUDA (-2)     /* a CUDA call failed */
 #define HLBM_ERR_UNSTABLE (-3) /* a non-finite or non-positive density or particle state */
 #define HLBM_ERR_CAPACITY (-4) /* a fixed-size work list overflowed: a tile's particle list
-                                  (bin_capacity), three particles overlapping at one cell, or
-                                  the list of interior cells; hlbm_last_error says which */
+                                  (bin_capacity) or three particles overlapping at one cell;
+                                  hlbm_last_error says which */
 #define HLBM_ERR_STATE (-5)    /* call not allowed in the current state */
 
 /* storage of the populations: the deviation f_i - w_i from the weights */
@@ -171,10 +171,10 @@ int hlbm_add_particles(hlbm_handle h, int n, const int* box_id, const int* shape
  * checked and staged on the host, the upload is queued on the stream and the
  * call returns without waiting for it: the arrays may be reused at once.
  * A new position or orientation changes the cells inside the particles, so
- * the next step takes the bounding-box momentum exchange; positions (and the
+ * the next step takes the link sums of the momentum exchange; positions (and the
  * orientations of non-spheres) that are not given, or that equal bit for bit
  * the state hlbm_particle_state returned after the current step, keep the
- * momentum exchange from the recorded moments.  HLBM_ERR_ARG (nothing
+ * moments form of the momentum exchange.  HLBM_ERR_ARG (nothing
  * changed) for a non-finite position or a zero or non-finite quaternion. */
 int hlbm_set_particle_state(hlbm_handle h, const double* X, const double* U, const double* omega,
                             const double* quat);
@@ -251,19 +251,15 @@ int hlbm_set_launch(hlbm_handle h, int tile_y, int tile_z, int cells_x);
 int hlbm_get_launch(hlbm_handle h, int* tile_y, int* tile_z, int* cells_x);
 
 /* How the momentum exchange (Eq. hlbm:mea) of a step is computed:
- *   HLBM_MEA_KERNEL   from the populations alone, by a kernel that walks the
- *                     bounding box of each particle (default);
- *   HLBM_MEA_MOMENTS  the collision of the previous step lists the cells
- *                     inside particles with the mass and momentum their
- *                     post-collision populations carry away; the momentum
- *                     exchange is then, per listed cell, the momentum gained
- *                     minus u_p times the mass gained, from the arrivals alone.
- *                     The bounding-box kernel still runs on the first step
- *                     after any change of state.  Needs max_particles > 0; the
- *                     list is split into 64 stripes that the collision's
- *                     blocks fill in turn, each holding 1/64 of half the
- *                     lattice's cells (at least 4096 entries);
- *                     HLBM_ERR_CAPACITY when one overflows.
+ *   HLBM_MEA_KERNEL   as the sum of Eq. hlbm:mea over the links of the cells
+ *                     inside a particle, added in a fixed order (default);
+ *   HLBM_MEA_MOMENTS  per interior cell, the momentum the cell gained by the last
+ *                     streaming minus u_p times the mass it gained, from the
+ *                     moments of what arrived and of what the collision sent
+ *                     out, added in fixed point (no order).  The link sums still
+ *                     run on the first step after any change of state.  Needs
+ *                     max_particles > 0.
+ * Both walk the cells of each particle and read the populations alone.
  * Both give the same force and torque up to FP32 summation order. */
 #define HLBM_MEA_KERNEL 0
 #define HLBM_MEA_MOMENTS 1
@@ -292,10 +288,10 @@ int hlbm_kernel_times(hlbm_handle h, int nsteps, float ms[3]);
 /* Writes to *n the number of (cell, particle) pairs whose cell centre lies
  * inside the particle (Sec. 3.2, the cells the sums of Eqs.
  * hydrodynamicforce and hydrodynamictorque run over) at the current
- * particle state: the entries the last collision listed in the moments
- * mode, i.e. the work of the next step's momentum exchange.  A cell inside
- * two particles counts twice.  Synchronises.  HLBM_ERR_STATE outside the
- * moments mode or before the first step after a change of state. */
+ * particle state, i.e. the work of the next step's momentum exchange.  A
+ * cell inside two particles counts twice.  Synchronises.  HLBM_ERR_STATE
+ * outside the moments mode or before the first step after a change of
+ * state. */
 int hlbm_interior_cells(hlbm_handle h, long long* n);
 
 /* Snapshots (checkpoint and restart; not part of the paper's method).
@@ -304,10 +300,9 @@ int hlbm_interior_cells(hlbm_handle h, long long* n);
  * distance grids, the populations as
  * stored (the handle's block layout and precision, bit for bit), the FP64
  * particle table with shapes and box ids, the step count (hence the AA
- * parity), the fluid force, the momentum-exchange mode and, when the next
- * step takes its momentum exchange from the recorded moments, the list of
- * interior cells the last collision wrote.  Launch shape and tuning are not
- * part of it.  The layout is host byte order with fixed-width fields; it is
+ * parity), the fluid force, the momentum-exchange mode and whether the next
+ * step takes the moments form.  Launch shape and tuning are not part of it.
+ * Snapshots of the version that kept a list of interior cells load as well.  The layout is host byte order with fixed-width fields; it is
  * meant for the same library on machines of the same byte order.
  *
  * hlbm_checkpoint_bytes: *bytes = the size of a snapshot of the current

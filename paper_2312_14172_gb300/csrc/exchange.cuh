@@ -218,4 +218,249 @@ __device__ __forceinline__ void exchange_share(const PartArgs& a, const Rec& R, 
   }
 }
 
+// ------------------------------------------------- the moments form
+// Per interior cell x the used-sign sum is the momentum the cell gained by
+// the last streaming, minus u_p times the mass it gained:
+//   F(x) = (j - j*) - u_p(x) (rho - rho*)  [links into a wall: - 2 c_i f_i(x)]
+// j, rho the moments of the arrivals f_i(x), j*, rho* those of the cell's own
+// post-collision values f*_i(x), which the populations still hold (as the
+// departures).  Each cell's terms are rounded to fixed point (ACC_FRAC_BITS)
+// and added as integers: the sums depend on no order, so the cells may be
+// spread over threads, warps and blocks in any way.
+
+// FP32 radius about the centre that holds the particle (rounded up; grid
+// particles carry theirs in a[0])
+__device__ __forceinline__ float exchange_reach(const Rec& R) {
+  float rc;
+  if (R.shape == 0 || R.shape == 4) rc = R.a[0];
+  else if (R.shape == 1) rc = fmaxf(R.a[0], fmaxf(R.a[1], R.a[2]));
+  else if (R.shape == 3) rc = R.a[0] + R.a[2];
+  else rc = sqrtf(R.a[0] * R.a[0] + R.a[1] * R.a[1] + R.a[2] * R.a[2]);
+  return rc * 1.00001f + 0.01f;
+}
+
+// cells [lo, lo + ext) of one axis whose centre can lie within rc of the
+// particle's centre, unwrapped; clipped at walls
+__device__ __forceinline__ void exchange_extent(float xh, float rc, bool wall, int w_lo, int w_hi, int& lo, int& ext) {
+  const float m = rc + fabsf(xh) * 2.4e-7f;  // the centre's rounding in FP32
+  int l = (int)ceilf(xh - m), h = (int)floorf(xh + m);
+  if (wall) {
+    l = max(l, w_lo);
+    h = min(h, w_hi);
+  }
+  lo = l;
+  ext = min(max(h - l + 1, 0), MAX_PLANES);
+}
+
+// Offsets [t0, t1] along x from the centre that can lie inside the particle,
+// on the x-parallel line at offset (ry, rz): the chord of the circumscribed
+// sphere, for elongated shapes cut to their enclosing capsule (to the
+// infinite cylinder about its axis and to its ends).  False: none.
+__device__ __forceinline__ bool exchange_chord(const Rec& R, const Capsule& cap, float rc, float ry, float rz,
+                                               float& t0, float& t1) {
+  const float d2 = ry * ry + rz * rz;
+  const float h2 = rc * rc - d2;
+  if (!(h2 >= 0.0f)) return false;
+  const float s = sqrtf(h2);
+  t0 = -s;
+  t1 = s;
+  if (R.shape == 0) return true;
+  if (capsule_row_dist2(cap, ry, rz) >= cap.r2) return false;
+  const float w = ry * cap.u[1] + rz * cap.u[2];
+  const float A = 1.0f - cap.u[0] * cap.u[0];
+  if (A > 1e-2f) {
+    // |(x, ry, rz)|^2 - ((x, ry, rz) . u)^2 < r^2
+    const float b = cap.u[0] * w;
+    const float disc = b * b - A * (d2 - w * w - cap.r2);
+    if (!(disc >= 0.0f)) return false;
+    const float q = sqrtf(disc);
+    t0 = fmaxf(t0, (b - q) / A);
+    t1 = fminf(t1, (b + q) / A);
+  }
+  if (fabsf(cap.u[0]) > 1e-2f) {
+    const float e = cap.h + sqrtf(cap.r2), iu = 1.0f / fabsf(cap.u[0]);
+    const float c = cap.u[0] > 0.0f ? -w : w;
+    t0 = fmaxf(t0, (c - e) * iu);
+    t1 = fminf(t1, (c + e) * iu);
+  }
+  return t1 >= t0;
+}
+
+// Rows of the bounding box that can hold interior cells, flattened: row r
+// covers the cells [start[r], start[r + 1]) of the flat index; xa is the
+// unwrapped x of its first cell, y and z are wrapped.
+struct ExchangeRows {
+  int start[XCH_MAX_T];
+  int xa[XCH_MAX_T], y[XCH_MAX_T], z[XCH_MAX_T];
+  int wtot[XCH_MAX_T / 32];
+};
+
+// Calls cell(x, y, z, rr) for every interior cell of planes [q0, q0 + nq) of
+// the particle's bounding box (rr its offset from the centre), spread over
+// the block's threads (blockDim.x a power of two; all of them call, it
+// synchronises).  One thread finds the x-range of one row; the rows' cells
+// are then flattened, so that lanes stay busy whatever the shape.
+template <bool GRIDS, typename Cell>
+__device__ __forceinline__ void for_interior(const Rec& R, const BoxDesc& bd, int q0, int nq, GridSet grids,
+                                             ExchangeRows& sh, Cell cell) {
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+  const GridSet gs = GRIDS ? grids : GridSet{};
+  const float rc = exchange_reach(R);
+  const bool cutz = bd.bc & BC_CUT_Z;  // a slab: owned planes only
+  int lox, extx, loy, exty, loz, extz;
+  exchange_extent(R.xh[0], rc, bd.bc & 1, 0, bd.nx - 1, lox, extx);
+  exchange_extent(R.xh[1], rc, bd.bc & 2, 0, bd.ny - 1, loy, exty);
+  exchange_extent(R.xh[2], rc, bd.bc & 4, cutz ? bd.own_lo : 0, cutz ? bd.own_hi - 1 : bd.nz - 1, loz, extz);
+  const int planes = min(nq, extz - q0);
+  const int rows = planes > 0 ? planes * exty : 0;
+  const Capsule cap = capsule_of(R, 0.0f);
+  for (int row0 = 0; row0 < rows; row0 += nt) {
+    const int row = row0 + tid;
+    int len = 0, xa = 0, y = 0, z = 0;
+    if (row < rows) {
+      const int iz = row / exty;
+      y = loy + (row - iz * exty);
+      z = loz + q0 + iz;
+      const float ry = ((float)y - R.xh[1]) - R.xl[1], rz = ((float)z - R.xh[2]) - R.xl[2];
+      float t0, t1;
+      if (exchange_chord(R, cap, rc, ry, rz, t0, t1)) {
+        const float m = 0.02f + fabsf(R.xh[0]) * 2.4e-7f;
+        xa = max((int)ceilf(R.xh[0] + t0 - m), lox);
+        const int xb = min((int)floorf(R.xh[0] + t1 + m), lox + extx - 1);
+        len = max(xb - xa + 1, 0);
+      }
+      y = y < 0 ? y + bd.ny : (y >= bd.ny ? y - bd.ny : y);
+      z = z < 0 ? z + bd.nz : (z >= bd.nz ? z - bd.nz : z);
+      if ((unsigned)y >= (unsigned)bd.ny || (unsigned)z >= (unsigned)bd.nz) len = 0;
+    }
+    int sum = len;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, sum, off);
+      if (lane >= off) sum += t;
+    }
+    if (lane == 31) sh.wtot[warp] = sum;
+    __syncthreads();
+    int before = 0, total = 0;
+    for (int w = 0; w < (nt >> 5); ++w) {
+      const int t = sh.wtot[w];
+      if (w < warp) before += t;
+      total += t;
+    }
+    sh.start[tid] = before + sum - len;
+    sh.xa[tid] = xa;
+    sh.y[tid] = y;
+    sh.z[tid] = z;
+    __syncthreads();
+    for (int q = tid; q < total; q += nt) {
+      int r = 0;  // the row holding flat index q: the last one starting at or before it
+      for (int step = nt >> 1; step > 0; step >>= 1)
+        if (sh.start[r + step] <= q) r += step;
+      const int xu = sh.xa[r] + (q - sh.start[r]);
+      const int x = xu < 0 ? xu + bd.nx : (xu >= bd.nx ? xu - bd.nx : xu);
+      float rr[3];
+      if ((unsigned)x < (unsigned)bd.nx && inside_fp32(R, bd, x, sh.y[r], sh.z[r], rr, gs)) cell(x, sh.y[r], sh.z[r], rr);
+    }
+    __syncthreads();  // the rows are rewritten by the next chunk
+  }
+}
+
+// force and torque terms of one interior cell; PAIRS: the departures summed
+// by opposite pairs, as the two-cell collision does, otherwise one by one, as
+// the one-cell collision (the sums agree to rounding)
+template <typename S, int PAR, bool W>
+__device__ __forceinline__ void exchange_moments(const S* f, const Rec& R, const BoxDesc& bd, int x, int y, int z,
+                                                 const float (&r)[3], float inv_s, bool pairs, float (&F)[3],
+                                                 float (&T)[3]) {
+  const RowBlocks rb = row_blocks<W>(bd, x, y, 1);
+  int zb[3];
+  slice_blocks<W>(bd, z, zb);
+  const S* own = cell_ptr(f, zb[1] + rb.yb[1] + rb.xb, rb.xin);
+  float va[Q], vb[Q];  // slot i of x; slot ibar of x - c_i (slot i of x when that lies beyond a wall)
+  unsigned walls = 0;  // bit i: x - c_i lies beyond a wall
+  va[0] = vb[0] = Pop<S>::ld_raw(own);
+#pragma unroll
+  for (int i = 1; i < Q; ++i) {
+    const int by = rb.yb[1 - cy(i)], bz = zb[1 - cz(i)];
+    const bool wall = W && (by < 0 || bz < 0 || (cx(i) > 0 && rb.wl) || (cx(i) < 0 && rb.wr));
+    const int dx = cx(i) > 0 ? rb.dl : (cx(i) < 0 ? rb.dr : 0);
+    const S* nb = wall ? own + i * VB : cell_ptr(f, bz + by + rb.xb, rb.xin) + (dx + opp(i) * VB);
+    if (wall) walls |= 1u << i;
+    va[i] = Pop<S>::ld_raw(own + i * VB);
+    vb[i] = Pop<S>::ld_raw(nb);
+  }
+  // arrivals f_i(x) are slot i of x (even parity) or slot ibar of x - c_i
+  // (odd parity); the departure f*_i(x) is the other kind for ibar.  Sums in
+  // stored units (the scale is a power of two).
+  float ms = 0.f, px = 0.f, py = 0.f, pz = 0.f;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const float d = PAR == 0 ? va[i] : vb[i];
+    ms += d;
+    if (cx(i)) px += (float)cx(i) * d;
+    if (cy(i)) py += (float)cy(i) * d;
+    if (cz(i)) pz += (float)cz(i) * d;
+  }
+  float m0, jx, jy, jz;
+  auto dep = [&](int i) { return PAR == 0 ? vb[opp(i)] : va[opp(i)]; };
+  if (pairs) {
+    float m[Q];
+    m0 = dep(0);
+#pragma unroll
+    for (int i = 1; i < Q; i += 2) {
+      m0 = m0 + (dep(i) + dep(i + 1));
+      m[i] = dep(i) - dep(i + 1);
+    }
+    jx = ((m[1] + m[7]) + (m[9] + m[11])) + m[13];
+    jy = (((m[3] + m[7]) - m[9]) + m[15]) + m[17];
+    jz = (((m[5] + m[11]) - m[13]) + m[15]) - m[17];
+  } else {
+    m0 = jx = jy = jz = 0.f;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      m0 += dep(i);
+      if (cx(i)) jx += (float)cx(i) * dep(i);
+      if (cy(i)) jy += (float)cy(i) * dep(i);
+      if (cz(i)) jz += (float)cz(i) * dep(i);
+    }
+  }
+  const float dm = Pop<S>::SCALED ? __fmul_rn(ms - m0, inv_s) : ms - m0;
+  const float dx = Pop<S>::SCALED ? __fmul_rn(px - jx, inv_s) : px - jx;
+  const float dy = Pop<S>::SCALED ? __fmul_rn(py - jy, inv_s) : py - jy;
+  const float dz = Pop<S>::SCALED ? __fmul_rn(pz - jz, inv_s) : pz - jz;
+  const float upx = R.u[0] + (R.w[1] * r[2] - R.w[2] * r[1]);
+  const float upy = R.u[1] + (R.w[2] * r[0] - R.w[0] * r[2]);
+  const float upz = R.u[2] + (R.w[0] * r[1] - R.w[1] * r[0]);
+  F[0] = dx - upx * dm;
+  F[1] = dy - upy * dm;
+  F[2] = dz - upz * dm;
+  if (W) {
+#pragma unroll
+    for (int i = 1; i < Q; ++i)
+      if ((walls >> i) & 1u) {
+        const float d = PAR == 0 ? va[i] : vb[i];
+        const float v = 2.0f * ((float)wq(i) + (Pop<S>::SCALED ? __fmul_rn(d, inv_s) : d));
+        if (cx(i)) F[0] -= (float)cx(i) * v;
+        if (cy(i)) F[1] -= (float)cy(i) * v;
+        if (cz(i)) F[2] -= (float)cz(i) * v;
+      }
+  }
+  T[0] = r[1] * F[2] - r[2] * F[1];
+  T[1] = r[2] * F[0] - r[0] * F[2];
+  T[2] = r[0] * F[1] - r[1] * F[0];
+}
+
+// Exact warp sum of 64-bit values, from three limbs with single-instruction
+// warp reductions: v = a 2^42 + b 2^21 + c with c, b in [0, 2^21) and
+// a = v >> 42 in [-2^21, 2^21), so 32 lanes' limb sums stay within 32 bits.
+__device__ __forceinline__ long long warp_sum_i64(long long v) {
+  const unsigned c = (unsigned)v & 0x1fffffu;
+  const unsigned b = (unsigned)(v >> 21) & 0x1fffffu;
+  const int hi = (int)(v >> 42);
+  const unsigned sc = __reduce_add_sync(0xffffffffu, c);
+  const unsigned sb = __reduce_add_sync(0xffffffffu, b);
+  const int sa = __reduce_add_sync(0xffffffffu, hi);
+  return (long long)(((unsigned long long)(long long)sa << 42) + ((unsigned long long)sb << 21) + sc);
+}
+
 }  // namespace hlbm

@@ -38,11 +38,9 @@ size_t align_up(size_t v) { return (v + ALIGN - 1) / ALIGN * ALIGN; }
 struct Layout {
   long long nblocks = 0, ncell = 0, ntiles = 0, stage_cells = 0;
   int cap = 0, bin_cap = 0;
-  size_t off_f, off_boxes, off_P, off_shape, off_box, off_rec, off_part, off_acc, off_chp, off_chq,
-      off_pc0, off_pnc, off_ppl, off_done, off_lcnt, off_lidx, off_lmom, off_cnt[2], off_ids[2], off_status,
-      off_stage, off_gdesc, off_gvals, total;
+  size_t off_f, off_boxes, off_P, off_shape, off_box, off_rec, off_part, off_acc, off_chunk[2], off_done,
+      off_count, off_cnt[2], off_ids[2], off_status, off_stage, off_gdesc, off_gvals, total;
   long long grid_floats = 0;
-  long long ilist_cap = 0;
 };
 
 bool make_layout(int nb, const hlbm_box* boxes, const hlbm_params* prm, Layout& L,
@@ -71,14 +69,11 @@ bool make_layout(int nb, const hlbm_box* boxes, const hlbm_params* prm, Layout& 
     if (cells + n >= (1LL << 31)) { err = "all boxes together may hold at most 2^31 - 1 cells"; return false; }
     BoxDesc& d = bd[b];
     d.nx = B.nx; d.ny = B.ny; d.nz = B.nz; d.bc = B.bc_flags;
-    d.div_x = make_fastdiv((unsigned)B.nx);
-    d.div_y = make_fastdiv((unsigned)B.ny);
     d.own_lo = 0;
     d.own_hi = B.nz;
     d.ntx = (B.nx + TILE_X - 1) / TILE_X;
     d.nty = (B.ny + TILE_Y - 1) / TILE_Y;
     d.ntz = (B.nz + TILE_Z - 1) / TILE_Z;
-    d.cell_off = cells;
     d.tile_off = tiles;
     d.blk_off = blocks;
     cells += n;
@@ -102,21 +97,9 @@ bool make_layout(int nb, const hlbm_box* boxes, const hlbm_params* prm, Layout& 
   L.off_rec = o; o = align_up(o + sizeof(Rec) * (size_t)L.cap);
   L.off_part = o; o = align_up(o + sizeof(double) * 6 * MAX_PLANES * (size_t)L.cap);
   L.off_acc = o; o = align_up(o + sizeof(double) * 6 * (size_t)L.cap);
-  L.off_chp = o; o = align_up(o + sizeof(int) * MAX_PLANES * (size_t)L.cap);
-  L.off_chq = o; o = align_up(o + sizeof(int) * MAX_PLANES * (size_t)L.cap);
-  L.off_pc0 = o; o = align_up(o + sizeof(int) * (size_t)L.cap);
-  L.off_pnc = o; o = align_up(o + sizeof(int) * (size_t)L.cap);
-  L.off_ppl = o; o = align_up(o + sizeof(int) * (size_t)L.cap);
+  for (int k = 0; k < 2; ++k) { L.off_chunk[k] = o; o = align_up(o + sizeof(int4) * MAX_PLANES * (size_t)L.cap); }
   L.off_done = o; o = align_up(o + sizeof(int) * (size_t)L.cap);
-  // interior-cell list for the momentum exchange from moments, in
-  // ILIST_STRIPES stripes: together room for half of all cells (more than
-  // any packing of non-overlapping particles needs), and each stripe for two
-  // entries per cell of a whole brick
-  L.ilist_cap = L.cap > 0 ? std::max((L.ncell / 2 + ILIST_STRIPES - 1) / ILIST_STRIPES,
-                                     (long long)2 * TILE_X * TILE_Y * TILE_Z) : 0;
-  L.off_lcnt = o; o = align_up(o + sizeof(int) * ILIST_STRIPES);
-  L.off_lidx = o; o = align_up(o + sizeof(int2) * (size_t)L.ilist_cap * ILIST_STRIPES);
-  L.off_lmom = o; o = align_up(o + sizeof(float4) * (size_t)L.ilist_cap * ILIST_STRIPES);
+  L.off_count = o; o = align_up(o + sizeof(unsigned long long));
   for (int k = 0; k < 2; ++k) {
     L.off_cnt[k] = o; o = align_up(o + sizeof(int) * (size_t)L.ntiles);
     L.off_ids[k] = o; o = align_up(o + sizeof(int) * (size_t)L.ntiles * L.bin_cap);
@@ -150,24 +133,20 @@ struct hlbm_ctx {
   Rec* rec = nullptr;
   double* partial = nullptr;
   long long* acc = nullptr;
-  int* chunk_p = nullptr;
-  int* chunk_q = nullptr;
-  int* p_chunk0 = nullptr;
-  int* p_nchunk = nullptr;
-  int* p_planes = nullptr;
+  // momentum-exchange blocks, [0] of the link sums, [1] of the moments form
+  int4* chunks[2] = {nullptr, nullptr};
+  int nchunks[2] = {0, 0};
+  int mea_threads[2] = {128, 128};
+  unsigned long long* count = nullptr;
   int* done = nullptr;
-  int* ilist_count = nullptr;
-  int2* ilist_idx = nullptr;
-  float4* ilist_mom = nullptr;
   int nsm = 0;
   // odd steps take the bricks in reverse order when the populations are
   // within twice the L2 (a step then starts on what the last one ended
   // with, still in L2); larger lattices gain nothing and keep one order
   bool reverse_odd = false;
-  int nchunks = 0;
   std::vector<int> h_planes;    // bounding-box planes per particle
   int mea_group = 1;            // planes whose cells are summed together
-  int mea_threads = 128;        // threads per momentum-exchange block
+  std::vector<double> h_cells;  // about the cells inside each particle
   int mea_mode = HLBM_MEA_KERNEL;
   int* cnt[2] = {nullptr, nullptr};
   int* ids[2] = {nullptr, nullptr};
@@ -195,7 +174,9 @@ struct hlbm_ctx {
   // GRAPH_STEPS steps in one graph, the same way (when more than two)
   cudaGraphExec_t execk[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
   bool graphs_ok = false;
-  bool moments_valid = false;  // the accumulator holds this state's momentum exchange
+  // the last collision knew this particle state, so in the moments mode the
+  // momentum exchange takes the moments form
+  bool moments_valid = false;
   int split = 0;  // a split step is open: 1 after its bounding-box exchange, 2 after its moments one
   // hstage holds the device's particle rows X .. T as downloaded by
   // hlbm_particle_state after step hst_steps (until an upload reuses it)
@@ -237,7 +218,6 @@ static LbmArgs lbm_args(const hlbm_ctx* h, int parity) {
   LbmArgs a{};
   a.nsm = h->nsm;
   a.f = h->f;
-  a.ncell = h->L.ncell;
   a.boxes = h->d_boxes;
   a.nboxes = (int)h->boxes.size();
   a.sub_y = h->sub_y;
@@ -257,19 +237,12 @@ static LbmArgs lbm_args(const hlbm_ctx* h, int parity) {
   a.bin_ids = h->ids[parity];
   a.bin_cap = h->L.bin_cap;
   a.rec = h->rec;
-  const bool rec = h->mea_mode == HLBM_MEA_MOMENTS && h->ilist_idx;
-  a.ilist_count = h->ilist_count;
-  a.ilist_idx = rec ? h->ilist_idx : nullptr;
-  a.ilist_mom = rec ? h->ilist_mom : nullptr;
-  a.ilist_cap = h->L.ilist_cap;
-  a.np = h->np;
-  a.acc = h->acc;
   a.grids = h->grids.empty() ? GridSet{} : GridSet{h->d_gdesc, h->d_gvals};
   a.status = h->status;
   return a;
 }
 
-static PartArgs part_args(const hlbm_ctx* h, int parity) {
+static PartArgs part_args(const hlbm_ctx* h, int parity, bool moments = false) {
   PartArgs a{};
   a.P = h->P;
   a.cap = h->L.cap;
@@ -284,23 +257,18 @@ static PartArgs part_args(const hlbm_ctx* h, int parity) {
   const double sc = h->prm.precision == HLBM_FP16 ? std::ldexp(1.0, h->prm.fp16_scale_log2) : 1.0;
   a.scale = (float)sc;
   a.inv_scale = (float)(1.0 / sc);
-  a.chunk_p = h->chunk_p;
-  a.chunk_q = h->chunk_q;
-  a.p_chunk0 = h->p_chunk0;
-  a.p_nchunk = h->p_nchunk;
-  a.nchunks = h->nchunks;
-  a.p_planes = h->p_planes;
+  a.chunks = h->chunks[moments];
+  a.nchunks = h->nchunks[moments];
+  a.mea_threads = h->mea_threads[moments];
   a.mea_group = h->mea_group;
-  a.mea_threads = h->mea_threads;
+  a.cells_x = h->cells_x;
   a.partial = h->partial;
   a.done = h->done;
   a.acc = h->acc;
-  a.from_acc = 0;
   a.contact_k = h->contact_k;
   a.contact_zeta = h->contact_zeta;
   a.grids = h->grids.empty() ? GridSet{} : GridSet{h->d_gdesc, h->d_gvals};
   a.nsm = h->nsm;
-  a.ilist_count = h->ilist_count;
   a.bin_count = h->cnt[parity];
   a.bin_ids = h->ids[parity];
   a.bin_count_clear = h->cnt[1 - parity];
@@ -310,10 +278,9 @@ static PartArgs part_args(const hlbm_ctx* h, int parity) {
   return a;
 }
 
-// moments: the collision of the previous step recorded the post-collision
-// moments of the cells inside particles, and the momentum exchange of this
-// step runs from them; otherwise the bounding-box kernel computes it from
-// the populations alone (always on the first step after a change of state).
+// moments: the momentum exchange of this step takes the moments form (the
+// collision of the previous step knew the particle state); otherwise the link
+// sums (always on the first step after a change of state).
 // Kernels captured into a step's graph use programmatic dependent launch.
 // steps per captured graph for long runs (two-step and one-step graphs
 // take the rest)
@@ -327,14 +294,9 @@ static cudaError_t enqueue_step(hlbm_ctx* h, int parity, bool moments, cudaStrea
   LbmArgs la = lbm_args(h, parity);
   la.pdl = 1;
   if (h->np > 0) {
-    PartArgs pa = part_args(h, parity);
+    PartArgs pa = part_args(h, parity, moments);
     pa.pdl = 1;
-    pa.from_acc = moments ? 1 : 0;
-    if (moments) {
-      if ((e = launch_mea_moments(la, h->prm.precision, parity, h->walls, h->nsm, s)) != cudaSuccess) return e;
-    } else if ((e = launch_mea(pa, h->prm.precision, parity, h->walls, s)) != cudaSuccess) {
-      return e;
-    }
+    if ((e = launch_mea(pa, h->prm.precision, parity, h->walls, moments, s)) != cudaSuccess) return e;
     if ((e = launch_contact(pa, s)) != cudaSuccess) return e;
     if ((e = launch_update(pa, s)) != cudaSuccess) return e;
   }
@@ -391,11 +353,7 @@ static int status_code(hlbm_ctx* h, int st) {
   if (st & ST_CAPACITY)
     return fail(h, HLBM_ERR_CAPACITY, "a 32x8x8 tile was touched by more particles than bin_capacity");
   if (st & ST_OVERLAP)
-    return fail(h, HLBM_ERR_CAPACITY, "three particles overlap at one cell (the list of interior cells takes two)");
-  if (st & ST_LIST_FULL)
-    return fail(h, HLBM_ERR_CAPACITY, "the list of interior cells is full");
-  if (st & ST_INTERNAL)
-    return fail(h, HLBM_ERR_STATE, "the list of cells inside particles held an invalid entry");
+    return fail(h, HLBM_ERR_CAPACITY, "three particles overlap at one cell (two at most may)");
   if (st & ST_LEFT_DOMAIN)
     return fail(h, HLBM_ERR_UNSTABLE, "a particle centre left the fluid domain through a wall");
   return fail(h, HLBM_ERR_UNSTABLE, "non-finite or non-positive density, or non-finite particle state");
@@ -485,15 +443,9 @@ int hlbm_init_batch(hlbm_handle* out, int nboxes, const hlbm_box* boxes, const h
   h->rec = (Rec*)(h->buf + h->L.off_rec);
   h->partial = (double*)(h->buf + h->L.off_part);
   h->acc = (long long*)(h->buf + h->L.off_acc);
-  h->chunk_p = (int*)(h->buf + h->L.off_chp);
-  h->chunk_q = (int*)(h->buf + h->L.off_chq);
-  h->p_chunk0 = (int*)(h->buf + h->L.off_pc0);
-  h->p_nchunk = (int*)(h->buf + h->L.off_pnc);
-  h->p_planes = (int*)(h->buf + h->L.off_ppl);
+  for (int k = 0; k < 2; ++k) h->chunks[k] = (int4*)(h->buf + h->L.off_chunk[k]);
   h->done = (int*)(h->buf + h->L.off_done);
-  h->ilist_count = (int*)(h->buf + h->L.off_lcnt);
-  h->ilist_idx = h->L.ilist_cap > 0 ? (int2*)(h->buf + h->L.off_lidx) : nullptr;
-  h->ilist_mom = h->L.ilist_cap > 0 ? (float4*)(h->buf + h->L.off_lmom) : nullptr;
+  h->count = (unsigned long long*)(h->buf + h->L.off_count);
   {
     int dev = 0;
     cudaGetDevice(&dev);
@@ -812,6 +764,8 @@ int hlbm_add_grid(hlbm_handle h, int nx, int ny, int nz, double spacing, const f
 // block waits for another's sum (us, 256 threads and 6 planes against 128
 // and 24: 200 spheres FP32 35 / 57, 2000 ellipsoids and cuboids 249 / 170,
 // 50 000 spheres FP16 2869 / 1470).
+// In the moments form neither is: there a block takes about as many cells
+// as its threads walk in six (few particles) or twenty (many) rounds.
 static int plan_exchange(hlbm_ctx* h) {
   const int nsm = h->nsm > 0 ? h->nsm : 152;
   long long planes = 0;
@@ -819,28 +773,23 @@ static int plan_exchange(hlbm_ctx* h) {
   const int G = (int)std::min(3LL, std::max(1LL, planes / (4LL * nsm * 8)));
   h->mea_group = G;
   const bool few = h->np < 4 * nsm;
-  h->mea_threads = few ? 256 : 128;
-  const int per = few ? 6 : 24;
-  std::vector<int> cp, cq, c0(h->np), cn(h->np), pl(h->np);
-  for (int p = 0; p < h->np; ++p) {
-    // whole groups per block, about `per` planes
-    const int groups = (h->h_planes[p] + G - 1) / G;
-    const int parts = std::max(1, (h->h_planes[p] + per - 1) / per);
-    const int gp = (groups + parts - 1) / parts;
-    pl[p] = gp * G;
-    cn[p] = (groups + gp - 1) / gp;
-    c0[p] = (int)cp.size();
-    for (int k = 0; k < cn[p]; ++k) {
-      cp.push_back(p);
-      cq.push_back(k * pl[p]);
+  std::vector<int4> ck[2];
+  for (int form = 0; form < 2; ++form) {
+    const int t = few ? 256 : 128;
+    h->mea_threads[form] = t;
+    for (int p = 0; p < h->np; ++p) {
+      // whole groups of planes per block
+      const int g = form ? 1 : G, groups = (h->h_planes[p] + g - 1) / g;
+      int want = form ? (int)std::ceil(h->h_cells[p] / ((few ? 6.0 : 20.0) * t))
+                      : (h->h_planes[p] + (few ? 5 : 23)) / (few ? 6 : 24);
+      want = std::max(1, std::max(want, nsm / h->np));  // at least a block per SM
+      const int per = (groups + want - 1) / want, parts = (groups + per - 1) / per;
+      for (int k = 0; k < parts; ++k) ck[form].push_back(make_int4(p, k * per * g, per * g, parts));
     }
+    h->nchunks[form] = (int)ck[form].size();
+    CK(cudaMemcpyAsync(h->chunks[form], ck[form].data(), sizeof(int4) * ck[form].size(), cudaMemcpyHostToDevice,
+                       h->stream));
   }
-  h->nchunks = (int)cp.size();
-  CK(cudaMemcpyAsync(h->chunk_p, cp.data(), sizeof(int) * cp.size(), cudaMemcpyHostToDevice, h->stream));
-  CK(cudaMemcpyAsync(h->chunk_q, cq.data(), sizeof(int) * cq.size(), cudaMemcpyHostToDevice, h->stream));
-  CK(cudaMemcpyAsync(h->p_chunk0, c0.data(), sizeof(int) * c0.size(), cudaMemcpyHostToDevice, h->stream));
-  CK(cudaMemcpyAsync(h->p_nchunk, cn.data(), sizeof(int) * cn.size(), cudaMemcpyHostToDevice, h->stream));
-  CK(cudaMemcpyAsync(h->p_planes, pl.data(), sizeof(int) * pl.size(), cudaMemcpyHostToDevice, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   return HLBM_OK;
 }
@@ -856,6 +805,7 @@ int hlbm_add_particles(hlbm_handle h, int n, const int* box_id, const int* shape
   if (n == 0) return HLBM_OK;
   std::vector<double> tab((size_t)PF_COUNT * n, 0.0);
   std::vector<int> sh(n), bx(n), nch(n);
+  std::vector<double> cells(n);
   auto T = [&](int fld, int k) -> double& { return tab[(size_t)fld * n + k]; };
   for (int k = 0; k < n; ++k) {
     const int b = box_id ? box_id[k] : 0;
@@ -939,6 +889,7 @@ int hlbm_add_particles(hlbm_handle h, int n, const int* box_id, const int* shape
     sh[k] = s;
     bx[k] = b;
     nch[k] = (int)std::ceil(2.0 * rc) + 2;  // bounding-box planes, at most MAX_PLANES
+    cells[k] = 4.0 / 3.0 * PI_D * std::pow(std::cbrt(V * 3.0 / (4.0 * PI_D)) + 0.5, 3.0);
   }
   const int p0 = h->np;
   int rc = upload_fields(h, p0, n, tab);
@@ -950,6 +901,7 @@ int hlbm_add_particles(hlbm_handle h, int n, const int* box_id, const int* shape
   h->h_shape.insert(h->h_shape.end(), sh.begin(), sh.end());
   h->h_box.insert(h->h_box.end(), bx.begin(), bx.end());
   h->h_planes.insert(h->h_planes.end(), nch.begin(), nch.end());
+  h->h_cells.insert(h->h_cells.end(), cells.begin(), cells.end());
   rc = plan_exchange(h);
   if (rc != HLBM_OK) return rc;
   CK(launch_records(part_args(h, 0), h->stream));
@@ -1101,22 +1053,8 @@ int hlbm_step_forces(hlbm_handle h, double* F, double* T) {
     return HLBM_OK;
   }
   const bool moments = h->moments_valid;
-  if (moments) {
-    LbmArgs la = lbm_args(h, parity);
-    CK(launch_mea_moments(la, h->prm.precision, parity, h->walls, h->nsm, h->stream));
-    std::vector<long long> acc((size_t)6 * n);
-    CK(cudaMemcpyAsync(acc.data(), h->acc, sizeof(long long) * acc.size(), cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaMemsetAsync(h->acc, 0, sizeof(long long) * acc.size(), h->stream));
-    const int st = read_status(h);
-    if (st != HLBM_OK) return st;
-    const double unit = 1.0 / (double)(1LL << ACC_FRAC_BITS);
-    for (int k = 0; k < n; ++k)
-      for (int j = 0; j < 3; ++j) {
-        F[3 * k + j] = (double)acc[6 * (size_t)k + j] * unit;
-        T[3 * k + j] = (double)acc[6 * (size_t)k + 3 + j] * unit;
-      }
-  } else {
-    CK(launch_mea(part_args(h, parity), h->prm.precision, parity, h->walls, h->stream));
+  CK(launch_mea(part_args(h, parity, moments), h->prm.precision, parity, h->walls, moments, h->stream));
+  {
     std::vector<double> rows((size_t)6 * n);
     CK(cudaMemcpy2DAsync(rows.data(), sizeof(double) * n, h->P + (size_t)PF_F * h->L.cap, sizeof(double) * h->L.cap,
                          sizeof(double) * n, 6, cudaMemcpyDeviceToHost, h->stream));
@@ -1150,7 +1088,6 @@ int hlbm_step_with_forces(hlbm_handle h, const double* F, const double* T) {
     CK(cudaMemcpy2DAsync(h->P + (size_t)PF_F * h->L.cap, sizeof(double) * h->L.cap, rows.data(), sizeof(double) * n,
                          sizeof(double) * n, 6, cudaMemcpyHostToDevice, h->stream));
     PartArgs pa = part_args(h, parity);
-    pa.from_acc = 0;
     CK(launch_contact(pa, h->stream));
     CK(launch_update(pa, h->stream));
   }
@@ -1301,7 +1238,7 @@ int hlbm_set_contact(hlbm_handle h, double k, double zeta) {
 int hlbm_set_mea_mode(hlbm_handle h, int mode) {
   if (!h) return HLBM_ERR_ARG;
   if (mode != HLBM_MEA_KERNEL && mode != HLBM_MEA_MOMENTS) return fail(h, HLBM_ERR_ARG, "unknown momentum-exchange mode");
-  if (mode == HLBM_MEA_MOMENTS && !h->ilist_idx) return fail(h, HLBM_ERR_STATE, "no particle capacity");
+  if (mode == HLBM_MEA_MOMENTS && h->L.cap == 0) return fail(h, HLBM_ERR_STATE, "no particle capacity");
   if (mode != h->mea_mode) {
     CK(cudaStreamSynchronize(h->stream));
     h->mea_mode = mode;
@@ -1483,12 +1420,10 @@ int hlbm_kernel_times(hlbm_handle h, int nsteps, float ms[3]) {
   int rc = HLBM_OK;
   for (int s = 0; s < nsteps; ++s) {
     const int parity = (int)(h->steps & 1);
-    PartArgs pa = part_args(h, parity);
-    const bool fused = h->moments_valid && h->np > 0;
-    pa.from_acc = fused ? 1 : 0;
+    const bool moments = h->moments_valid && h->np > 0;
+    PartArgs pa = part_args(h, parity, moments);
     cudaEventRecord(ev[0], h->stream);
-    if (h->np > 0 && !fused) launch_mea(pa, h->prm.precision, parity, h->walls, h->stream);
-    if (h->np > 0 && fused) launch_mea_moments(lbm_args(h, parity), h->prm.precision, parity, h->walls, h->nsm, h->stream);
+    if (h->np > 0) launch_mea(pa, h->prm.precision, parity, h->walls, moments, h->stream);
     cudaEventRecord(ev[1], h->stream);
     if (h->np > 0) launch_contact(pa, h->stream);
     if (h->np > 0) launch_update(pa, h->stream);
@@ -1515,14 +1450,14 @@ int hlbm_interior_cells(hlbm_handle h, long long* n) {
   if (!h || !n) return HLBM_ERR_ARG;
   *n = 0;
   if (h->np == 0) return HLBM_OK;
-  if (h->mea_mode != HLBM_MEA_MOMENTS || !h->moments_valid || !h->ilist_idx)
-    return fail(h, HLBM_ERR_STATE, "interior cells are counted by a collision in the moments mode");
-  int cnt[ILIST_STRIPES];
-  CK(cudaMemcpyAsync(cnt, h->ilist_count, sizeof(cnt), cudaMemcpyDeviceToHost, h->stream));
+  if (h->mea_mode != HLBM_MEA_MOMENTS || !h->moments_valid)
+    return fail(h, HLBM_ERR_STATE, "interior cells are counted in the moments mode, after a step");
+  unsigned long long t = 0;
+  CK(cudaMemsetAsync(h->count, 0, sizeof(t), h->stream));
+  CK(launch_count_interior(part_args(h, 0, true), h->count, h->stream));
+  CK(cudaMemcpyAsync(&t, h->count, sizeof(t), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
-  long long t = 0;
-  for (int k = 0; k < ILIST_STRIPES; ++k) t += std::min((long long)cnt[k], h->L.ilist_cap);
-  *n = t;
+  *n = (long long)t;
   return read_status(h);
 }
 
@@ -1531,17 +1466,20 @@ int hlbm_interior_cells(hlbm_handle h, long long* n) {
 // Layout (host byte order, no padding): the header below; per box nx, ny,
 // nz, bc (int64); per distance grid nx, ny, nz (int64), the spacing and the
 // samples (FP32); shape and box id per particle (int32); the particle
-// table, PF_COUNT rows of np doubles; the interior-cell list when the next
-// step takes its momentum exchange from it (ILIST_STRIPES int32 counts,
-// then per stripe its int2 entries and its float4 moments); the populations
-// as stored (the handle's own block layout and precision).
+// table, PF_COUNT rows of np doubles; the populations as stored (the
+// handle's own block layout and precision).  A snapshot of the version
+// before ("HLBMCKP3") held, when has_list was set, the list of interior cells
+// between the table and the populations (OLD_STRIPES int32 counts, per stripe
+// 8 + 16 bytes per entry); it is stepped over, the populations hold the same.
 namespace {
 
-constexpr char CK_MAGIC[8] = {'H', 'L', 'B', 'M', 'C', 'K', 'P', '3'};
+constexpr char CK_MAGIC[8] = {'H', 'L', 'B', 'M', 'C', 'K', 'P', '4'};
+constexpr char CK_MAGIC_OLD[8] = {'H', 'L', 'B', 'M', 'C', 'K', 'P', '3'};
+constexpr int OLD_STRIPES = 64;
 
 struct CkHeader {
   char magic[8];
-  int64_t nboxes, precision, fp16_scale_log2, np, pf_count, steps, mea_mode, has_list, pop_bytes, ngrids;
+  int64_t nboxes, precision, fp16_scale_log2, np, pf_count, steps, mea_mode, moments_valid, pop_bytes, ngrids;
   double tau, eps, gravity[3], fluid_force[3], contact_k, contact_zeta;
 };
 
@@ -1549,24 +1487,12 @@ size_t pop_bytes(const hlbm_ctx* h) {
   return (size_t)QVB * h->L.nblocks * (h->prm.precision == HLBM_FP32 ? 4 : 2);
 }
 
-// the snapshot's size, with the interior-list counts it will hold (read
-// from the device when the next step uses the list)
-int snapshot_plan(hlbm_ctx* h, size_t* total, bool* has_list, int cnt[ILIST_STRIPES]) {
+int snapshot_plan(hlbm_ctx* h, size_t* total) {
   const int st = read_status(h);
   if (st != HLBM_OK) return st;
-  *has_list = h->np > 0 && h->moments_valid && h->mea_mode == HLBM_MEA_MOMENTS && h->ilist_idx;
   size_t t = sizeof(CkHeader) + sizeof(int64_t) * 4 * h->boxes.size() + sizeof(int32_t) * 2 * (size_t)h->np +
              sizeof(double) * PF_COUNT * (size_t)h->np;
   for (const auto& g : h->grids) t += sizeof(int64_t) * 3 + sizeof(double) + sizeof(float) * g.v.size();
-  if (*has_list) {
-    CK(cudaMemcpyAsync(cnt, h->ilist_count, sizeof(int) * ILIST_STRIPES, cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-    t += sizeof(int32_t) * ILIST_STRIPES;
-    for (int k = 0; k < ILIST_STRIPES; ++k) {
-      if (cnt[k] < 0 || cnt[k] > h->L.ilist_cap) return fail(h, HLBM_ERR_STATE, "interior-cell list count out of range");
-      t += (sizeof(int2) + sizeof(float4)) * (size_t)cnt[k];
-    }
-  }
   *total = t + pop_bytes(h);
   return HLBM_OK;
 }
@@ -1578,18 +1504,14 @@ extern "C" {
 int hlbm_checkpoint_bytes(hlbm_handle h, size_t* bytes) {
   if (!h || !bytes) return HLBM_ERR_ARG;
   *bytes = 0;
-  bool has_list = false;
-  int cnt[ILIST_STRIPES];
-  return snapshot_plan(h, bytes, &has_list, cnt);
+  return snapshot_plan(h, bytes);
 }
 
 int hlbm_save(hlbm_handle h, void* buf, size_t bytes) {
   if (!h) return HLBM_ERR_ARG;
   if (!buf) return fail(h, HLBM_ERR_ARG, "NULL buffer");
   size_t total = 0;
-  bool has_list = false;
-  int cnt[ILIST_STRIPES];
-  int rc = snapshot_plan(h, &total, &has_list, cnt);
+  int rc = snapshot_plan(h, &total);
   if (rc != HLBM_OK) return rc;
   if (bytes < total) return fail(h, HLBM_ERR_ARG, "buffer smaller than hlbm_checkpoint_bytes");
   char* o = (char*)buf;
@@ -1604,7 +1526,7 @@ int hlbm_save(hlbm_handle h, void* buf, size_t bytes) {
   hd.pf_count = PF_COUNT;
   hd.steps = h->steps;
   hd.mea_mode = h->mea_mode;
-  hd.has_list = has_list ? 1 : 0;
+  hd.moments_valid = h->np > 0 && h->moments_valid && h->mea_mode == HLBM_MEA_MOMENTS ? 1 : 0;
   hd.pop_bytes = (int64_t)pop_bytes(h);
   hd.tau = h->prm.tau;
   hd.eps = h->prm.eps;
@@ -1634,17 +1556,6 @@ int hlbm_save(hlbm_handle h, void* buf, size_t bytes) {
                          cudaMemcpyDeviceToHost, h->stream));
     o += sizeof(double) * PF_COUNT * np;
   }
-  if (has_list) {
-    put(cnt, sizeof(int32_t) * ILIST_STRIPES);
-    for (int k = 0; k < ILIST_STRIPES; ++k) {
-      if (cnt[k] == 0) continue;
-      const size_t k0 = (size_t)k * h->L.ilist_cap;
-      CK(cudaMemcpyAsync(o, h->ilist_idx + k0, sizeof(int2) * cnt[k], cudaMemcpyDeviceToHost, h->stream));
-      o += sizeof(int2) * cnt[k];
-      CK(cudaMemcpyAsync(o, h->ilist_mom + k0, sizeof(float4) * cnt[k], cudaMemcpyDeviceToHost, h->stream));
-      o += sizeof(float4) * cnt[k];
-    }
-  }
   CK(cudaMemcpyAsync(o, h->f, pop_bytes(h), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   return HLBM_OK;
@@ -1665,7 +1576,7 @@ int hlbm_load(hlbm_handle h, const void* buf, size_t bytes) {
     return true;
   };
   CkHeader hd;
-  if (!get(&hd, sizeof(hd)) || std::memcmp(hd.magic, CK_MAGIC, 8) != 0)
+  if (!get(&hd, sizeof(hd)) || (std::memcmp(hd.magic, CK_MAGIC, 8) != 0 && std::memcmp(hd.magic, CK_MAGIC_OLD, 8) != 0))
     return fail(h, HLBM_ERR_ARG, "not a snapshot of this library");
   if (hd.pf_count != PF_COUNT) return fail(h, HLBM_ERR_ARG, "snapshot of another particle table layout");
   if (hd.nboxes != (int64_t)h->boxes.size() || hd.precision != h->prm.precision ||
@@ -1711,16 +1622,13 @@ int hlbm_load(hlbm_handle h, const void* buf, size_t bytes) {
   if (!get(shp.data(), sizeof(int32_t) * n) || !get(bx.data(), sizeof(int32_t) * n) ||
       !get(tab.data(), sizeof(double) * tab.size()))
     return fail(h, HLBM_ERR_ARG, "truncated snapshot");
-  int cnt[ILIST_STRIPES] = {0};
-  std::vector<const char*> lst(ILIST_STRIPES, nullptr);
-  if (hd.has_list) {
+  if (hd.moments_valid && std::memcmp(hd.magic, CK_MAGIC_OLD, 8) == 0) {
+    int32_t cnt[OLD_STRIPES];
     if (!get(cnt, sizeof(cnt))) return fail(h, HLBM_ERR_ARG, "truncated snapshot");
-    for (int k = 0; k < ILIST_STRIPES; ++k) {
-      if (cnt[k] < 0 || cnt[k] > h->L.ilist_cap || !h->ilist_idx)
-        return fail(h, HLBM_ERR_ARG, "snapshot's interior-cell list does not fit this handle");
+    for (int k = 0; k < OLD_STRIPES; ++k) {
+      if (cnt[k] < 0 || h->L.cap == 0) return fail(h, HLBM_ERR_ARG, "snapshot's interior-cell list does not fit this handle");
       const size_t nb = (sizeof(int2) + sizeof(float4)) * (size_t)cnt[k];
       if ((size_t)(end - i) < nb) return fail(h, HLBM_ERR_ARG, "truncated snapshot");
-      lst[k] = i;
       i += nb;
     }
   }
@@ -1750,27 +1658,16 @@ int hlbm_load(hlbm_handle h, const void* buf, size_t bytes) {
                          PF_COUNT, cudaMemcpyHostToDevice, h->stream));
     CK(launch_records(part_args(h, 0), h->stream));
   }
-  CK(cudaMemsetAsync(h->ilist_count, 0, sizeof(int) * ILIST_STRIPES, h->stream));
-  if (hd.has_list) {
-    CK(cudaMemcpyAsync(h->ilist_count, cnt, sizeof(cnt), cudaMemcpyHostToDevice, h->stream));
-    for (int k = 0; k < ILIST_STRIPES; ++k) {
-      if (cnt[k] == 0) continue;
-      const size_t k0 = (size_t)k * h->L.ilist_cap;
-      CK(cudaMemcpyAsync(h->ilist_idx + k0, lst[k], sizeof(int2) * cnt[k], cudaMemcpyHostToDevice, h->stream));
-      CK(cudaMemcpyAsync(h->ilist_mom + k0, lst[k] + sizeof(int2) * cnt[k], sizeof(float4) * cnt[k],
-                         cudaMemcpyHostToDevice, h->stream));
-    }
-  }
   for (int k = 0; k < 2; ++k) CK(cudaMemsetAsync(h->cnt[k], 0, sizeof(int) * (size_t)h->L.ntiles, h->stream));
   CK(cudaMemcpyAsync(h->f, pops, pop_bytes(h), cudaMemcpyHostToDevice, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   for (int j = 0; j < 3; ++j) h->prm.fluid_force[j] = hd.fluid_force[j];
   h->contact_k = hd.contact_k;
   h->contact_zeta = hd.contact_zeta;
-  // the saver's momentum-exchange mode, where this handle can hold its list
-  if (hd.mea_mode == HLBM_MEA_KERNEL || h->ilist_idx) h->mea_mode = (int)hd.mea_mode;
+  // the saver's momentum-exchange mode, where this handle has particles
+  if (hd.mea_mode == HLBM_MEA_KERNEL || h->L.cap > 0) h->mea_mode = (int)hd.mea_mode;
   h->steps = hd.steps;
-  h->moments_valid = hd.has_list != 0 && h->mea_mode == HLBM_MEA_MOMENTS;
+  h->moments_valid = hd.moments_valid != 0 && h->mea_mode == HLBM_MEA_MOMENTS;
   drop_graphs(h);
   return read_status(h);
 }

@@ -49,57 +49,19 @@ __host__ __device__ constexpr double wq(int i) {
   return i == 0 ? 1.0 / 3.0 : (i <= 6 ? 1.0 / 18.0 : 1.0 / 36.0);
 }
 
-// Division of an unsigned 32-bit n by a divisor d >= 1 fixed at set-up, with
-// one high multiply (Granlund and Montgomery 1994, the unsigned case of
-// their Fig. 4.1): with l = ceil(log2 d), m = floor(2^32 (2^l - d) / d) + 1
-// and t = mulhi(m, n), n / d = (t + ((n - t) >> min(l, 1))) >> max(l - 1, 0),
-// exact for every n.
-struct FastDiv {
-  unsigned m;
-  int s1, s2;
-};
-inline FastDiv make_fastdiv(unsigned d) {
-  int l = 0;
-  while ((1ull << l) < d) ++l;
-  FastDiv f;
-  f.m = (unsigned)(((1ull << 32) * ((1ull << l) - d)) / d + 1);
-  f.s1 = l < 1 ? l : 1;
-  f.s2 = l > 1 ? l - 1 : 0;
-  return f;
-}
-__device__ __forceinline__ unsigned fast_div(unsigned n, const FastDiv& f) {
-  const unsigned t = __umulhi(f.m, n);
-  return (t + ((n - t) >> f.s1)) >> f.s2;
-}
-
 struct BoxDesc {
   int nx, ny, nz, bc;        // bc: bit a set = walls on axis a; BC_CUT_Z: see below
   int ntx, nty, ntz;         // bin tiles per axis (ntx = storage blocks per row)
   int own_lo, own_hi;        // owned z planes [own_lo, own_hi) of a BC_CUT_Z box
-  FastDiv div_x, div_y;      // division by nx and by ny
-  long long cell_off;        // first cell of the box in the global cell numbering
   long long tile_off;        // first bin tile of the box
   long long blk_off;         // first storage block of the box
 };
-
-// coordinates of cell c (c < nx ny nz) of a box
-__device__ __forceinline__ void cell_coords(const BoxDesc& bd, unsigned c, int& x, int& y, int& z) {
-  const unsigned r = fast_div(c, bd.div_x);
-  const unsigned q = fast_div(r, bd.div_y);
-  x = (int)(c - r * (unsigned)bd.nx);
-  y = (int)(r - q * (unsigned)bd.ny);
-  z = (int)q;
-}
 
 // A box with BC_CUT_Z (set together with the z-wall bit) is one z slab of a
 // larger lattice: its z faces bound the lattice as walls do (only its ghost
 // planes meet them), particle centres may lie beyond them, and only the
 // cells of the owned planes [own_lo, own_hi) enter the momentum exchange.
 constexpr int BC_CUT_Z = 8;
-
-__host__ __device__ __forceinline__ bool owned_plane(const BoxDesc& bd, int z) {
-  return !(bd.bc & BC_CUT_Z) || (z >= bd.own_lo && z < bd.own_hi);
-}
 
 // blocked population storage (layout above)
 constexpr int VB = 32;       // cells per storage block (= TILE_X)
@@ -127,9 +89,6 @@ enum {
 // a particle's bounding box spans at most this many planes (circumscribed
 // radius <= 30 cells)
 constexpr int MAX_PLANES = 64;
-
-// stripes of the list of interior cells (a power of two)
-constexpr int ILIST_STRIPES = 64;
 
 // Signed-distance grids (shape 4): FP32 samples of a body-frame signed
 // distance, point (i, j, k) at ((i - half_0) h, (j - half_1) h, (k - half_2) h)
@@ -185,7 +144,7 @@ struct __align__(16) Rec {
   float xh[3], xl[3];  // centre as float pair: X = xh + xl
   float u[3], w[3];    // velocity, angular velocity
   float M[9];          // rotation body -> world, row-major; a sphere's
-                       // first four: its collision bounds (SPH_* below)
+                       // first two: its collision bounds (SPH_* below)
   float a[3];          // radius / semi-axes / half-extents / capsule (r, r, h);
                        // a grid's circumscribed radius
   float ia[3];         // fp32(1 / a_j) (ellipsoid inside test)
@@ -197,10 +156,9 @@ struct __align__(16) Rec {
   int pid;
 };
 static_assert(sizeof(Rec) == 128, "record size");
-// a sphere's record: in2 * 0.99999 and in2 * 1.00001 (below / above them the
-// centre-inside decision needs no exact test), (a - eps/2)^2 (-1 when
-// a <= eps/2) and (a + eps/2)^2 (B is 1 within, 0 beyond), all FP32
-enum { SPH_IN_LO = 0, SPH_IN_HI = 1, SPH_R2_IN = 2, SPH_R2_OUT = 3 };
+// a sphere's record: (a - eps/2)^2 (-1 when a <= eps/2) and (a + eps/2)^2 (B is
+// 1 within, 0 beyond), FP32
+enum { SPH_R2_IN = 0, SPH_R2_OUT = 1 };
 
 // The moments-mode momentum exchange adds its per-cell FP32 terms as 64-bit
 // integers in units of 2^-ACC_FRAC_BITS: integer sums do not depend on the
@@ -210,9 +168,8 @@ enum { SPH_IN_LO = 0, SPH_IN_HI = 1, SPH_R2_IN = 2, SPH_R2_OUT = 3 };
 constexpr int ACC_FRAC_BITS = 44;
 
 // status flags: ST_CAPACITY a tile's particle list is full; ST_OVERLAP three
-// particles hold one cell (the list of interior cells takes two per cell);
-// ST_LIST_FULL a stripe of the list of interior cells is full
-enum { ST_UNSTABLE = 1, ST_CAPACITY = 2, ST_LEFT_DOMAIN = 4, ST_INTERNAL = 8, ST_OVERLAP = 16, ST_LIST_FULL = 32 };
+// particles hold one cell
+enum { ST_UNSTABLE = 1, ST_CAPACITY = 2, ST_LEFT_DOMAIN = 4, ST_OVERLAP = 16 };
 
 // neighbour index helper: per-axis neighbour offsets; -1 marks a node beyond
 // a wall (only possible when WALLS)
@@ -265,18 +222,6 @@ __device__ __forceinline__ NbrB make_nbr_blocked(const BoxDesc& bd, int x, int y
   return n;
 }
 
-// neighbour offsets in global cell indices (the box's first cell added):
-// at() returns the global index, or a negative value beyond a wall
-template <bool WALLS>
-__device__ __forceinline__ Nbr<WALLS> make_nbr_global(const BoxDesc& bd, int x, int y, int z) {
-  Nbr<WALLS> n = make_nbr<WALLS>(bd, x, y, z);
-  const int off = (int)bd.cell_off;
-  n.z += off;
-  n.zm = n.zm < 0 ? n.zm : n.zm + off;
-  n.zp = n.zp < 0 ? n.zp : n.zp + off;
-  return n;
-}
-
 template <bool WALLS>
 __device__ __forceinline__ Nbr<WALLS> make_nbr(const BoxDesc& bd, int x, int y, int z) {
   Nbr<WALLS> n;
@@ -326,7 +271,6 @@ struct LbmArgs {
   // finish, take no SM room this grid's remaining blocks still need
   long long pdl_tail;
   void* f;                  // populations, blocked layout (float* or __half*)
-  long long ncell;          // cells of all boxes (global cell numbering)
   const BoxDesc* boxes;
   int nboxes;
   int sub_y, sub_z;         // brick per block: 32 x sub_y x sub_z cells
@@ -344,20 +288,6 @@ struct LbmArgs {
   const int* bin_ids;
   int bin_cap;
   const Rec* rec;
-  // list of the cells inside particles, appended by the collision for the
-  // next step's momentum exchange (nullptr: not recorded):
-  //   ilist_idx[k] = (global cell index, particle), ilist_mom[k] = mass and
-  //   momentum of the cell's post-collision deviations as stored.
-  // It is split into ILIST_STRIPES stripes of ilist_cap entries, stripe s at
-  // [s * ilist_cap, (s + 1) * ilist_cap) with its own count ilist_count[s];
-  // a collision block appends to stripe (block index mod ILIST_STRIPES), so
-  // the appends of the whole grid do not contend for one counter.
-  int* ilist_count;
-  int2* ilist_idx;
-  float4* ilist_mom;
-  long long ilist_cap;
-  int np;                   // particles (list entries name 0 .. np-1)
-  long long* acc;           // [cap][6] momentum exchange of a particle, fixed point
   GridSet grids;            // signed-distance grids of shape-4 particles
   int* status;
 };
@@ -375,28 +305,23 @@ struct PartArgs {
   // momentum exchange input
   const void* f;            // populations, blocked layout
   float scale, inv_scale;
-  // momentum-exchange kernel: one block per particle and run of planes
-  const int* chunk_p;       // [chunks] particle of the block
-  const int* chunk_q;       // [chunks] first plane of the block
-  const int* p_chunk0;      // [cap] first block of a particle
-  const int* p_nchunk;      // [cap] blocks of a particle
-  const int* p_planes;      // [cap] bounding-box planes per block of a particle
-  int mea_group;            // planes whose cells are summed together
+  // momentum exchange: block k walks part of particle chunks[k].x, from plane
+  // chunks[k].y on chunks[k].z planes; the particle has chunks[k].w blocks
+  const int4* chunks;
   int nchunks;
+  int mea_group;            // planes whose cells are summed together
   int mea_threads;          // threads per momentum-exchange block
   double* partial;          // [cap][MAX_PLANES][6] FP64 sums of the groups of planes
   int* done;                // [cap] blocks finished per particle (reset to 0)
-  // the same sums added up by the moments-mode momentum exchange from the
-  // moments the previous collision recorded
-  long long* acc;           // [cap][6] momentum exchange, fixed point (ACC_FRAC_BITS)
-  int from_acc;             // 1: the update takes acc, 0: the table's F and T
+  // the moments-mode momentum exchange adds the blocks of a particle here
+  long long* acc;           // [cap][6] momentum exchange, fixed point (ACC_FRAC_BITS); 0 between steps
+  int cells_x;              // the collision's cells per thread (its order of summing a cell's departures)
   // contact between the particles' enclosing capsules and with the walls
   // (an extension; off when contact_k == 0): stiffness and range
   double contact_k, contact_zeta;
   GridSet grids;            // signed-distance grids of shape-4 particles
   int nsm;                  // SMs of the GPU (update grid size)
   int ppb;                  // particles per update block (set by the launcher)
-  int* ilist_count;         // [ILIST_STRIPES], reset by the update for the next collision
   // bins written by the update (this step) and cleared (other parity)
   int* bin_count;
   int* bin_ids;
@@ -479,11 +404,11 @@ cudaError_t launch_collide(const LbmArgs& a, int precision, int parity, bool wal
 // the collision with two x-adjacent cells per thread (a.cells_x == 2)
 cudaError_t launch_collide_pair(const LbmArgs& a, int precision, int parity, bool walls, bool couple,
                                 cudaStream_t s);
-// momentum exchange from the arrivals and the moments recorded in the list of
-// interior cells (a.rec must describe the particle state of this step)
-cudaError_t launch_mea_moments(const LbmArgs& a, int precision, int parity, bool walls, int nsm,
-                               cudaStream_t s);
-cudaError_t launch_mea(const PartArgs& a, int precision, int parity, bool walls, cudaStream_t s);
+// momentum exchange; moments: the fixed-point form, otherwise the link sums in
+// their fixed order
+cudaError_t launch_mea(const PartArgs& a, int precision, int parity, bool walls, bool moments, cudaStream_t s);
+// number of (cell, particle) pairs with the cell centre inside, added to *count
+cudaError_t launch_count_interior(const PartArgs& a, unsigned long long* count, cudaStream_t s);
 cudaError_t launch_update(const PartArgs& a, cudaStream_t s);
 // contact force and torque of every particle into PF_FC / PF_TC (only when
 // a.contact_k > 0)

@@ -2,8 +2,7 @@
 // per thread in lbm_kernels.cu, two x-adjacent cells per thread in
 // lbm_pair_kernels.cu): storage access, the indicator of Eq. B, the signed
 // distances of the four shapes, the per-tile particle candidates and the
-// per-cell coupling of Eq. hlbm:du (Sec. 3.2), and the list of cells inside
-// particles that the collision appends for the next momentum exchange.
+// per-cell coupling of Eq. hlbm:du (Sec. 3.2).
 #pragma once
 #include "hlbm_internal.cuh"
 
@@ -39,13 +38,6 @@ template <> struct Pop<__half> {
     *reinterpret_cast<__half2*>(p) = __float22half2_rn(v);
   }
 };
-// the value a store of v leaves in memory, read back as a deviation
-template <typename S>
-__device__ __forceinline__ float stored_value(float v, float s, float inv_s) {
-  if (sizeof(S) == 4) return v;
-  return __half2float(__float2half_rn(v * s)) * inv_s;
-}
-
 // Addressing of a thread's cells x .. x + n - 1 (one row, one storage block)
 // for the collide-and-stream: the rows y - 1, y, y + 1 as block offsets, and
 // the x neighbours left of the first and right of the last cell as element
@@ -347,12 +339,13 @@ __device__ __forceinline__ void load_candidates(const LbmArgs& a, const Brick& k
 
 // Coupling of N consecutive cells x, x+1, .. of one row with the candidates
 // in rm: the largest indicator B (ties to the lowest particle id) with its
-// particle velocity u_p(x) = U + w x (x - X) (Eq. hlbm:du), and up to two
-// particles whose inside holds the cell's centre.
+// particle velocity u_p(x) = U + w x (x - X) (Eq. hlbm:du).  Three particles
+// holding one cell's centre are flagged; only rows of three or more
+// candidates can, and only they pay for the inside test.
 template <int N>
 struct RowCoupling {
   float B[N], upx[N], upy[N], upz[N];
-  int bestp[N], ip0[N], ip1[N];
+  int bestp[N];
 };
 
 template <int N, bool GRIDS>
@@ -366,8 +359,11 @@ __device__ __forceinline__ void couple_row(const Rec* srec, unsigned long long r
     cc.B[j] = 0.0f;
     cc.upx[j] = cc.upy[j] = cc.upz[j] = 0.0f;
     cc.bestp[j] = 0x7fffffff;
-    cc.ip0[j] = cc.ip1[j] = -1;
   }
+  const bool crowded = __popcll(rm) > 2;
+  int inside[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) inside[j] = 0;
   const float Lx = (float)bd.nx, Ly = (float)bd.ny, Lz = (float)bd.nz;
   while (rm) {
     const int k = __ffsll((long long)rm) - 1;
@@ -378,13 +374,12 @@ __device__ __forceinline__ void couple_row(const Rec* srec, unsigned long long r
     if (!(bd.bc & 4)) { if (r0z > 0.5f * Lz) r0z -= Lz; else if (r0z < -0.5f * Lz) r0z += Lz; }
     const float ry = __fsub_rn(r0y, R.xl[1]), rz = __fsub_rn(r0z, R.xl[2]);
     const float d2 = ry * ry + rz * rz;
-    // the cell's coupling to R: the particle id if its centre is inside, and
-    // the indicator with the particle velocity there when it is the largest
-    auto take = [&](int j, float rx, bool in, float B) {
-      if (in) {
-        if (cc.ip0[j] < 0) cc.ip0[j] = R.pid;
-        else if (cc.ip1[j] < 0) cc.ip1[j] = R.pid;
-        else atomicOr(status, ST_OVERLAP);  // three overlapping particles
+    // the cell's coupling to R: the indicator with the particle velocity
+    // there when it is the largest
+    auto take = [&](int j, float rx, float B) {
+      if (crowded) {
+        const float rr[3] = {rx, ry, rz};
+        if (inside_from_offset(R, rr, gs) && ++inside[j] > 2) atomicOr(status, ST_OVERLAP);
       }
       if (B > cc.B[j] || (B == cc.B[j] && B > 0.0f && R.pid < cc.bestp[j])) {
         cc.B[j] = B;
@@ -399,28 +394,18 @@ __device__ __forceinline__ void couple_row(const Rec* srec, unsigned long long r
       if (!(bd.bc & 1)) { if (r0x > 0.5f * Lx) r0x -= Lx; else if (r0x < -0.5f * Lx) r0x += Lx; }
       return __fsub_rn(r0x, R.xl[0]);
     };
-    // The inside decision is the exactly rounded test of inside_from_offset;
-    // away from the surface the distance evaluated here (contracted
-    // arithmetic) has the same sign, and only cells within a margin far above
-    // the rounding difference of the two take the exact test (sphere: 1e-5
-    // relative in r^2; other shapes: 1e-3 cells).
     if (R.shape == 0) {
       // a sphere's indicator is 1 within r <= a - eps/2 and 0 beyond a + eps/2:
       // only cells in that shell need the distance and the ramp (bounds
       // precomputed in the record)
-      const float in_lo = R.M[SPH_IN_LO], in_hi = R.M[SPH_IN_HI];
       const float r2_in = R.M[SPH_R2_IN], r2_out = R.M[SPH_R2_OUT];
 #pragma unroll
       for (int j = 0; j < N; ++j) {
         const float rx = arm_x(j);
         const float r2 = rx * rx + d2;
         if (r2 < R.rinf2) {
-          bool in;
-          if (r2 < in_lo) in = true;
-          else if (r2 > in_hi) in = false;
-          else { const float rr[3] = {rx, ry, rz}; in = inside_from_offset(R, rr); }
           const float B = r2 <= r2_in ? 1.0f : (r2 >= r2_out ? 0.0f : indicator(sdf(R, rx, ry, rz, r2), eps, inv_eps));
-          take(j, rx, in, B);
+          take(j, rx, B);
         }
       }
     } else {
@@ -433,72 +418,8 @@ __device__ __forceinline__ void couple_row(const Rec* srec, unsigned long long r
         const float r2 = rx * rx + d2;
         if (r2 < R.rinf2 && capsule_dist2(cap, rx, ry, rz) < cap.r2) {
           const float d = sdf(R, rx, ry, rz, r2, gs);
-          bool in;
-          if (d < -1e-3f) in = true;
-          else if (d > 1e-3f) in = false;
-          else { const float rr[3] = {rx, ry, rz}; in = inside_from_offset(R, rr, gs); }
-          take(j, rx, in, indicator(d, eps, inv_eps));
+          take(j, rx, indicator(d, eps, inv_eps));
         }
-      }
-    }
-  }
-}
-
-__device__ __forceinline__ unsigned lane_id() {
-  unsigned l;
-  asm("mov.u32 %0, %%laneid;" : "=r"(l));
-  return l;
-}
-
-__device__ __forceinline__ unsigned lanemask_lt() {
-  unsigned m;
-  asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
-  return m;
-}
-
-// Warp-aggregated append of the cells g, g+1, .. g+N-1 that lie inside a
-// particle to the list of interior cells: one entry (cell, particle) per
-// particle holding the cell, with the mass and momentum of the cell's
-// post-collision deviations as stored.  Called by all active lanes, which
-// may be any subset of the warp: a lane's offset among the warp's entries
-// is taken bit by bit of its entry count (one ballot per bit), so no lane
-// depends on a value passed through another.
-template <int N>
-__device__ __forceinline__ void append_interior(const LbmArgs& a, unsigned g, const RowCoupling<N>& cc,
-                                                const float4 (&mom)[N]) {
-  int nent = 0;
-#pragma unroll
-  for (int j = 0; j < N; ++j) nent += (cc.ip0[j] >= 0) + (cc.ip1[j] >= 0);
-  const unsigned act = __activemask();
-  if (!__ballot_sync(act, nent > 0)) return;
-  const unsigned lt = lanemask_lt();
-  int before = 0, total = 0;
-#pragma unroll
-  for (int b = 0; (1 << b) <= 2 * N; ++b) {
-    const unsigned m = __ballot_sync(act, (nent >> b) & 1);
-    before += __popc(m & lt) << b;
-    total += __popc(m) << b;
-  }
-  const int leader = __ffs(act) - 1;
-  const int stripe = (int)(blockIdx.x & (ILIST_STRIPES - 1));
-  int base = 0;
-  if ((int)lane_id() == leader) base = atomicAdd(&a.ilist_count[stripe], total);
-  base = __shfl_sync(act, base, leader);
-  long long k = (long long)base + before;  // within the stripe
-  const long long k0 = (long long)stripe * a.ilist_cap;
-#pragma unroll
-  for (int j = 0; j < N; ++j) {
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int p = e == 0 ? cc.ip0[j] : cc.ip1[j];
-      if (p >= 0) {
-        if (k < a.ilist_cap) {
-          a.ilist_idx[k0 + k] = make_int2((int)(g + j), p);
-          a.ilist_mom[k0 + k] = mom[j];
-        } else {
-          atomicOr(a.status, ST_LIST_FULL);
-        }
-        ++k;
       }
     }
   }

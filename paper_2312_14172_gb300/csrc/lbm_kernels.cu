@@ -51,7 +51,6 @@ __global__ void __launch_bounds__(256, HLBM_CS_MINBLOCKS) collide_stream_kernel(
 
 #pragma unroll 1
   for (int z = z0; z < z1; ++z) {
-    const unsigned g = (unsigned)(bd.cell_off + (z * bd.ny + y) * bd.nx + x);  // global cell index
     int zb[3];
     slice_blocks<WALLS>(bd, z, zb);
     S* const own = cell_ptr(f, zb[1] + rb.yb[1] + rb.xb, rb.xin);
@@ -152,216 +151,8 @@ __global__ void __launch_bounds__(256, HLBM_CS_MINBLOCKS) collide_stream_kernel(
         Pop<S>::st_raw(p, o[i]);
       }
     }
-    // cells inside a particle record the mass and momentum they send out, as
-    // stored, for the next step's momentum exchange (one entry per particle)
-    if (COUPLE && a.ilist_idx) {
-      float4 mom[1] = {make_float4(0.f, 0.f, 0.f, 0.f)};
-      if (cc.ip0[0] >= 0) {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-          const float v = stored_value<S>(o[i], 1.0f, isc);
-          mom[0].x += v;
-          if (cx(i)) mom[0].y += (float)cx(i) * v;
-          if (cy(i)) mom[0].z += (float)cy(i) * v;
-          if (cz(i)) mom[0].w += (float)cz(i) * v;
-        }
-      }
-      if (owned_plane(bd, z)) append_interior<1>(a, g, cc, mom);
-    }
   }
   if (!early) pdl_trigger();
-}
-
-// ---------------------------------------------------------------------------
-// Momentum exchange (Eq. hlbm:mea, summed by Eqs. hydrodynamicforce and
-// hydrodynamictorque) from moments.  Per interior cell x the used-sign sum
-//   F(x) = sum_i (c_i - u_p) f_i(x) + (c_i + u_p) f_ibar(x - c_i)
-// is the momentum the cell gained by the last streaming, minus u_p times the
-// mass it gained: the arrivals f_i(x) give j(x) and rho(x); the departures
-// f_ibar(x - c_i) = f*_ibar(x) are the cell's own post-collision values, whose
-// moments the previous collision recorded in the list of interior cells:
-//   F(x) = (j - j*) - u_p(x) (rho - rho*)  [links into a wall: - 2 c_i f_i(x)]
-// A persistent grid walks the list (one entry per thread, all 19 loads of a
-// cell in flight together); each cell's terms are rounded to fixed point
-// (ACC_FRAC_BITS), and the lanes of a warp that belong to the same particle
-// are summed as integers before one 64-bit integer atomic per particle,
-// component and warp: the sums do not depend on the list's order.
-
-// Exact warp sum of the 64-bit values of the lanes in mask (the others give
-// 0), from three limbs with single-instruction warp reductions: v =
-// a 2^42 + b 2^21 + c with c, b in [0, 2^21) and a = v >> 42 in [-2^21,
-// 2^21), so 32 lanes' limb sums stay within 32 bits.
-__device__ __forceinline__ long long warp_sum_i64(long long v) {
-  const unsigned c = (unsigned)v & 0x1fffffu;
-  const unsigned b = (unsigned)(v >> 21) & 0x1fffffu;
-  const int hi = (int)(v >> 42);
-  const unsigned sc = __reduce_add_sync(0xffffffffu, c);
-  const unsigned sb = __reduce_add_sync(0xffffffffu, b);
-  const int sa = __reduce_add_sync(0xffffffffu, hi);
-  return (long long)(((unsigned long long)(long long)sa << 42) + ((unsigned long long)sb << 21) + sc);
-}
-
-// resident blocks per SM: four with walls (64 registers), five without
-#ifndef HLBM_ML_MINBLOCKS_W
-#define HLBM_ML_MINBLOCKS_W 4
-#endif
-#ifndef HLBM_ML_MINBLOCKS
-#define HLBM_ML_MINBLOCKS 5
-#endif
-template <typename S, int PAR, bool WALLS>
-__global__ void __launch_bounds__(256, WALLS ? HLBM_ML_MINBLOCKS_W : HLBM_ML_MINBLOCKS) mea_list_kernel(LbmArgs a) {
-  pdl_trigger();
-  pdl_wait();
-  // The list is walked in chunks of 32 entries, the stripes taken in turn
-  // and each stripe from its end: the first wave reads the arrivals the
-  // collision wrote last, which L2 still holds.  Chunk q covers entries
-  // [c_s - 32 (j + 1), c_s - 32 j) of stripe s = q mod 64, j = q / 64, c_s the
-  // stripe's count; the lanes take them in ascending order, so that a run of
-  // cells the collision appended together stays in one warp.
-  __shared__ int s_cnt[ILIST_STRIPES];
-  __shared__ int s_chunks;  // chunks per stripe
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    const int c0 = (int)min((long long)a.ilist_count[lane], a.ilist_cap);
-    const int c1 = (int)min((long long)a.ilist_count[lane + 32], a.ilist_cap);
-    s_cnt[lane] = c0;
-    s_cnt[lane + 32] = c1;
-    int m = max(c0, c1);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if (lane == 0) s_chunks = (m + 31) / 32;
-  }
-  __syncthreads();
-  const long long nq = (long long)ILIST_STRIPES * s_chunks;
-  const int lane = threadIdx.x & 31;
-  const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
-  const S* fbase = reinterpret_cast<const S*>(a.f);
-  // position of this lane's entry in chunk q (negative: none), its index in
-  // the striped list, and the entry with its recorded moments; loaded one
-  // chunk ahead, so that the next entry is on its way while this one's
-  // arrivals are read
-  auto fetch = [&](long long q, int& pos, int2& e, float4& m) {
-    pos = -1;
-    e = make_int2(0, -1);
-    m = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (q < nq) {
-      const int st = (int)(q & (ILIST_STRIPES - 1)), j = (int)(q / ILIST_STRIPES);
-      pos = s_cnt[st] - 32 * (j + 1) + lane;
-      if (pos >= 0) {
-        const long long k = (long long)st * a.ilist_cap + pos;
-        e = a.ilist_idx[k];
-        m = a.ilist_mom[k];
-      }
-    }
-  };
-  long long q = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5);
-  int pos_next;
-  int2 e_next;
-  float4 m_next;
-  fetch(q, pos_next, e_next, m_next);
-  for (; q < nq; q += nwarps) {
-    bool valid = pos_next >= 0;
-    const bool listed = valid;
-    int pid = -1;
-    float F[3] = {0.f, 0.f, 0.f}, T[3] = {0.f, 0.f, 0.f};
-    const int2 e = e_next;
-    const float4 sd = m_next;
-    fetch(q + nwarps, pos_next, e_next, m_next);
-    // an entry names a particle and a cell of that particle's box; anything
-    // else was never written by the collision and is skipped with a flag
-    if (valid && (e.y < 0 || e.y >= a.np)) valid = false;
-    // one box: its descriptor does not wait for the particle's record
-    const BoxDesc bd = a.boxes[a.nboxes == 1 || !valid ? 0 : a.rec[e.y].box];
-    const long long cl = (long long)e.x - bd.cell_off;
-    if (valid && (cl < 0 || cl >= (long long)bd.nx * bd.ny * bd.nz)) valid = false;
-    if (listed && !valid) atomicOr(a.status, ST_INTERNAL);
-    int x = 0, y = 0, z = 0;
-    if (valid) cell_coords(bd, (unsigned)cl, x, y, z);
-    // cells next to a wall take the wall selects; a warp without any runs
-    // the plain neighbour arithmetic (the same for cells off the walls)
-    bool edge = false;
-    if (WALLS && valid)
-      edge = ((bd.bc & 1) && (x == 0 || x == bd.nx - 1)) || ((bd.bc & 2) && (y == 0 || y == bd.ny - 1)) ||
-             ((bd.bc & 4) && (z == 0 || z == bd.nz - 1));
-    auto cell_terms = [&](auto wtag) {
-      constexpr bool W = decltype(wtag)::value;
-      const Rec& R = a.rec[pid];
-      float r[3];
-      r[0] = offset_fp32(x, bd.nx, bd.bc & 1, R.xh[0], R.xl[0]);
-      r[1] = offset_fp32(y, bd.ny, bd.bc & 2, R.xh[1], R.xl[1]);
-      r[2] = offset_fp32(z, bd.nz, bd.bc & 4, R.xh[2], R.xl[2]);
-      // arrivals f_i(x) (AA accessor): slot i of x (even parity), slot ibar of
-      // x - c_i (odd parity), or slot i of x when x - c_i lies beyond a wall
-      const RowBlocks rb = row_blocks<W>(bd, x, y, 1);
-      int zb[3];
-      slice_blocks<W>(bd, z, zb);
-      const S* own = cell_ptr(fbase, zb[1] + rb.yb[1] + rb.xb, rb.xin);
-      float d[Q];
-      unsigned walls = 0;  // bit i: x - c_i lies beyond a wall
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        const int by = rb.yb[1 - cy(i)], bz = zb[1 - cz(i)];
-        const bool wall = W && i > 0 && (by < 0 || bz < 0 || (cx(i) > 0 && rb.wl) || (cx(i) < 0 && rb.wr));
-        if (wall) walls |= 1u << i;
-        if (PAR == 0 || i == 0) {
-          d[i] = Pop<S>::ld(own + i * VB, a.inv_scale);
-        } else {
-          const int dx = cx(i) > 0 ? rb.dl : (cx(i) < 0 ? rb.dr : 0);
-          const S* src = wall ? own + i * VB : cell_ptr(fbase, bz + by + rb.xb, rb.xin) + (dx + opp(i) * VB);
-          d[i] = Pop<S>::ld(src, a.inv_scale);
-        }
-      }
-      float ms = 0.f, px = 0.f, py = 0.f, pz = 0.f;
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        ms += d[i];
-        if (cx(i)) px += (float)cx(i) * d[i];
-        if (cy(i)) py += (float)cy(i) * d[i];
-        if (cz(i)) pz += (float)cz(i) * d[i];
-      }
-      const float upx = R.u[0] + (R.w[1] * r[2] - R.w[2] * r[1]);
-      const float upy = R.u[1] + (R.w[2] * r[0] - R.w[0] * r[2]);
-      const float upz = R.u[2] + (R.w[0] * r[1] - R.w[1] * r[0]);
-      const float dm = ms - sd.x;
-      F[0] = (px - sd.y) - upx * dm;
-      F[1] = (py - sd.z) - upy * dm;
-      F[2] = (pz - sd.w) - upz * dm;
-      if (W) {
-#pragma unroll
-        for (int i = 1; i < Q; ++i)
-          if ((walls >> i) & 1u) {
-            const float v = 2.0f * ((float)wq(i) + d[i]);
-            if (cx(i)) F[0] -= (float)cx(i) * v;
-            if (cy(i)) F[1] -= (float)cy(i) * v;
-            if (cz(i)) F[2] -= (float)cz(i) * v;
-          }
-      }
-      T[0] = r[1] * F[2] - r[2] * F[1];
-      T[1] = r[2] * F[0] - r[0] * F[2];
-      T[2] = r[0] * F[1] - r[1] * F[0];
-    };
-    if (valid) pid = e.y;
-    if (WALLS && __any_sync(0xffffffffu, edge)) {
-      if (valid) cell_terms(std::integral_constant<bool, WALLS>{});
-    } else if (valid) {
-      cell_terms(std::integral_constant<bool, false>{});
-    }
-    // sum the lanes of each particle present in the warp
-    unsigned todo = __ballot_sync(0xffffffffu, valid);
-    while (todo) {
-      const int leader = __ffs(todo) - 1;
-      const int p = __shfl_sync(0xffffffffu, pid, leader);
-      const bool mine = valid && pid == p;
-      todo &= ~__ballot_sync(0xffffffffu, mine);
-#pragma unroll
-      for (int c = 0; c < 6; ++c) {
-        const float t = c < 3 ? F[c] : T[c - 3];
-        const long long v = warp_sum_i64(mine ? __float2ll_rn(__fmul_rn(t, (float)(1LL << ACC_FRAC_BITS))) : 0LL);
-        if (lane == leader)
-          atomicAdd(reinterpret_cast<unsigned long long*>(&a.acc[(long long)p * 6 + c]), (unsigned long long)v);
-      }
-    }
-  }
 }
 
 template <typename S, int PAR, bool W, int C>
@@ -393,32 +184,6 @@ cudaError_t launch_collide(const LbmArgs& a, int precision, int parity, bool wal
   if (a.cells_x == 2) return launch_collide_pair(a, precision, parity, walls, couple, s);
   return precision == 0 ? launch_cs_prec<float>(a, parity, walls, couple, s)
                         : launch_cs_prec<__half>(a, parity, walls, couple, s);
-}
-
-// one wave of resident blocks walks the whole list
-template <typename S, int PAR, bool W>
-static unsigned ml_blocks(int nsm) {
-  static int per_sm = 0;  // the same on every GPU of this architecture
-  if (per_sm == 0) {
-    int v = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, mea_list_kernel<S, PAR, W>, 256, 0) != cudaSuccess || v < 1)
-      v = 1;
-    per_sm = v;
-  }
-  return (unsigned)((nsm > 0 ? nsm : 152) * per_sm);
-}
-
-template <typename S, int PAR>
-static cudaError_t launch_ml(const LbmArgs& a, bool walls, int nsm, cudaStream_t s) {
-  if (walls) return launch_k(mea_list_kernel<S, PAR, true>, dim3(ml_blocks<S, PAR, true>(nsm)), dim3(256), 0, s,
-                            a.pdl != 0, a);
-  return launch_k(mea_list_kernel<S, PAR, false>, dim3(ml_blocks<S, PAR, false>(nsm)), dim3(256), 0, s, a.pdl != 0, a);
-}
-
-cudaError_t launch_mea_moments(const LbmArgs& a, int precision, int parity, bool walls, int nsm,
-                               cudaStream_t s) {
-  if (precision == 0) return parity == 0 ? launch_ml<float, 0>(a, walls, nsm, s) : launch_ml<float, 1>(a, walls, nsm, s);
-  return parity == 0 ? launch_ml<__half, 0>(a, walls, nsm, s) : launch_ml<__half, 1>(a, walls, nsm, s);
 }
 
 // logical populations of a range of cells of one box

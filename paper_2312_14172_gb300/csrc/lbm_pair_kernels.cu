@@ -157,7 +157,6 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
     if (COUPLE) {
       couple_row<2, (C > 1)>(srec, s_rowmask[threadIdx.y + a.sub_y * (z - z0)], bd, x0, y, z, a.eps,
                              a.inv_eps, a.status, cc, a.grids);
-      if (single) cc.ip0[1] = cc.ip1[1] = -1;
     }
     // mass and momentum of the arrivals
     float2 drho, jx, jy, jz;
@@ -224,22 +223,6 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
     pair(13, h2, q2, w3r2, sub2(ux, uz), sub2(vx, vz));
     pair(15, h2, q2, w3r2, add2(uy, uz), add2(vy, vz));
     pair(17, h2, q2, w3r2, sub2(uy, uz), sub2(vy, vz));
-    // cells inside a particle record the mass and momentum they send out, as
-    // stored, for the next step's momentum exchange (taken before the stores,
-    // so that the values need not stay in registers through them)
-    float4 mom[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
-    if (COUPLE && a.ilist_idx && (cc.ip0[0] >= 0 || cc.ip0[1] >= 0)) {
-      float2 ms, mx, my, mz;  // of the values as stored
-      moments2<T>(d, ms, mx, my, mz);
-      if (Pop<S>::SCALED) {
-        ms = mul2(ms, f2(isc));
-        mx = mul2(mx, f2(isc));
-        my = mul2(my, f2(isc));
-        mz = mul2(mz, f2(isc));
-      }
-      mom[0] = make_float4(ms.x, mx.x, my.x, mz.x);
-      mom[1] = make_float4(ms.y, mx.y, my.y, mz.y);
-    }
     // store the post-collision deviations (now in d), streamed (AA pattern):
     // slot i of x + c_i, or slot ibar of x when x + c_i lies beyond a wall
 #pragma unroll
@@ -272,8 +255,6 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
         }
       }
     }
-    if (COUPLE && a.ilist_idx && owned_plane(bd, z))
-      append_interior<2>(a, (unsigned)(bd.cell_off + (z * bd.ny + y) * bd.nx + x0), cc, mom);
   };
   // one z slice at a time: an unrolled loop would hold two slices' arrivals
 #pragma unroll 1
