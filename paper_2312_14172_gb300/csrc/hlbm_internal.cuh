@@ -311,6 +311,7 @@ struct PartArgs {
   int nchunks;
   int mea_group;            // planes whose cells are summed together
   int mea_threads;          // threads per momentum-exchange block
+  int move;                 // 1: the exchange moves the particles too (no update kernel)
   double* partial;          // [cap][MAX_PLANES][6] FP64 sums of the groups of planes
   int* done;                // [cap] blocks finished per particle (reset to 0)
   // the moments-mode momentum exchange adds the blocks of a particle here

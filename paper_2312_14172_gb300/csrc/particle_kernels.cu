@@ -77,6 +77,242 @@ __device__ void build_record(const double* P, int cap, int p, int shape, int box
   make_record(X, U, W, q, A, iA, pget(P, cap, PF_RINF, p), eps, p, shape, box, R);
 }
 
+// the bin tiles along one axis touched by cells [lo, hi]: one range
+// [a0, a1], plus a second range [b0, b1] (empty when b1 < b0) where the cell
+// range wraps around a periodic axis
+struct AxisTiles {
+  int a0, a1, b0, b1;
+  __device__ __forceinline__ int count() const { return (a1 - a0 + 1) + max(b1 - b0 + 1, 0); }
+  __device__ __forceinline__ int at(int t) const {
+    const int na = a1 - a0 + 1;
+    return t < na ? a0 + t : b0 + (t - na);
+  }
+};
+
+__device__ AxisTiles axis_tiles(int lo, int hi, int n, int T, bool wall) {
+  AxisTiles r{0, -1, 0, -1};
+  if (wall) {
+    lo = max(lo, 0);
+    hi = min(hi, n - 1);
+    if (lo <= hi) { r.a0 = lo / T; r.a1 = hi / T; }
+    return r;
+  }
+  if (hi - lo + 1 >= n) {  // the whole periodic axis
+    r.a0 = 0; r.a1 = (n - 1) / T;
+    return r;
+  }
+  if (lo < 0) {            // [lo + n, n - 1] and [0, hi]
+    r.a0 = (lo + n) / T; r.a1 = (n - 1) / T;
+    r.b0 = 0; r.b1 = hi / T;
+  } else if (hi >= n) {    // [lo, n - 1] and [0, hi - n]
+    r.a0 = lo / T; r.a1 = (n - 1) / T;
+    r.b0 = 0; r.b1 = (hi - n) / T;
+  } else {
+    r.a0 = lo / T; r.a1 = hi / T;
+  }
+  // both ends in the same tiles (an axis of one or two tiles): merge
+  if (r.b1 >= r.b0 && r.b1 >= r.a0) {
+    r.a0 = 0; r.a1 = max(r.a1, r.b1);
+    r.b0 = 0; r.b1 = -1;
+  }
+  return r;
+}
+
+// Tiles of one particle's bin range, kept in shared memory between the
+// Newton-Euler step and the binning.
+struct BinRange {
+  AxisTiles at[3];
+  long long tile_off;
+  int ntx, nty;
+  int count;  // tiles; 0 when the particle is not binned
+};
+
+// cells [lo, hi] along one axis of the bin range of a particle at X: its
+// influence sphere, widened so that the cells next to the interior (which
+// feed its momentum exchange) see it too, rounded outwards in FP32
+__device__ __forceinline__ AxisTiles bin_axis(double X, float rb, int n, int T, bool wall) {
+  const int lo = (int)floorf(__fsub_rd(__double2float_rd(X), rb)) - 1;
+  const int hi = (int)ceilf(__fadd_ru(__double2float_ru(X), rb)) + 1;
+  return axis_tiles(lo, hi, n, T, wall);
+}
+
+// adds particle p to the lists of the tiles of its bin range: threads sub,
+// sub + step, ... take the tiles in turn
+__device__ __forceinline__ void bin_particle(const PartArgs& a, const BinRange& br, int p, int sub, int step) {
+  const int cx_ = br.at[0].count(), cy_ = br.at[1].count();
+  for (int t = sub; t < br.count; t += step) {
+    const int ix = t % cx_, r = t / cx_, iy = r % cy_, iz = r / cy_;
+    const long long tile = br.tile_off + ((long long)br.at[2].at(iz) * br.nty + br.at[1].at(iy)) * br.ntx +
+                           br.at[0].at(ix);
+    const int slot = atomicAdd(&a.bin_count[tile], 1);
+    if (slot < a.bin_cap) a.bin_ids[tile * a.bin_cap + slot] = p;
+    else atomicOr(a.status, ST_CAPACITY);
+  }
+}
+
+// clears the tile counts the next step will fill
+__device__ __forceinline__ void clear_bins(const PartArgs& a) {
+  const long long nthr = (long long)gridDim.x * blockDim.x;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < a.ntiles; t += nthr) a.bin_count_clear[t] = 0;
+}
+
+// ------------------------------------------- one particle moved by one block
+// The Newton-Euler step of the update kernel (below) for the particle whose
+// momentum exchange this block has just summed, with the vector components
+// and the quaternion's on lanes of their own: an FP64 instruction costs a
+// GB300 SM 16 cycles per warp whether one lane runs it or 32, so a particle
+// takes a third of the instructions that it takes on one lane.  Translation
+// on warp 0, rotation on warp 1.  Every operation is the one of the update
+// kernel, in its order (contractions written out), so that both move a
+// particle to the same bits.
+struct MoveScratch {
+  double P[PF_COUNT];  // the particle's row of the table before the step
+  double F[6];         // force and torque of the momentum exchange
+  double v[7];         // w x y z and the angular velocity of the quaternion step
+  double R[9], wb[3], Lb[3];
+  BinRange br;
+};
+
+__device__ __forceinline__ double sum2(double a, double b, double c, double d) {  // a b + c d
+  return __fma_rn(a, b, __dmul_rn(c, d));
+}
+__device__ __forceinline__ double dif2(double a, double b, double c, double d) {  // a b - c d
+  return __fma_rn(a, b, -__dmul_rn(c, d));
+}
+
+// entry e of the rotation matrix of the quaternion v[0..3] (as rotation_rn):
+// v[a] v[b] +- v[c] v[d], doubled, on the diagonal taken from 1
+__device__ __forceinline__ double rotation_entry(const double* v, int e) {
+  // w x y z = 0 1 2 3; per entry a, b, c, d as digits of base 4
+  const unsigned tab[9] = {0xAF, 0x63, 0x72, 0x63, 0x5F, 0xB1, 0x72, 0xB1, 0x5A};
+  const unsigned t = tab[e];
+  const double p = __dmul_rn(v[(t >> 6) & 3], v[(t >> 4) & 3]), q = __dmul_rn(v[(t >> 2) & 3], v[t & 3]);
+  const bool minus = e == 1 || e == 5 || e == 6;
+  const double s = __dmul_rn(2.0, minus ? __dsub_rn(p, q) : __dadd_rn(p, q));
+  return e % 4 == 0 ? __dsub_rn(1.0, s) : s;
+}
+
+// called by all threads of the block; m.P, m.F are filled (and synchronised);
+// R holds the particle's record before the step
+__device__ __forceinline__ void move_particle(const PartArgs& a, int p, const BoxDesc& bd, Rec& R, MoveScratch& m) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int cap = a.cap;
+  if (warp == 0) {
+    if (lane < 3) {
+      const int j = lane;
+      double Fh = m.F[j];
+      if (a.contact_k > 0.0) Fh += m.P[PF_FC + j];
+      const double F = __fma_rn(__dmul_rn(__dsub_rn(m.P[PF_RHO], 1.0), m.P[PF_V]), a.g[j], Fh);
+      const double U = __fma_rn(F, m.P[PF_IM], m.P[PF_U + j]);
+      double X = __dadd_rn(m.P[PF_X + j], U);
+      if (!(isfinite(X) && isfinite(U))) atomicOr(a.status, ST_UNSTABLE);
+      const int n = j == 0 ? bd.nx : (j == 1 ? bd.ny : bd.nz);
+      const bool wall = (bd.bc >> j) & 1;
+      if (wall) {
+        const bool cut = j == 2 && (bd.bc & BC_CUT_Z);
+        if (!cut && !(X > -0.5 && X < n - 0.5)) atomicOr(a.status, ST_LEFT_DOMAIN);
+      } else {
+        const double L = (double)n;
+        if (X >= L) X -= L;
+        else if (X < 0.0) X += L;
+      }
+      pset(a.P, cap, PF_X + j, p, X);
+      pset(a.P, cap, PF_U + j, p, U);
+      const float xh = __double2float_rn(X);
+      R.xh[j] = xh;
+      R.xl[j] = __double2float_rn(X - (double)xh);
+      R.u[j] = (float)U;
+      const bool binned = X > -1.0e6 && X < 1.0e6;  // flagged above otherwise
+      const float rb = __double2float_ru(fmax(m.P[PF_RINF], __dadd_rn(m.P[PF_RC], 1.5)));
+      m.br.at[j] = binned ? bin_axis(X, rb, n, j == 0 ? TILE_X : (j == 1 ? TILE_Y : TILE_Z), wall) : AxisTiles{0, -1, 0, -1};
+    }
+    __syncwarp();
+    if (lane == 0) {
+      m.br.tile_off = bd.tile_off;
+      m.br.ntx = bd.ntx;
+      m.br.nty = bd.nty;
+      m.br.count = m.br.at[0].count() * m.br.at[1].count() * m.br.at[2].count();
+    }
+  } else if (warp == 1) {
+    const bool sphere = R.shape == 0;
+    const int j = lane < 3 ? lane : 0, j1 = j == 2 ? 0 : j + 1, j2 = j == 0 ? 2 : j - 1;
+    if (lane < 4) m.v[lane] = m.P[PF_Q + lane];
+    __syncwarp();
+    double W = m.P[PF_W + j], Th = m.F[3 + j];
+    if (a.contact_k > 0.0) Th += m.P[PF_TC + j];
+    if (sphere) {
+      W = __fma_rn(Th, m.P[PF_II + j], W);
+      if (lane < 3) m.v[4 + lane] = W;
+    } else {
+      if (lane < 9) m.R[lane] = rotation_entry(m.v, lane);
+      if (lane < 3) {
+        m.wb[lane] = W;
+        m.Lb[lane] = Th;
+      }
+      __syncwarp();
+      // into the body frame
+      double wb = __fma_rn(m.R[6 + j], m.wb[2], sum2(m.R[j], m.wb[0], m.R[3 + j], m.wb[1]));
+      const double Tb = __fma_rn(m.R[6 + j], m.Lb[2], sum2(m.R[j], m.Lb[0], m.R[3 + j], m.Lb[1]));
+      __syncwarp();
+      if (lane < 3) {
+        m.wb[lane] = wb;
+        m.Lb[lane] = __dmul_rn(m.P[PF_I + j], wb);
+      }
+      __syncwarp();
+      const double gy = dif2(m.wb[j1], m.Lb[j2], m.wb[j2], m.Lb[j1]);
+      wb = __fma_rn(__dsub_rn(Tb, gy), m.P[PF_II + j], wb);
+      if (lane < 3) m.v[4 + lane] = wb;
+      __syncwarp();
+      W = __fma_rn(m.R[3 * j + 2], m.v[6], sum2(m.R[3 * j], m.v[4], m.R[3 * j + 1], m.v[5]));
+    }
+    __syncwarp();
+    // q += q (x) (0, omega_b) / 2, for a sphere in the equal form (0, omega)
+    // (x) q / 2: per component s (v[a] v[b] + v[c] v[d] -+ v[e] v[f])
+    double q = 0.0, nq;
+    if (lane < 4) {
+      const double* v = m.v;
+      const int l = lane;
+      double t;
+      if (l == 0) {
+        t = sphere ? -__fma_rn(v[6], v[3], sum2(v[4], v[1], v[5], v[2]))
+                   : __fma_rn(-v[3], v[6], dif2(-v[1], v[4], v[2], v[5]));
+      } else if (sphere) {
+        // w W_l-1 + W_l y_l+1 - W_l+1 y_l, y = x y z
+        const int b = l - 1, c = l % 3, d = (l + 1) % 3;
+        t = __fma_rn(-v[4 + d], v[1 + c], sum2(v[0], v[4 + b], v[4 + c], v[1 + d]));
+      } else {
+        const int b = l - 1, c = l % 3, d = (l + 1) % 3;
+        t = __fma_rn(-v[1 + d], v[4 + c], sum2(v[0], v[4 + b], v[1 + c], v[4 + d]));
+      }
+      q = __fma_rn(0.5, t, v[l]);
+    }
+    {
+      const double q0 = __shfl_sync(0xffffffffu, q, 0), q1 = __shfl_sync(0xffffffffu, q, 1);
+      const double q2 = __shfl_sync(0xffffffffu, q, 2), q3 = __shfl_sync(0xffffffffu, q, 3);
+      nq = __fma_rn(q3, q3, __fma_rn(q2, q2, sum2(q0, q0, q1, q1)));
+    }
+    q = __dmul_rn(q, rsqrt(nq));
+    __syncwarp();
+    if (lane < 4) {
+      m.v[lane] = q;
+      pset(a.P, cap, PF_Q + lane, p, q);
+    }
+    if (lane < 3) {
+      if (!isfinite(W)) atomicOr(a.status, ST_UNSTABLE);
+      pset(a.P, cap, PF_W + lane, p, W);
+      R.w[lane] = (float)W;
+    }
+    __syncwarp();
+    if (!sphere && lane < 9) R.M[lane] = __double2float_rn(rotation_entry(m.v, lane));
+  } else if (warp == 2 && lane < 6) {
+    pset(a.P, cap, (lane < 3 ? PF_F : PF_T - 3) + lane, p, m.F[lane]);
+  }
+  __syncthreads();
+  if (threadIdx.x < 32)
+    reinterpret_cast<int*>(&a.rec[p])[threadIdx.x] = reinterpret_cast<const int*>(&R)[threadIdx.x];
+  bin_particle(a, m.br, p, threadIdx.x, blockDim.x);
+}
+
 // Momentum exchange of every particle from the populations alone: block
 // `chunk` walks p_planes planes of the bounding box of particle
 // chunk_p[chunk] from plane chunk_q[chunk] on, in groups of mea_group planes.
@@ -100,9 +336,14 @@ __global__ void __launch_bounds__(XCH_MAX_T, 2) mea_kernel(PartArgs a) {
   __shared__ ExchangeBox box;
   __shared__ float wsum[MAX_PLANES][4][6];
   __shared__ double gsum[MAX_PLANES][6];
+  __shared__ MoveScratch mv;
   __shared__ int s_last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid < 32) reinterpret_cast<int*>(&R)[tid] = reinterpret_cast<const int*>(&a.rec[p])[tid];
+  if (a.move) {
+    clear_bins(a);
+    if (tid >= 64 && tid < 64 + PF_COUNT) mv.P[tid - 64] = pget(a.P, a.cap, tid - 64, p);
+  }
   exchange_box(a, p, bd, q0, planes, box);
   const int G = a.mea_group;
   const int here = max(min(planes, box.ext[2] - q0), 0);  // planes that hold cells
@@ -143,8 +384,12 @@ __global__ void __launch_bounds__(XCH_MAX_T, 2) mea_kernel(PartArgs a) {
   if (tid < 6) {
     double t = 0.0;
     for (int g = 0; g < total; ++g) t += gsum[g][tid];
-    pset(a.P, a.cap, (tid < 3 ? PF_F : PF_T - 3) + tid, p, t);
+    if (a.move) mv.F[tid] = t;
+    else pset(a.P, a.cap, (tid < 3 ? PF_F : PF_T - 3) + tid, p, t);
   }
+  if (!a.move) return;
+  __syncthreads();
+  move_particle(a, p, bd, R, mv);
 }
 
 // Momentum exchange of every particle in the moments form (after a collision
@@ -167,9 +412,14 @@ __global__ void __launch_bounds__(XCH_MAX_T, 2) mea_moments_kernel(PartArgs a) {
   __shared__ Rec R;
   __shared__ ExchangeRows rows;
   __shared__ long long wsum[XCH_MAX_T / 32][6];
+  __shared__ MoveScratch mv;
   __shared__ int s_last;
   const int tid = threadIdx.x, lane = tid & 31;
   if (tid < 32) reinterpret_cast<int*>(&R)[tid] = reinterpret_cast<const int*>(&a.rec[p])[tid];
+  if (a.move) {
+    clear_bins(a);
+    if (tid >= 64 && tid < 64 + PF_COUNT) mv.P[tid - 64] = pget(a.P, a.cap, tid - 64, p);
+  }
   __syncthreads();
   long long s[6] = {0, 0, 0, 0, 0, 0};
   const S* f = reinterpret_cast<const S*>(a.f);
@@ -216,9 +466,14 @@ __global__ void __launch_bounds__(XCH_MAX_T, 2) mea_moments_kernel(PartArgs a) {
     }
     if (tid == 0) a.done[p] = 0;
   }
-  if (tid < 6)
-    pset(a.P, a.cap, (tid < 3 ? PF_F : PF_T - 3) + tid, p,
-         (double)sum * (1.0 / (double)(1LL << ACC_FRAC_BITS)));
+  if (tid < 6) {
+    const double t = (double)sum * (1.0 / (double)(1LL << ACC_FRAC_BITS));
+    if (a.move) mv.F[tid] = t;
+    else pset(a.P, a.cap, (tid < 3 ? PF_F : PF_T - 3) + tid, p, t);
+  }
+  if (!a.move) return;
+  __syncthreads();
+  move_particle(a, p, bd, R, mv);
 }
 
 // interior cells of every particle, added to *count
@@ -237,47 +492,6 @@ __global__ void __launch_bounds__(XCH_MAX_T) count_interior_kernel(PartArgs a, u
   if ((threadIdx.x & 31) == 0 && n) atomicAdd(count, (unsigned long long)n);
 }
 
-// the bin tiles along one axis touched by cells [lo, hi]: one range
-// [a0, a1], plus a second range [b0, b1] (empty when b1 < b0) where the cell
-// range wraps around a periodic axis
-struct AxisTiles {
-  int a0, a1, b0, b1;
-  __device__ __forceinline__ int count() const { return (a1 - a0 + 1) + max(b1 - b0 + 1, 0); }
-  __device__ __forceinline__ int at(int t) const {
-    const int na = a1 - a0 + 1;
-    return t < na ? a0 + t : b0 + (t - na);
-  }
-};
-
-__device__ AxisTiles axis_tiles(int lo, int hi, int n, int T, bool wall) {
-  AxisTiles r{0, -1, 0, -1};
-  if (wall) {
-    lo = max(lo, 0);
-    hi = min(hi, n - 1);
-    if (lo <= hi) { r.a0 = lo / T; r.a1 = hi / T; }
-    return r;
-  }
-  if (hi - lo + 1 >= n) {  // the whole periodic axis
-    r.a0 = 0; r.a1 = (n - 1) / T;
-    return r;
-  }
-  if (lo < 0) {            // [lo + n, n - 1] and [0, hi]
-    r.a0 = (lo + n) / T; r.a1 = (n - 1) / T;
-    r.b0 = 0; r.b1 = hi / T;
-  } else if (hi >= n) {    // [lo, n - 1] and [0, hi - n]
-    r.a0 = lo / T; r.a1 = (n - 1) / T;
-    r.b0 = 0; r.b1 = (hi - n) / T;
-  } else {
-    r.a0 = lo / T; r.a1 = hi / T;
-  }
-  // both ends in the same tiles (an axis of one or two tiles): merge
-  if (r.b1 >= r.b0 && r.b1 >= r.a0) {
-    r.a0 = 0; r.a1 = max(r.a1, r.b1);
-    r.b0 = 0; r.b1 = -1;
-  }
-  return r;
-}
-
 __device__ __forceinline__ void cross3(const double a[3], const double b[3], double o[3]) {
   o[0] = a[1] * b[2] - a[2] * b[1];
   o[1] = a[2] * b[0] - a[0] * b[2];
@@ -294,15 +508,6 @@ __device__ __forceinline__ void cross3(const double a[3], const double b[3], dou
 // few lanes are active, so the translation and the rotation of a block's
 // particles run on two warps (two SM sub-partitions) at once, each lane one
 // particle, and meet in shared memory for the record and the binning.
-
-// Tiles of one particle's bin range, kept in shared memory between the
-// Newton-Euler step and the binning.
-struct BinRange {
-  AxisTiles at[3];
-  long long tile_off;
-  int ntx, nty;
-  int count;  // tiles; 0 when the particle is not binned
-};
 
 // force of the momentum exchange (row base PF_F) or torque (PF_T) of particle
 // p, as the exchange left it in the table, with the contact force or torque
@@ -356,9 +561,6 @@ __device__ __forceinline__ void translate_particle(const PartArgs& a, int p, Rec
     R.xl[j] = __double2float_rn(X[j] - (double)xh);
     R.u[j] = (float)U[j];
   }
-  // bin tiles touched by the influence sphere, widened so that the cells next
-  // to the particle's interior (which feed its momentum exchange) see it too;
-  // the cell range is rounded outwards in FP32
   br.tile_off = bd.tile_off;
   br.ntx = bd.ntx;
   br.nty = bd.nty;
@@ -367,9 +569,7 @@ __device__ __forceinline__ void translate_particle(const PartArgs& a, int p, Rec
   const int T[3] = {TILE_X, TILE_Y, TILE_Z};
   for (int j = 0; j < 3; ++j) {
     if (!(X[j] > -1.0e6 && X[j] < 1.0e6)) return;  // flagged above; not binned
-    const int lo = (int)floorf(__fsub_rd(__double2float_rd(X[j]), rb)) - 1;
-    const int hi = (int)ceilf(__fadd_ru(__double2float_ru(X[j]), rb)) + 1;
-    br.at[j] = axis_tiles(lo, hi, n[j], T[j], (bd.bc >> j) & 1);
+    br.at[j] = bin_axis(X[j], rb, n[j], T[j], (bd.bc >> j) & 1);
   }
   br.count = br.at[0].count() * br.at[1].count() * br.at[2].count();
 }
@@ -459,9 +659,7 @@ __global__ void __launch_bounds__(UPD_T) update_kernel(PartArgs a) {
   __shared__ Rec s_rec[UPD_P];
   pdl_trigger();
   pdl_wait();
-  const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long nthr = (long long)gridDim.x * blockDim.x;
-  for (long long t = tid; t < a.ntiles; t += nthr) a.bin_count_clear[t] = 0;
+  clear_bins(a);
   const int ppb = a.ppb;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (long long base = blockIdx.x * (long long)ppb; base < a.np; base += (long long)gridDim.x * ppb) {
@@ -479,17 +677,7 @@ __global__ void __launch_bounds__(UPD_T) update_kernel(PartArgs a) {
     for (int e = threadIdx.x; e < nrec * 32; e += UPD_T)
       reinterpret_cast<int*>(&a.rec[base + (e >> 5)])[e & 31] = reinterpret_cast<const int*>(&s_rec[e >> 5])[e & 31];
     const int k = threadIdx.x % ppb, sub = threadIdx.x / ppb;
-    const BinRange& br = s_br[k];
-    const int cx_ = br.at[0].count(), cy_ = br.at[1].count();
-    const int p = (int)(base + k);
-    for (int t = sub; t < br.count; t += UPD_T / ppb) {
-      const int ix = t % cx_, r = t / cx_, iy = r % cy_, iz = r / cy_;
-      const long long tile = br.tile_off + ((long long)br.at[2].at(iz) * br.nty + br.at[1].at(iy)) * br.ntx +
-                             br.at[0].at(ix);
-      const int slot = atomicAdd(&a.bin_count[tile], 1);
-      if (slot < a.bin_cap) a.bin_ids[tile * a.bin_cap + slot] = p;
-      else atomicOr(a.status, ST_CAPACITY);
-    }
+    bin_particle(a, s_br[k], (int)(base + k), sub, UPD_T / ppb);
     __syncthreads();
   }
 }
