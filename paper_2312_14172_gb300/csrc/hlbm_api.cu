@@ -144,6 +144,7 @@ struct hlbm_ctx {
   // within twice the L2 (a step then starts on what the last one ended
   // with, still in L2); larger lattices gain nothing and keep one order
   bool reverse_odd = false;
+  int prefetch = 0;  // rows a collision block prefetches at most
   std::vector<int> h_planes;    // bounding-box planes per particle
   int mea_group = 1;            // planes whose cells are summed together
   bool fused = false;           // the momentum exchange moves the particles too
@@ -227,6 +228,7 @@ static LbmArgs lbm_args(const hlbm_ctx* h, int parity) {
   a.nsub = (TILE_Y / h->sub_y) * (TILE_Z / h->sub_z);
   a.nbricks = h->L.ntiles * a.nsub;
   a.reverse = parity && h->reverse_odd;
+  a.prefetch = std::min(h->prefetch, h->sub_y * h->sub_z);
   a.omega = (float)(1.0 / h->prm.tau);
   for (int j = 0; j < 3; ++j) a.ff[j] = (float)h->prm.fluid_force[j];
   a.eps = (float)h->prm.eps;
@@ -455,7 +457,15 @@ int hlbm_init_batch(hlbm_handle* out, int nboxes, const hlbm_box* boxes, const h
     int l2 = 0;
     if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) l2 = 0;
     const size_t s = h->prm.precision == HLBM_FP16 ? 2 : 4;
-    h->reverse_odd = l2 > 0 && (size_t)QVB * h->L.nblocks * s <= 2 * (size_t)l2;
+    const size_t pops = (size_t)QVB * h->L.nblocks * s;
+    h->reverse_odd = l2 > 0 && pops <= 2 * (size_t)l2;
+    // larger populations stream through L2: a collision block asks for its
+    // brick's rows (up to 32) before it waits and stages its candidates, so
+    // that its loads find them there.  Collision in us, without and with:
+    // dense 512x512x1024 FP16 4545 / 4280, non-spherical 256^3 FP32 457 / 422,
+    // 64 boxes FP32 922 / 842.  Within twice the L2 it gives nothing (128^3
+    // FP32 55.1 / 55.8 us) or costs (duct 101x67x83 15.3 / 15.9 us a step).
+    h->prefetch = h->reverse_odd ? 0 : 32;
   }
   for (int k = 0; k < 2; ++k) {
     h->cnt[k] = (int*)(h->buf + h->L.off_cnt[k]);

@@ -269,6 +269,13 @@ __device__ __forceinline__ float capsule_row_dist2(const Capsule& c, float ry, f
   return qy * qy + qz * qz;
 }
 
+// asks L2 for the storage block at element b * QVB of f (its 19 slots are one
+// contiguous run of a multiple of 16 bytes)
+template <typename S>
+__device__ __forceinline__ void prefetch_block(const S* f, long long b) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(f + b * QVB), "n"(QVB * (int)sizeof(S)) : "memory");
+}
+
 // Stage the particle candidates of the brick's tile in shared memory and
 // mark, for each row (local y + sub_y * local z) of the brick, the
 // candidates whose influence sphere meets the row.  Called by every thread
