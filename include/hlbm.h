@@ -245,7 +245,8 @@ long long hlbm_steps_done(hlbm_handle h);
 /* Launch shape of the collision kernel: each thread block covers a brick of
  * 32 x tile_y x tile_z cells, tile_y and tile_z in {1, 2, 4, 8}, with
  * cells_x = 1 or 2 x-adjacent cells per thread (32 x tile_y or 16 x tile_y
- * threads); cells_x = 2 is the default.  Both compute the same step; their
+ * threads); cells_x = 2 is the default, with tile_y = 4 and a tile_z that
+ * follows the lattice's size until this call or hlbm_autotune.  Both compute the same step; their
  * results differ by FP32 rounding order only. */
 int hlbm_set_launch(hlbm_handle h, int tile_y, int tile_z, int cells_x);
 int hlbm_get_launch(hlbm_handle h, int* tile_y, int* tile_z, int* cells_x);
@@ -266,8 +267,9 @@ int hlbm_get_launch(hlbm_handle h, int* tile_y, int* tile_z, int* cells_x);
 int hlbm_set_mea_mode(hlbm_handle h, int mode);
 int hlbm_get_mea_mode(hlbm_handle h);
 
-/* Times every momentum-exchange mode and launch shape (tile_y, tile_z,
- * cells_x; cells_x = 2 only with tile_y >= 2) on about 20 ms of steps
+/* Sets the moments form of the momentum exchange where there are particles
+ * (the faster mode at every size) and times every launch shape (tile_y,
+ * tile_z, cells_x; cells_x = 2 only with tile_y >= 2) on about 20 ms of steps
  * (nsteps to 4 nsteps) from the current state, times the three fastest once
  * more and keeps the fastest; writes the chosen shape and its time per step
  * in ms (any pointer may be NULL).  The run is left where it was: the

@@ -165,7 +165,8 @@ struct hlbm_ctx {
   double contact_k = 0.0, contact_zeta = 1.0;
   int np = 0;
   long long steps = 0;
-  int sub_y = 4, sub_z = 2;
+  int sub_y = 4, sub_z = 2;  // bricks of the collision (default_launch, until hlbm_set_launch)
+  bool launch_set = false;
   int cells_x = 1;       // cells per thread along x
   bool pair_ok = false;  // the two-cell kernel may run
   // [0][parity]: step with the momentum-exchange kernel (after any change of
@@ -348,6 +349,29 @@ static int build_graphs(hlbm_ctx* h) {
   return HLBM_OK;
 }
 
+// The bricks of the collision until the caller or the autotuner sets them:
+// 32 x 4 x 2 cells, or taller ones as long as they leave two and a half
+// resident waves of blocks (8 blocks of 64 threads per SM in FP32, 10 in
+// FP16).  A taller brick stages its candidates for more cells: 32x4x4 against
+// 32x4x2, collision in us: 128^3 FP16 45.3 / 47.8, non-spherical 256^3 FP32
+// 422 / 470; FP16, with its lighter slices, gains up to 32x4x8 (non-spherical
+// 256^3 387 / 398 / 445, dense 512x512x1024 4280 / 4549 / 5237), FP32 does not
+// (470 / 422).  Small lattices want the blocks (duct 101x67x83 18.1 / 15.3 us
+// a step), and so do distance grids, whose cells cost unevenly (128^3 FP16
+// 91 / 85).
+static void default_launch(hlbm_ctx* h) {
+  if (h->launch_set) return;
+  const bool half = h->prm.precision == HLBM_FP16;
+  const long long resident = (long long)(h->nsm > 0 ? h->nsm : 152) * (half ? 10 : 8);
+  h->sub_z = 2;
+  if (!h->grids.empty()) return;
+  for (int z = half ? 8 : 4; z > 2; z /= 2)
+    if (2 * h->L.ntiles * (TILE_Y / h->sub_y) * (TILE_Z / z) >= 5 * resident) {
+      h->sub_z = z;
+      break;
+    }
+}
+
 // the status word already copied to the host: HLBM_OK, or clears the device
 // flags and returns the error they name
 static int status_code(hlbm_ctx* h, int st) {
@@ -466,6 +490,7 @@ int hlbm_init_batch(hlbm_handle* out, int nboxes, const hlbm_box* boxes, const h
     // 64 boxes FP32 922 / 842.  Within twice the L2 it gives nothing (128^3
     // FP32 55.1 / 55.8 us) or costs (duct 101x67x83 15.3 / 15.9 us a step).
     h->prefetch = h->reverse_odd ? 0 : 32;
+    default_launch(h);
   }
   for (int k = 0; k < 2; ++k) {
     h->cnt[k] = (int*)(h->buf + h->L.off_cnt[k]);
@@ -762,6 +787,7 @@ int hlbm_add_grid(hlbm_handle h, int nx, int ny, int nz, double spacing, const f
   CK(cudaStreamSynchronize(h->stream));
   h->grid_used += nv;
   h->grids.push_back(std::move(g));
+  default_launch(h);
   drop_graphs(h);  // the captured steps name the grids by pointer (set once grids exist)
   *grid_id = id;
   return HLBM_OK;
@@ -907,7 +933,7 @@ int hlbm_add_particles(hlbm_handle h, int n, const int* box_id, const int* shape
     sh[k] = s;
     bx[k] = b;
     nch[k] = (int)std::ceil(2.0 * rc) + 2;  // bounding-box planes, at most MAX_PLANES
-    cells[k] = 4.0 / 3.0 * PI_D * std::pow(std::cbrt(V * 3.0 / (4.0 * PI_D)) + 0.5, 3.0);
+    cells[k] = 1.3 * V;  // about the cells its momentum exchange walks
   }
   const int p0 = h->np;
   int rc = upload_fields(h, p0, n, tab);
@@ -1219,6 +1245,7 @@ int hlbm_set_launch(hlbm_handle h, int tile_y, int tile_z, int cells_x) {
   if (!ok(tile_y) || !ok(tile_z)) return fail(h, HLBM_ERR_ARG, "tile_y and tile_z must be 1, 2, 4 or 8");
   if (cells_x != 1 && cells_x != 2) return fail(h, HLBM_ERR_ARG, "cells_x must be 1 or 2");
   if (cells_x == 2 && !h->pair_ok) return fail(h, HLBM_ERR_ARG, "cells_x = 2 is not available");
+  h->launch_set = true;
   if (tile_y != h->sub_y || tile_z != h->sub_z || cells_x != h->cells_x) {
     h->sub_y = tile_y;
     h->sub_z = tile_z;
@@ -1359,10 +1386,13 @@ int hlbm_autotune(hlbm_handle h, int nsteps, int* tile_y, int* tile_z, int* cell
   struct Cand { int ty, tz, cx, mode; float ms; };
   std::vector<Cand> cand;
   const int vals[4] = {1, 2, 4, 8};
-  const int nmodes = h->np > 0 ? 2 : 1;
+  // the moments form of the exchange walks the same cells as the link sums
+  // without their fixed order: it is the faster mode at every size (us: one
+  // sphere 9.7 / 11.7, 200 spheres FP16 21.5 / 31.5, 50 000 958 / 1484)
+  const int mode = h->np > 0 ? HLBM_MEA_MOMENTS : HLBM_MEA_KERNEL;
   const int nkinds = h->pair_ok ? 2 : 1;
-  for (int im = 0; im < nkinds * nmodes * 16; ++im) {
-    const int kind = im / (nmodes * 16), mode = (im / 16) % nmodes, iy = (im / 4) % 4, iz = im % 4;
+  for (int im = 0; im < nkinds * 16; ++im) {
+    const int kind = im / 16, iy = (im / 4) % 4, iz = im % 4;
     if (kind == 1 && vals[iy] == 1) continue;  // 16-thread blocks leave half of each warp idle
     cand.push_back({vals[iy], vals[iz], kind + 1, mode, 0.f});
   }

@@ -350,8 +350,8 @@ class Lattice:
         return {HLBM_MEA_KERNEL: "kernel", HLBM_MEA_MOMENTS: "moments"}[load().hlbm_get_mea_mode(self.h)]
 
     def autotune(self, nsteps=10):
-        """Times every launch shape and momentum-exchange mode, keeps the
-        fastest; returns (tile_y, tile_z, cells_x, ms per step)."""
+        """Sets the moments form of the exchange, times every launch shape and
+        keeps the fastest; returns (tile_y, tile_z, cells_x, ms per step)."""
         ty, tz, cx, ms = ctypes.c_int(), ctypes.c_int(), ctypes.c_int(), ctypes.c_float()
         _check(self.h, load().hlbm_autotune(self.h, int(nsteps), ctypes.byref(ty), ctypes.byref(tz),
                                             ctypes.byref(cx), ctypes.byref(ms)))
