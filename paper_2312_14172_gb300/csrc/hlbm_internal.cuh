@@ -416,12 +416,12 @@ cudaError_t launch_update(const PartArgs& a, cudaStream_t s);
 // a.contact_k > 0)
 cudaError_t launch_contact(const PartArgs& a, cudaStream_t s);
 cudaError_t launch_records(const PartArgs& a, cudaStream_t s);
-// logical populations f_i - w_i of cells [c0, c0 + n) of one box, as float,
+// logical populations f_i of cells [c0, c0 + n) of one box in FP64,
 // into/out of stage[i * n + k]
 cudaError_t launch_gather(const LbmArgs& a, int precision, int parity, int box, long long c0,
-                          long long n, float* stage, cudaStream_t s);
+                          long long n, double* stage, cudaStream_t s);
 cudaError_t launch_scatter(const LbmArgs& a, int precision, int parity, int box, long long c0,
-                           long long n, const float* stage, cudaStream_t s);
+                           long long n, const double* stage, cudaStream_t s);
 // the five stored slots with c_z = dir of the cells of plane z of one box
 // (ncell = nx ny of the box), to (put = 0) or from (put = 1) stage
 cudaError_t launch_plane_slots(const LbmArgs& a, int precision, int box, int z, int dir, int ncell, void* stage,

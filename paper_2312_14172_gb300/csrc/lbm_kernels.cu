@@ -186,9 +186,12 @@ cudaError_t launch_collide(const LbmArgs& a, int precision, int parity, bool wal
                         : launch_cs_prec<__half>(a, parity, walls, couple, s);
 }
 
-// logical populations of a range of cells of one box
+// logical populations f_i in FP64 of a range of cells of one box: the weight
+// is added to (taken off) the stored deviation here, so that the host's FP64
+// arrays are copied as they are (on the host the two conversions and the
+// staging copies of 0.55 million cells took 11 ms)
 template <typename S, int PAR, bool GATHER>
-__global__ void gather_scatter_kernel(LbmArgs a, int box, long long c0, long long n, float* stage) {
+__global__ void gather_scatter_kernel(LbmArgs a, int box, long long c0, long long n, double* stage) {
   const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (k >= n) return;
   const BoxDesc bd = a.boxes[box];
@@ -209,8 +212,8 @@ __global__ void gather_scatter_kernel(LbmArgs a, int box, long long c0, long lon
       const long long src = nb.at(-cx(i), -cy(i), -cz(i));
       slot = (src >= 0) ? f + src + opp(i) * VB : f + e + i * VB;
     }
-    if (GATHER) stage[i * n + k] = Pop<S>::ld(slot, a.inv_scale);
-    else Pop<S>::st(slot, stage[i * n + k], a.scale);
+    if (GATHER) stage[i * n + k] = wq(i) + (double)Pop<S>::ld(slot, a.inv_scale);
+    else Pop<S>::st(slot, (float)(stage[i * n + k] - wq(i)), a.scale);
   }
 }
 
@@ -303,7 +306,7 @@ cudaError_t launch_plane_slots(const LbmArgs& a, int precision, int box, int z, 
 
 template <typename S, bool G>
 static cudaError_t launch_gs(const LbmArgs& a, int parity, int box, long long c0, long long n,
-                             float* stage, cudaStream_t s) {
+                             double* stage, cudaStream_t s) {
   const unsigned blocks = (unsigned)((n + 255) / 256);
   if (parity == 0) gather_scatter_kernel<S, 0, G><<<blocks, 256, 0, s>>>(a, box, c0, n, stage);
   else gather_scatter_kernel<S, 1, G><<<blocks, 256, 0, s>>>(a, box, c0, n, stage);
@@ -311,16 +314,16 @@ static cudaError_t launch_gs(const LbmArgs& a, int parity, int box, long long c0
 }
 
 cudaError_t launch_gather(const LbmArgs& a, int precision, int parity, int box, long long c0,
-                          long long n, float* stage, cudaStream_t s) {
+                          long long n, double* stage, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   return precision == 0 ? launch_gs<float, true>(a, parity, box, c0, n, stage, s)
                         : launch_gs<__half, true>(a, parity, box, c0, n, stage, s);
 }
 
 cudaError_t launch_scatter(const LbmArgs& a, int precision, int parity, int box, long long c0,
-                           long long n, const float* stage, cudaStream_t s) {
+                           long long n, const double* stage, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  float* st = const_cast<float*>(stage);
+  double* st = const_cast<double*>(stage);
   return precision == 0 ? launch_gs<float, false>(a, parity, box, c0, n, st, s)
                         : launch_gs<__half, false>(a, parity, box, c0, n, st, s);
 }

@@ -256,7 +256,7 @@ class Lattice:
 
     def populations(self, box=0):
         nx, ny, nz = self.boxes[box][:3]
-        f = np.zeros((19, nz, ny, nx))
+        f = np.empty((19, nz, ny, nx))
         _check(self.h, load().hlbm_get_populations(self.h, int(box), f.ctypes.data_as(_dp)))
         return f
 
