@@ -172,6 +172,7 @@ struct hlbm_ctx {
   bool launch_set = false;
   int cells_x = 1;       // cells per thread along x
   bool pair_ok = false;  // the two-cell kernel may run
+  bool wide_slices = false;  // a z slice of some box takes 4 GB or more
   // [0][parity]: step with the momentum-exchange kernel (after any change of
   // state); [1][parity]: step that takes the sums the previous collision made
   cudaGraphExec_t exec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
@@ -220,6 +221,13 @@ static int fail(hlbm_ctx* h, int code, const std::string& msg) {
   return code;
 }
 
+// cells per thread as launched: with half storage or walls the two-cell
+// kernel addresses a z slice with 32-bit offsets, and lattices of larger
+// slices run the one-cell kernel
+static int run_cells_x(const hlbm_ctx* h) {
+  return h->wide_slices && (h->walls || h->prm.precision == HLBM_FP16) ? 1 : h->cells_x;
+}
+
 static LbmArgs lbm_args(const hlbm_ctx* h, int parity) {
   LbmArgs a{};
   a.nsm = h->nsm;
@@ -228,7 +236,7 @@ static LbmArgs lbm_args(const hlbm_ctx* h, int parity) {
   a.nboxes = (int)h->boxes.size();
   a.sub_y = h->sub_y;
   a.sub_z = h->sub_z;
-  a.cells_x = h->cells_x;
+  a.cells_x = run_cells_x(h);
   a.nsub = (TILE_Y / h->sub_y) * (TILE_Z / h->sub_z);
   a.nbricks = h->L.ntiles * a.nsub;
   a.reverse = parity && h->reverse_odd;
@@ -268,7 +276,7 @@ static PartArgs part_args(const hlbm_ctx* h, int parity, bool moments = false) {
   a.nchunks = h->nchunks[moments];
   a.mea_threads = h->mea_threads[moments];
   a.mea_group = h->mea_group;
-  a.cells_x = h->cells_x;
+  a.cells_x = run_cells_x(h);
   a.partial = h->partial;
   a.done = h->done;
   a.acc = h->acc;
@@ -430,7 +438,11 @@ int hlbm_init_batch(hlbm_handle* out, int nboxes, const hlbm_box* boxes, const h
   if (h->prm.bin_capacity == 0) h->prm.bin_capacity = DEFAULT_BIN_CAP;
   h->stream = (cudaStream_t)cuda_stream;
   h->pair_ok = true;  // any nx: an odd nx leaves one cell in a row's last pair
-  for (int b = 0; b < nboxes; ++b) h->walls |= boxes[b].bc_flags != 0;
+  for (int b = 0; b < nboxes; ++b) {
+    h->walls |= boxes[b].bc_flags != 0;
+    const BoxDesc& d = h->boxes[b];
+    h->wide_slices |= (unsigned long long)d.ny * d.ntx * QVB * (prm->precision == HLBM_FP32 ? 4 : 2) > 0xffffffffULL;
+  }
   h->cells_x = 2;
   cudaError_t e;
   if (device_buf) {

@@ -63,6 +63,13 @@ template <> struct Two<__half> {
   }
 };
 
+// v, which all lanes of the warp hold alike, as a value the compiler may keep
+// once per warp (uniform registers)
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(__activemask(), v, 0); }
+__device__ __forceinline__ long long uniform(long long v) {
+  return (long long)(((unsigned long long)(unsigned)uniform((int)(v >> 32)) << 32) | (unsigned)uniform((int)v));
+}
+
 // mass and momentum of the two cells' values v_i (opposite directions taken
 // together: s = v_i + v_ibar, m = v_i - v_ibar)
 template <typename T>
@@ -94,6 +101,14 @@ struct PairBlocks { static constexpr int value = sizeof(S) == 4 ? HLBM_CP_MINBLO
 template <typename S, int PAR, bool WALLS, int C>
 __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel(LbmArgs a) {
   constexpr bool COUPLE = C > 0;
+  // Odd steps address the neighbour rows by 32-bit offsets (below): a tenth
+  // fewer instructions, and the collision is bound by them with half storage
+  // (odd step, us: dense 512x512x1024 FP16 5105 -> 4546, non-spherical 256^3
+  // FP16 432 -> 388) and where walls add to them (128^3 FP32 61.5 -> 57.1).
+  // FP32 without walls waits for HBM instead, and there the pointer form's
+  // slower stream of requests is the faster one (non-spherical 256^3 FP32 452
+  // against 465); an even step touches its own cells only.
+  constexpr bool FAST = PAR == 1 && (sizeof(S) == 2 || WALLS);
   using T = Two<S>;
   __shared__ Rec srec[COUPLE ? MAX_CAND : 1];
   __shared__ unsigned long long s_rowmask[COUPLE ? TILE_Y * TILE_Z : 1];
@@ -111,6 +126,10 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
   pdl_wait();
   if (COUPLE) load_candidates(a, k, srec, s_rowmask);
 
+  const int z0 = uniform(k.z0), nz = uniform(bd.nz);
+  const int z1 = min(z0 + a.sub_z, nz);
+  const long long slice_bytes = uniform((long long)bd.ny * bd.ntx * (QVB * (int)sizeof(S)));
+  char* const base = reinterpret_cast<char*>(a.f) + uniform(bd.blk_off * (long long)(QVB * sizeof(S)));
   const int x0 = k.x0 + 2 * threadIdx.x;
   const int y = k.y0 + threadIdx.y;
   if (x0 >= bd.nx || y >= bd.ny) return;
@@ -118,26 +137,44 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
   // row's padding, computed but never stored, and the cell's right
   // neighbour is x0 + 1 wrapped (rb.dr, rb.wr refer to x0 + 1 there)
   const bool single = x0 + 1 == bd.nx;
-  const int z0 = k.z0;
-  const int z1 = min(z0 + a.sub_z, bd.nz);
   const RowBlocks rb = row_blocks<WALLS>(bd, x0, y, single ? 1 : 2);
   S* const f = reinterpret_cast<S*>(a.f);
   const float sc = Pop<S>::SCALED ? a.scale : 1.0f, isc = Pop<S>::SCALED ? a.inv_scale : 1.0f;
 
-  // Walls need selects in every direction, but only the slices and rows next
-  // to a wall and the lanes at an x wall meet one; everything else runs the
-  // slice without them.
-  const bool row_free = !WALLS || (!((bd.bc & 2) && (y == 0 || y == bd.ny - 1)) && !rb.wl && !rb.wr);
-  auto slice = [&](auto wtag, int z) {
-    constexpr bool W = decltype(wtag)::value;
+  // Walls need selects in every direction, and so does a row's single last
+  // cell, but few warps hold such cells: they run the slice with the selects,
+  // all others without (a warp runs one of the two).
+  const bool special = single || (WALLS && (((bd.bc & 2) && (y == 0 || y == bd.ny - 1)) || rb.wl || rb.wr));
+  const bool plain_row = FAST && !__any_sync(__activemask(), special);
+  // Byte offsets within a z slice (below 4 GB, the caller sees to it) of slot 0
+  // of x0 in the rows y - 1, y, y + 1, and from there to x0 - 1 and x0 + 2:
+  // they hold for every slice, and with the slices' base addresses, which are
+  // the same for the whole warp, address the slots in few instructions.
+  unsigned ro[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) ro[j] = ((unsigned)(max(rb.yb[j], 0) + rb.xb) * QVB + rb.xin) * (unsigned)sizeof(S);
+  const unsigned dl = (unsigned)(rb.dl * (int)sizeof(S)), dr = (unsigned)(rb.dr * (int)sizeof(S));
+  auto slice = [&](auto ptag, int z) {
+    constexpr bool PLAIN = decltype(ptag)::value;
+    constexpr bool W = WALLS && !PLAIN;
     int zb[3];
     slice_blocks<W>(bd, z, zb);
     S* const own = cell_ptr(f, zb[1] + rb.yb[1] + rb.xb, rb.xin);  // slot 0 of cell x0
+    char* const sb[3] = {base + (z > 0 ? z - 1 : nz - 1) * slice_bytes, base + z * slice_bytes,
+                         base + (z < nz - 1 ? z + 1 : 0) * slice_bytes};
+    // slot i of the cell at byte offset o of slice z + dz
+    auto at = [&](int dz, unsigned o, int i) { return reinterpret_cast<S*>(sb[1 + dz] + o) + i * VB; };
     // arrivals (stored units), both cells
     typename T::raw d[Q];
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-      if (PAR == 0 || i == 0) {
+      if (PLAIN) {
+        const int o = opp(i), ry = 1 - cy(i), dz = -cz(i);
+        if (i == 0) d[i] = T::ld(at(0, ro[1], i));
+        else if (cx(i) == 0) d[i] = T::ld(at(dz, ro[ry], o));
+        else if (cx(i) > 0) d[i] = T::ld(at(dz, ro[ry] + dl, o), at(dz, ro[ry], o));  // sources x0 - 1, x0
+        else d[i] = T::ld(at(dz, ro[ry], o) + 1, at(dz, ro[ry] + dr, o));             // sources x0 + 1, x0 + 2
+      } else if (PAR == 0 || i == 0) {
         d[i] = T::ld(own + i * VB);
       } else {
         // slot ibar of x - c_i, or slot i of x when x - c_i lies beyond a wall
@@ -234,7 +271,13 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
     // slot i of x + c_i, or slot ibar of x when x + c_i lies beyond a wall
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-      if (PAR == 0 || i == 0) {
+      if (PLAIN) {
+        const int ry = 1 + cy(i), dz = cz(i);
+        if (i == 0) T::st(at(0, ro[1], 0), d[i]);
+        else if (cx(i) == 0) T::st(at(dz, ro[ry], i), d[i]);
+        else if (cx(i) > 0) T::st(at(dz, ro[ry], i) + 1, at(dz, ro[ry] + dr, i), d[i]);  // destinations x0 + 1, x0 + 2
+        else T::st(at(dz, ro[ry] + dl, i), at(dz, ro[ry], i), d[i]);                     // destinations x0 - 1, x0
+      } else if (PAR == 0 || i == 0) {
         T::st(own + opp(i) * VB, d[i]);
       } else {
         const int by = rb.yb[1 + cy(i)], bz = zb[1 + cz(i)];
@@ -266,8 +309,8 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
   // one z slice at a time: an unrolled loop would hold two slices' arrivals
 #pragma unroll 1
   for (int z = z0; z < z1; ++z) {
-    if (WALLS && !(row_free && !((bd.bc & 4) && (z == 0 || z == bd.nz - 1))))
-      slice(std::integral_constant<bool, WALLS>{}, z);
+    if (FAST && (plain_row && !(WALLS && (bd.bc & 4) && (z == 0 || z == nz - 1))))
+      slice(std::integral_constant<bool, true>{}, z);
     else
       slice(std::integral_constant<bool, false>{}, z);
   }
