@@ -812,11 +812,12 @@ int hlbm_add_grid(hlbm_handle h, int nx, int ny, int nz, double spacing, const f
 // mea_group, the planes whose cells a group of four warps sums together, is
 // part of the result (to the last bit of a force): one plane up to four
 // resident waves of one-plane blocks, then up to three.  The blocks are not:
-// few particles are split over several blocks of 256 threads to shorten one
-// particle's latency, many take one block of 128 threads each, where no
-// block waits for another's sum (us, 256 threads and 6 planes against 128
-// and 24: 200 spheres FP32 35 / 57, 2000 ellipsoids and cuboids 249 / 170,
-// 50 000 spheres FP16 2869 / 1470).
+// up to four particles per SM get blocks of 256 threads, several per
+// particle while that leaves no more than three blocks per SM, more particles
+// one block of 128 threads each, where no block waits for another's sum (us,
+// 256 threads with two to three blocks a particle / with one / 128 threads:
+// 200 spheres FP32 35 / 38 / 57, 495 spheres 64 / 50 / 51, 2000 ellipsoids
+// and cuboids 249 / 174 / 170, 50 000 spheres FP16 2869 / 1813 / 1470).
 // In the moments form neither is: there a block takes about as many cells
 // as its threads walk in six (few particles) or twenty (many) rounds.
 static int plan_exchange(hlbm_ctx* h) {
@@ -839,9 +840,9 @@ static int plan_exchange(hlbm_ctx* h) {
     for (int p = 0; p < h->np; ++p) {
       // whole groups of planes per block
       const int g = form ? 1 : G, groups = (h->h_planes[p] + g - 1) / g;
-      int want = form ? (int)std::ceil(h->h_cells[p] / ((few ? 6.0 : 20.0) * t))
-                      : (h->h_planes[p] + (few ? 5 : 23)) / (few ? 6 : 24);
-      want = std::max(1, std::max(want, nsm / h->np));  // at least a block per SM
+      int want = form ? (int)std::ceil(h->h_cells[p] / ((few ? 6.0 : 20.0) * t)) : (h->h_planes[p] + 23) / 24;
+      // at least a block (three) per SM
+      want = std::max(1, std::max(want, (form ? 1 : 3) * nsm / h->np));
       const int per = (groups + want - 1) / want, parts = (groups + per - 1) / per;
       for (int k = 0; k < parts; ++k) ck[form].push_back(make_int4(p, k * per * g, per * g, parts));
     }
