@@ -763,25 +763,43 @@ __device__ __forceinline__ double contact_ramp(double k, double zeta, double gap
   return k * x * x;
 }
 
-// one warp per particle: the lanes take the other particles of its box in
-// turn (an FP32 test of the centre distance against the capsules' reach
-// first), lane 0 the walls; the warp's FP64 sums are added in a fixed order
-__global__ void __launch_bounds__(256) contact_kernel(PartArgs a) {
-  pdl_trigger();
-  pdl_wait();
-  const int i = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (i >= a.np) return;  // whole warps
+// One warp per particle.  The block stages the others' centres and reaches
+// in shared memory, CT_CHUNK at a time; the lanes test them in FP32 (centre
+// distance against the capsules' reach) and list those near enough, which
+// then take the FP64 arithmetic together, a lane each: its long dependent
+// chains cost the same for one lane and for 32, and a warp that ran them at
+// every group of 32 with a near particle spent its time there (495 spheres 33
+// us before).  Lane 0 takes the walls; the warp's FP64 sums are added in a
+// fixed order.
+constexpr int CT_WARPS = 4, CT_CHUNK = 256, CT_NEAR = 64;
+
+__global__ void __launch_bounds__(CT_WARPS * 32) contact_kernel(PartArgs a) {
+  __shared__ float4 s_pos[CT_CHUNK];  // centre, reach of the contact capsule
+  __shared__ int s_box[CT_CHUNK];
+  __shared__ int s_near[CT_WARPS][CT_NEAR];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int i = blockIdx.x * CT_WARPS + warp;
+  const bool active = i < a.np;  // whole warps; all threads stage
   const double* P = a.P;
   const int cap = a.cap;
-  const Rec& Ri = a.rec[i];
-  const int si = a.shape[i], box = a.box[i];
+  // what no step changes is read before the wait for the kernel before
+  const int box = active ? a.box[i] : 0, shape = active ? a.shape[i] : 0;
   const BoxDesc bd = a.boxes[box];
+  pdl_trigger();
+  pdl_wait();
   const int n[3] = {bd.nx, bd.ny, bd.nz};
-  double Xi[3], ei[3], hi, ri;
-  for (int j = 0; j < 3; ++j) Xi[j] = pget(P, cap, PF_X + j, i);
-  contact_capsule(P, cap, i, si, ei, hi, ri);
-  const float reach_i = contact_reach(Ri);
+  const float L[3] = {(float)bd.nx, (float)bd.ny, (float)bd.nz};
+  float xi[3] = {0.f, 0.f, 0.f}, reach_i = 0.f;
+  double Xi[3] = {0.0, 0.0, 0.0}, ei[3] = {0.0, 0.0, 1.0}, hi = 0.0, ri = 0.0;
+  if (active) {
+    const Rec& Ri = a.rec[i];
+    for (int c = 0; c < 3; ++c) {
+      xi[c] = Ri.xh[c];
+      Xi[c] = pget(P, cap, PF_X + c, i);
+    }
+    reach_i = contact_reach(Ri);
+    contact_capsule(P, cap, i, shape, ei, hi, ri);
+  }
   const double k = a.contact_k, zeta = a.contact_zeta;
   double F[3] = {0.0, 0.0, 0.0}, T[3] = {0.0, 0.0, 0.0};
   auto add = [&](const double pt[3], const double f[3]) {
@@ -793,34 +811,20 @@ __global__ void __launch_bounds__(256) contact_kernel(PartArgs a) {
       T[c] += tq[c];
     }
   };
-  for (int j = lane; j < a.np; j += 32) {
-    if (j == i || a.box[j] != box) continue;
-    const Rec& Rj = a.rec[j];
-    float d2 = 0.0f;
-    for (int c = 0; c < 3; ++c) {
-      float dc = Rj.xh[c] - Ri.xh[c];
-      if (!((bd.bc >> c) & 1)) {
-        const float L = (float)n[c];
-        if (dc > 0.5f * L) dc -= L;
-        else if (dc < -0.5f * L) dc += L;
-      }
-      d2 += dc * dc;
-    }
-    const float lim = reach_i + contact_reach(Rj) + (float)zeta + 0.05f;
-    if (d2 >= lim * lim) continue;
+  auto pair = [&](int j) {
     double Xj[3], ej[3], hj, rj;
     for (int c = 0; c < 3; ++c) {
       double dc = pget(P, cap, PF_X + c, j) - Xi[c];
       if (!((bd.bc >> c) & 1)) {
-        const double L = (double)n[c];
-        if (dc > L / 2.0) dc -= L;
-        else if (dc < -L / 2.0) dc += L;
+        const double Ld = (double)n[c];
+        if (dc > Ld / 2.0) dc -= Ld;
+        else if (dc < -Ld / 2.0) dc += Ld;
       }
       Xj[c] = Xi[c] + dc;
     }
     contact_capsule(P, cap, j, a.shape[j], ej, hj, rj);
-    double s, t;
-    segment_closest(Xi, ei, hi, Xj, ej, hj, s, t);
+    double s = 0.0, t = 0.0;
+    if (hi > 0.0 || hj > 0.0) segment_closest(Xi, ei, hi, Xj, ej, hj, s, t);  // two spheres: the centres
     double pi[3], dv[3], dist = 0.0;
     for (int c = 0; c < 3; ++c) {
       pi[c] = Xi[c] + s * ei[c];
@@ -829,12 +833,57 @@ __global__ void __launch_bounds__(256) contact_kernel(PartArgs a) {
     }
     dist = sqrt(dist);
     const double gap = dist - ri - rj;
-    if (gap >= zeta || !(dist > 0.0)) continue;
+    if (gap >= zeta || !(dist > 0.0)) return;
     const double fm = contact_ramp(k, zeta, gap);
     const double f[3] = {fm * dv[0] / dist, fm * dv[1] / dist, fm * dv[2] / dist};
     add(pi, f);
+  };
+  int near = 0;
+  auto flush = [&]() {
+    __syncwarp();
+    for (int c = lane; c < near; c += 32) pair(s_near[warp][c]);
+    __syncwarp();
+    near = 0;
+  };
+  const float far = (float)zeta + 0.05f;
+  for (int j0 = 0; j0 < a.np; j0 += CT_CHUNK) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < CT_CHUNK && j0 + e < a.np; e += CT_WARPS * 32) {
+      const Rec& Rj = a.rec[j0 + e];
+      s_pos[e] = make_float4(Rj.xh[0], Rj.xh[1], Rj.xh[2], contact_reach(Rj));
+      s_box[e] = Rj.box;
+    }
+    __syncthreads();
+    if (!active) continue;
+    const int m = min(CT_CHUNK, a.np - j0);
+    for (int e0 = 0; e0 < m; e0 += 32) {
+      const int e = e0 + lane;
+      bool hit = false;
+      if (e < m && j0 + e != i && s_box[e] == box) {
+        const float4 q = s_pos[e];
+        float d2 = 0.0f;
+        const float xj[3] = {q.x, q.y, q.z};
+        for (int c = 0; c < 3; ++c) {
+          float dc = xj[c] - xi[c];
+          if (!((bd.bc >> c) & 1)) {
+            if (dc > 0.5f * L[c]) dc -= L[c];
+            else if (dc < -0.5f * L[c]) dc += L[c];
+          }
+          d2 += dc * dc;
+        }
+        const float lim = reach_i + q.w + far;
+        hit = d2 < lim * lim;
+      }
+      const unsigned h = __ballot_sync(0xffffffffu, hit);
+      if (!h) continue;
+      if (near + __popc(h) > CT_NEAR) flush();
+      if (hit) s_near[warp][near + __popc(h & ((1u << lane) - 1u))] = j0 + e;
+      near += __popc(h);
+    }
   }
-  if (lane == 0) {
+  if (!active) return;
+  flush();
+  if (lane == 0)
     for (int c = 0; c < 3; ++c) {
       if (!((bd.bc >> c) & 1) || (c == 2 && (bd.bc & BC_CUT_Z))) continue;
       for (int side = 0; side < 2; ++side) {
@@ -848,12 +897,12 @@ __global__ void __launch_bounds__(256) contact_kernel(PartArgs a) {
         add(pt, f);
       }
     }
-  }
-  for (int c = 0; c < 3; ++c)
-    for (int o = 16; o > 0; o >>= 1) {
-      F[c] += __shfl_xor_sync(0xffffffffu, F[c], o);
-      T[c] += __shfl_xor_sync(0xffffffffu, T[c], o);
-    }
+  if (__any_sync(0xffffffffu, F[0] != 0.0 || F[1] != 0.0 || F[2] != 0.0))
+    for (int c = 0; c < 3; ++c)
+      for (int o = 16; o > 0; o >>= 1) {
+        F[c] += __shfl_xor_sync(0xffffffffu, F[c], o);
+        T[c] += __shfl_xor_sync(0xffffffffu, T[c], o);
+      }
   if (lane == 0)
     for (int c = 0; c < 3; ++c) {
       pset(a.P, cap, PF_FC + c, i, F[c]);
@@ -913,8 +962,8 @@ cudaError_t launch_update(const PartArgs& a_in, cudaStream_t s) {
 
 cudaError_t launch_contact(const PartArgs& a, cudaStream_t s) {
   if (a.np <= 0 || !(a.contact_k > 0.0)) return cudaSuccess;
-  const long long threads = (long long)a.np * 32;
-  return launch_k(contact_kernel, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, s, a.pdl != 0, a);
+  return launch_k(contact_kernel, dim3((unsigned)((a.np + CT_WARPS - 1) / CT_WARPS)), dim3(CT_WARPS * 32), 0, s,
+                  a.pdl != 0, a);
 }
 
 cudaError_t launch_records(const PartArgs& a, cudaStream_t s) {
