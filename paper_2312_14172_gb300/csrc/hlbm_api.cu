@@ -116,6 +116,10 @@ bool make_layout(int nb, const hlbm_box* boxes, const hlbm_params* prm, Layout& 
   return true;
 }
 
+// steps per captured graph: a run takes the longest that fit
+constexpr int GRAPH_KINDS = 4;
+constexpr int GRAPH_STEPS[GRAPH_KINDS] = {8, 4, 2, 1};
+
 thread_local std::string g_init_err;
 
 }  // namespace
@@ -173,14 +177,9 @@ struct hlbm_ctx {
   int cells_x = 1;       // cells per thread along x
   bool pair_ok = false;  // the two-cell kernel may run
   bool wide_slices = false;  // a z slice of some box takes 4 GB or more
-  // [0][parity]: step with the momentum-exchange kernel (after any change of
-  // state); [1][parity]: step that takes the sums the previous collision made
-  cudaGraphExec_t exec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
-  // two steps in one graph: [m][parity] = step(parity, m) then step(1 - parity)
-  cudaGraphExec_t exec2[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
-  // GRAPH_STEPS steps in one graph, the same way (when more than two)
-  cudaGraphExec_t execk[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
-  bool graphs_ok = false;
+  // captured steps [steps per graph][moments form in the first][parity], built
+  // when a run first asks for them
+  cudaGraphExec_t exec[GRAPH_KINDS][2][2] = {};
   // the last collision knew this particle state, so in the moments mode the
   // momentum exchange takes the moments form
   bool moments_valid = false;
@@ -297,13 +296,6 @@ static PartArgs part_args(const hlbm_ctx* h, int parity, bool moments = false) {
 // collision of the previous step knew the particle state); otherwise the link
 // sums (always on the first step after a change of state).
 // Kernels captured into a step's graph use programmatic dependent launch.
-// steps per captured graph for long runs (two-step and one-step graphs
-// take the rest)
-#ifndef HLBM_GRAPH_STEPS
-#define HLBM_GRAPH_STEPS 8
-#endif
-constexpr int GRAPH_STEPS = HLBM_GRAPH_STEPS;
-
 static cudaError_t enqueue_step(hlbm_ctx* h, int parity, bool moments, cudaStream_t s) {
   cudaError_t e;
   LbmArgs la = lbm_args(h, parity);
@@ -320,43 +312,34 @@ static cudaError_t enqueue_step(hlbm_ctx* h, int parity, bool moments, cudaStrea
 }
 
 static void drop_graphs(hlbm_ctx* h) {
-  for (int f = 0; f < 2; ++f)
-    for (int k = 0; k < 2; ++k) {
-      if (h->exec[f][k]) cudaGraphExecDestroy(h->exec[f][k]);
-      if (h->exec2[f][k]) cudaGraphExecDestroy(h->exec2[f][k]);
-      if (h->execk[f][k]) cudaGraphExecDestroy(h->execk[f][k]);
-      h->exec[f][k] = nullptr;
-      h->exec2[f][k] = nullptr;
-      h->execk[f][k] = nullptr;
-    }
-  h->graphs_ok = false;
+  for (auto& kind : h->exec)
+    for (auto& form : kind)
+      for (cudaGraphExec_t& g : form) {
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
+      }
 }
 
-static int build_graphs(hlbm_ctx* h) {
-  drop_graphs(h);
-  const bool mom = h->mea_mode == HLBM_MEA_MOMENTS;
-  for (int gi = 0; gi < 12; ++gi) {
-    const int kind = gi >> 2, moments = (gi >> 1) & 1, parity = gi & 1;
-    const int nst = kind == 0 ? 1 : (kind == 1 ? 2 : GRAPH_STEPS);
-    if (moments && !mom) continue;
-    if (kind == 2 && GRAPH_STEPS <= 2) continue;
-    cudaGraph_t g = nullptr;
-    CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = enqueue_step(h, parity, moments != 0, h->cap_stream);
-    for (int j = 1; j < nst && e == cudaSuccess; ++j) e = enqueue_step(h, (parity + j) & 1, mom, h->cap_stream);
-    cudaError_t e2 = cudaStreamEndCapture(h->cap_stream, &g);
-    if (e != cudaSuccess || e2 != cudaSuccess) {
-      if (g) cudaGraphDestroy(g);
-      return fail(h, HLBM_ERR_CUDA, std::string("graph capture: ") +
-                                        cudaGetErrorString(e != cudaSuccess ? e : e2));
-    }
-    cudaGraphExec_t* dst = kind == 0 ? &h->exec[moments][parity]
-                                     : (kind == 1 ? &h->exec2[moments][parity] : &h->execk[moments][parity]);
-    e = cudaGraphInstantiate(dst, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return fail(h, HLBM_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+// Captures the graph of GRAPH_STEPS[kind] steps from `parity` on, the first
+// with the given form of the momentum exchange, unless it is there.  Only the
+// graphs that a run asks for are built (all twelve of them, built at the
+// first step, took 170 us of a first pass of 20 steps at 48^3).
+static int need_graph(hlbm_ctx* h, int kind, int moments, int parity) {
+  cudaGraphExec_t* dst = &h->exec[kind][moments][parity];
+  if (*dst) return HLBM_OK;
+  cudaGraph_t g = nullptr;
+  CK(cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
+  cudaError_t e = cudaSuccess;
+  for (int j = 0; j < GRAPH_STEPS[kind] && e == cudaSuccess; ++j)
+    e = enqueue_step(h, (parity + j) & 1, j == 0 ? moments != 0 : h->mea_mode == HLBM_MEA_MOMENTS, h->cap_stream);
+  cudaError_t e2 = cudaStreamEndCapture(h->cap_stream, &g);
+  if (e != cudaSuccess || e2 != cudaSuccess) {
+    if (g) cudaGraphDestroy(g);
+    return fail(h, HLBM_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e != cudaSuccess ? e : e2));
   }
-  h->graphs_ok = true;
+  e = cudaGraphInstantiate(dst, g, 0);
+  cudaGraphDestroy(g);
+  if (e != cudaSuccess) return fail(h, HLBM_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
   return HLBM_OK;
 }
 
@@ -1045,24 +1028,24 @@ int hlbm_step(hlbm_handle h, int nsteps) {
   if (h->split) return fail(h, HLBM_ERR_STATE, "a split step is open (finish it with hlbm_step_with_forces)");
   if (nsteps < 0) return fail(h, HLBM_ERR_ARG, "nsteps < 0");
   if (nsteps == 0) return HLBM_OK;
-  if (!h->graphs_ok) {
-    const int rc = build_graphs(h);
-    if (rc != HLBM_OK) return rc;
-  }
-  for (int k = 0; k < nsteps;) {
-    const int moments = (h->moments_valid && h->np > 0) ? 1 : 0;
-    const int parity = (int)((h->steps + k) & 1);
-    if (GRAPH_STEPS > 2 && nsteps - k >= GRAPH_STEPS) {
-      CK(cudaGraphLaunch(h->execk[moments][parity], h->stream));
-      k += GRAPH_STEPS;
-    } else if (nsteps - k >= 2) {
-      CK(cudaGraphLaunch(h->exec2[moments][parity], h->stream));
-      k += 2;
-    } else {
-      CK(cudaGraphLaunch(h->exec[moments][parity], h->stream));
-      k += 1;
+  // the first round sees to the graphs, so that all are there before the
+  // second launches any
+  for (int launch = 0; launch < 2; ++launch) {
+    int moments = (h->moments_valid && h->np > 0) ? 1 : 0;
+    for (int k = 0; k < nsteps;) {
+      int kind = 0;
+      while (GRAPH_STEPS[kind] > nsteps - k) ++kind;
+      const int parity = (int)((h->steps + k) & 1);
+      if (launch) {
+        CK(cudaGraphLaunch(h->exec[kind][moments][parity], h->stream));
+        h->moments_valid = h->mea_mode == HLBM_MEA_MOMENTS;
+      } else {
+        const int rc = need_graph(h, kind, moments, parity);
+        if (rc != HLBM_OK) return rc;
+      }
+      k += GRAPH_STEPS[kind];
+      moments = h->mea_mode == HLBM_MEA_MOMENTS && h->np > 0 ? 1 : 0;
     }
-    h->moments_valid = h->mea_mode == HLBM_MEA_MOMENTS;
   }
   h->steps += nsteps;
   return HLBM_OK;
