@@ -168,6 +168,7 @@ struct hlbm_ctx {
   int* hstatus = nullptr;
   cudaEvent_t hstage_ev = nullptr;
   bool walls = false;
+  bool elongated = false;  // some particle is no sphere
   // contact stiffness and range (an extension; 0 = off)
   double contact_k = 0.0, contact_zeta = 1.0;
   int np = 0;
@@ -251,6 +252,7 @@ static LbmArgs lbm_args(const hlbm_ctx* h, int parity) {
   a.bin_ids = h->ids[parity];
   a.bin_cap = h->L.bin_cap;
   a.rec = h->rec;
+  a.elongated = h->elongated;
   a.grids = h->grids.empty() ? GridSet{} : GridSet{h->d_gdesc, h->d_gvals};
   a.status = h->status;
   return a;
@@ -942,6 +944,7 @@ int hlbm_add_particles(hlbm_handle h, int n, const int* box_id, const int* shape
   h->np += n;
   h->hst_valid = false;
   h->h_shape.insert(h->h_shape.end(), sh.begin(), sh.end());
+  for (int s : sh) h->elongated = h->elongated || s != HLBM_SPHERE;
   h->h_box.insert(h->h_box.end(), bx.begin(), bx.end());
   h->h_planes.insert(h->h_planes.end(), nch.begin(), nch.end());
   h->h_cells.insert(h->h_cells.end(), cells.begin(), cells.end());

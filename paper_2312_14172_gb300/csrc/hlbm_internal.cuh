@@ -289,6 +289,7 @@ struct LbmArgs {
   const int* bin_ids;
   int bin_cap;
   const Rec* rec;
+  int elongated;            // some particle is no sphere
   GridSet grids;            // signed-distance grids of shape-4 particles
   int* status;
 };

@@ -29,6 +29,7 @@ template <typename S, int PAR, bool WALLS, int C>
 __global__ void __launch_bounds__(256, HLBM_CS_MINBLOCKS) collide_stream_kernel(LbmArgs a) {
   constexpr bool COUPLE = C > 0;
   __shared__ Rec srec[COUPLE ? MAX_CAND : 1];
+  __shared__ Capsule scap[C == 1 ? MAX_CAND : 1];
   // per row of the brick (local y + sub_y * local z): the candidates whose
   // influence sphere meets the row
   __shared__ unsigned long long s_rowmask[COUPLE ? TILE_Y * TILE_Z : 1];
@@ -37,7 +38,7 @@ __global__ void __launch_bounds__(256, HLBM_CS_MINBLOCKS) collide_stream_kernel(
   pdl_wait();
   const Brick k = brick_of(a);
   const BoxDesc& bd = k.bd;
-  if (COUPLE) load_candidates(a, k, srec, s_rowmask);
+  if (COUPLE) load_candidates<(C > 1)>(a, k, srec, scap, s_rowmask);
 
   const int x = k.x0 + threadIdx.x;
   const int y = k.y0 + threadIdx.y;
@@ -73,7 +74,7 @@ __global__ void __launch_bounds__(256, HLBM_CS_MINBLOCKS) collide_stream_kernel(
     // positions only and runs while the loads above are in flight
     RowCoupling<1> cc;
     if (COUPLE)
-      couple_row<1, (C > 1)>(srec, s_rowmask[threadIdx.y + a.sub_y * (z - z0)], bd, x, y, z, a.eps,
+      couple_row<1, (C > 1)>(srec, scap, s_rowmask[threadIdx.y + a.sub_y * (z - z0)], bd, x, y, z, a.eps,
                              a.inv_eps, a.status, cc, a.grids);
     float drho = 0.0f, jx = 0.0f, jy = 0.0f, jz = 0.0f;
 #pragma unroll

@@ -111,6 +111,7 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
   constexpr bool FAST = PAR == 1 && (sizeof(S) == 2 || WALLS);
   using T = Two<S>;
   __shared__ Rec srec[COUPLE ? MAX_CAND : 1];
+  __shared__ Capsule scap[C == 1 ? MAX_CAND : 1];
   __shared__ unsigned long long s_rowmask[COUPLE ? TILE_Y * TILE_Z : 1];
   const bool early = (long long)blockIdx.x + a.pdl_tail >= (long long)gridDim.x;
   if (early) pdl_trigger();
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
     if (py < bd.ny && pz < bd.nz) prefetch_block(reinterpret_cast<const S*>(a.f), block_of(bd, k.x0, py, pz));
   }
   pdl_wait();
-  if (COUPLE) load_candidates(a, k, srec, s_rowmask);
+  if (COUPLE) load_candidates<(C > 1)>(a, k, srec, scap, s_rowmask);
 
   const int z0 = uniform(k.z0), nz = uniform(bd.nz);
   const int z1 = min(z0 + a.sub_z, nz);
@@ -199,7 +200,7 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
     // loads above are in flight
     RowCoupling<2> cc;
     if (COUPLE) {
-      couple_row<2, (C > 1)>(srec, s_rowmask[threadIdx.y + a.sub_y * (z - z0)], bd, x0, y, z, a.eps,
+      couple_row<2, (C > 1)>(srec, scap, s_rowmask[threadIdx.y + a.sub_y * (z - z0)], bd, x0, y, z, a.eps,
                              a.inv_eps, a.status, cc, a.grids);
     }
     // mass and momentum of the arrivals
