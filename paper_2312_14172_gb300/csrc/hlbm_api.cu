@@ -156,6 +156,7 @@ struct hlbm_ctx {
   int mea_group = 1;            // planes whose cells are summed together
   bool fused = false;           // the momentum exchange moves the particles too
   std::vector<double> h_cells;  // about the cells inside each particle
+  std::vector<int> h_tile;      // the bin tile each was added in
   int mea_mode = HLBM_MEA_KERNEL;
   int* cnt[2] = {nullptr, nullptr};
   int* ids[2] = {nullptr, nullptr};
@@ -818,11 +819,22 @@ static int plan_exchange(hlbm_ctx* h) {
   // exchange's blocks from waiting on FP64 (50 000 spheres: 5550 us per step
   // against 5729)
   h->fused = few;
+  // particles in the reverse order of the tiles they were added in (counting
+  // sort): blocks that run together then read neighbouring rows, the first
+  // ones those that the collision wrote last (us, against the order of
+  // addition: 50 000 spheres FP16 963 -> 904, 2000 ellipsoids and cuboids 117
+  // -> 110, 64 boxes 230 -> 220).  Particles move little in a run; an order
+  // gone stale costs only time.
+  std::vector<int> order(h->np), at((size_t)h->L.ntiles + 1, 0);
+  for (int t : h->h_tile) ++at[h->L.ntiles - 1 - t + 1];
+  for (size_t t = 1; t < at.size(); ++t) at[t] += at[t - 1];
+  for (int p = 0; p < h->np; ++p) order[at[h->L.ntiles - 1 - h->h_tile[p]]++] = p;
   std::vector<int4> ck[2];
   for (int form = 0; form < 2; ++form) {
     const int t = few ? 256 : 128;
     h->mea_threads[form] = t;
-    for (int p = 0; p < h->np; ++p) {
+    ck[form].reserve(h->np);
+    for (int p : order) {
       // whole groups of planes per block
       const int g = form ? 1 : G, groups = (h->h_planes[p] + g - 1) / g;
       int want = form ? (int)std::ceil(h->h_cells[p] / ((few ? 6.0 : 20.0) * t)) : (h->h_planes[p] + 23) / 24;
@@ -851,6 +863,7 @@ int hlbm_add_particles(hlbm_handle h, int n, const int* box_id, const int* shape
   std::vector<double> tab((size_t)PF_COUNT * n, 0.0);
   std::vector<int> sh(n), bx(n), nch(n);
   std::vector<double> cells(n);
+  std::vector<int> tile(n);
   auto T = [&](int fld, int k) -> double& { return tab[(size_t)fld * n + k]; };
   for (int k = 0; k < n; ++k) {
     const int b = box_id ? box_id[k] : 0;
@@ -924,6 +937,8 @@ int hlbm_add_particles(hlbm_handle h, int n, const int* box_id, const int* shape
     }
     wrap_host(bd, x);
     for (int j = 0; j < 3; ++j) T(PF_X + j, k) = x[j];
+    auto cell = [&](int j) { return (int)std::min(std::max(x[j], 0.0), nn[j] - 1.0); };  // a slab's centres may lie beyond
+    tile[k] = (int)(bd.tile_off + ((long long)(cell(2) / TILE_Z) * bd.nty + cell(1) / TILE_Y) * bd.ntx + cell(0) / TILE_X);
     for (int j = 0; j < 4; ++j) T(PF_Q + j, k) = q[j];
     T(PF_M, k) = m;
     T(PF_IM, k) = 1.0 / m;
@@ -948,6 +963,7 @@ int hlbm_add_particles(hlbm_handle h, int n, const int* box_id, const int* shape
   h->h_box.insert(h->h_box.end(), bx.begin(), bx.end());
   h->h_planes.insert(h->h_planes.end(), nch.begin(), nch.end());
   h->h_cells.insert(h->h_cells.end(), cells.begin(), cells.end());
+  h->h_tile.insert(h->h_tile.end(), tile.begin(), tile.end());
   rc = plan_exchange(h);
   if (rc != HLBM_OK) return rc;
   CK(launch_records(part_args(h, 0), h->stream));
