@@ -1,0 +1,175 @@
+"""Edges of the kernels around the momentum exchange: particle sizes and
+counts that change its blocks and its form, contacts beyond one list and one
+staging chunk, the FP64 exchange of populations in several runs, and the
+snapshot layout of the version before.
+
+Tolerances: a force is a sum over links of stored FP32 values, each relative
+to 6e-8 of itself, added in FP32 over the twenty or so cells of a thread and
+five levels of a warp, in FP64 or fixed point beyond; against the same sum in
+FP64 that is about 1e-6 of its magnitude, bounded here by 1e-5 of the largest
+force (torque) of the case.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+W = np.array([1 / 3] + [1 / 18] * 6 + [1 / 36] * 12)
+
+
+@pytest.fixture(scope="module")
+def H():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_2312_14172_gb300 import build, hlbm
+    build.build()
+    hlbm.load()
+    return hlbm
+
+
+def _pops(n, seed):
+    rng = np.random.default_rng(seed)
+    return W[:, None, None, None] * (1.0 + 1e-3 * rng.standard_normal((19, n[2], n[1], n[0])))
+
+
+def _pair(H, O, n, bc, parts, mode, seed=1):
+    shape, a, X, quat = parts
+    m = len(shape)
+    rng = np.random.default_rng(seed)
+    U, om = rng.uniform(-1e-3, 1e-3, (m, 3)), rng.uniform(-1e-3, 1e-3, (m, 3))
+    lat = H.Lattice([tuple(n) + (bc,)], H.make_params(tau=0.7, gravity=(1e-6, 0, -1e-5), max_particles=m))
+    orc = O.Oracle(n, 0.7, 0.5, bc, (1e-6, 0, -1e-5))
+    lat.add_particles(shape, a, X, U, om, quat, np.full(m, 2.0))
+    orc.add_particles(shape, a, X, U, om, quat, np.full(m, 2.0))
+    lat.set_mea_mode(mode)
+    f = _pops(n, seed + 1)
+    lat.set_populations(f)
+    orc.set_populations(f)
+    return lat, orc
+
+
+def _steps_agree(lat, orc, steps):
+    # the first step takes the link sums, later ones the mode's form
+    for _ in range(steps):
+        lat.step(1)
+        orc.step(1)
+        sg, so = lat.particle_state(), orc.particle_state()
+        for k in ("F", "T"):
+            assert np.max(np.abs(sg[k] - so[k])) <= 1e-5 * np.abs(so[k]).max(), k
+    fg, fo = lat.populations(), orc.populations()
+    assert np.max(np.abs(fg - fo) / fo) <= 1e-5
+    lat.close()
+
+
+@pytest.mark.parametrize("mode", ["kernel", "moments"])
+@pytest.mark.parametrize("r,X,bc", [
+    (0.45, (7.1, 6.2, 5.3), 0),       # at most a cell or two inside
+    (1.0, (0.2, 21.9, 0.4), 0),       # across three periodic faces
+    (12.3, (30.2, 3.1, 33.7), 7),     # cut by a wall, several blocks
+    (29.4, (39.7, 1.2, 68.9), 0),     # the most planes a particle may span
+])
+def test_one_particle_of_any_size(H, O, mode, r, X, bc):
+    n = (70, 67, 70) if r < 20 else (80, 72, 70)
+    lat, orc = _pair(H, O, n, bc, ([0], [[r] * 3], [X], [[1.0, 0, 0, 0]]), mode)
+    _steps_agree(lat, orc, 3)
+
+
+@pytest.mark.parametrize("mode", ["kernel", "moments"])
+@pytest.mark.parametrize("count", [40, 700])
+def test_few_and_many_particles_of_all_shapes(H, O, mode, count):
+    """Below four particles per SM the exchange moves its particle itself,
+    above it the update kernel does: the same step either way."""
+    n = (121, 90, 84)
+    rng = np.random.default_rng(count)
+    k = (10, 9, 8)
+    site = rng.permutation(k[0] * k[1] * k[2])[:count]
+    X = np.stack([site % k[0], site // k[0] % k[1], site // (k[0] * k[1])], 1) * (np.array(n) / k) + \
+        rng.uniform(0.0, 2.0, (count, 3))
+    shape = np.arange(count) % 4
+    a = rng.uniform(1.2, 2.6, (count, 3))
+    a[shape == 3, 1] = a[shape == 3, 0] = 1.5
+    q = rng.standard_normal((count, 4))
+    q /= np.linalg.norm(q, axis=1)[:, None]
+    lat, orc = _pair(H, O, n, 0, (shape, a, X, q), mode)
+    _steps_agree(lat, orc, 3)
+
+
+def test_contacts_beyond_one_list_and_one_chunk(H, O):
+    """A sphere with 90 neighbours in contact (a warp's list holds 64) among
+    300 particles (256 are staged at a time); fluid and particles at rest, so
+    the first step's velocities are contact and weight alone."""
+    n = (96, 90, 92)
+    k = np.arange(90) + 0.5
+    th, ph = np.arccos(1 - 2 * k / 90), np.pi * (1 + 5 ** 0.5) * k
+    shell = 11.4 * np.stack([np.sin(th) * np.cos(ph), np.sin(th) * np.sin(ph), np.cos(th)], 1) + (25.3, 26.1, 24.8)
+    g = np.arange(209)
+    # 7 cells apart: a bin tile holds at most 64 particles
+    far = np.stack([g % 7, g // 7 % 6, g // 42], 1) * 7.0 + (50.2, 45.1, 52.4)
+    X = np.concatenate([[(25.3, 26.1, 24.8)], shell, far])
+    r = np.concatenate([[10.0], np.full(len(X) - 1, 1.0)])
+    lat = H.Lattice([n + (4,)], H.make_params(tau=0.7, gravity=(0, 0, -1e-5), max_particles=len(X)))
+    orc = O.Oracle(n, 0.7, 0.5, 4, (0, 0, -1e-5))
+    a = np.repeat(r[:, None], 3, axis=1)
+    for o in (lat, orc):
+        o.add_particles(np.zeros(len(X), int), a, X, None, None, None, np.full(len(X), 2.0))
+        o.set_contact(1e-3, 1.5)
+    Fc, _ = orc.contact_forces()
+    assert np.count_nonzero(np.abs(Fc).max(axis=1) > 0) >= 91
+    lat.step(1)
+    orc.step(1)
+    sg, so = lat.particle_state(), orc.particle_state()
+    # FP64 on both sides: the sums of a particle's contacts in another order
+    assert np.max(np.abs(sg["U"] - so["U"])) <= 1e-12 * np.abs(so["U"]).max() + 1e-15
+    lat.close()
+
+
+@pytest.mark.parametrize("precision,dt,scale", [("fp32", np.float32, 1.0), ("fp16", np.float16, 2.0 ** 14)])
+def test_populations_in_several_runs(H, precision, dt, scale):
+    """A box of more cells than the staging area holds in FP64 (2^17), odd in
+    every axis, at both parities: set and get convert as stated, each value
+    f = w + (stored deviation), the deviation rounded once to FP32 and, with
+    half storage, once more."""
+    n = (67, 61, 71)
+    lat = H.Lattice([n + (2,)], H.make_params(tau=0.7, precision=precision))
+    w = W[:, None, None, None]
+    for seed in (3, 4):
+        f = _pops(n, seed)
+        lat.set_populations(f)
+        stored = ((f - w).astype(np.float32) * np.float32(scale)).astype(dt)
+        want = w + stored.astype(np.float32).astype(np.float64) / scale
+        assert np.array_equal(lat.populations(), want)
+        lat.step(1)
+    lat.close()
+
+
+def test_snapshot_of_the_version_before_loads(H):
+    """HLBMCKP3 held the list of interior cells before the populations: 64
+    int32 counts, 24 bytes per entry; it is stepped over."""
+    from paper_2312_14172_gb300 import workloads
+    w = workloads.hindered_settling(n=(70, 45, 48), count=14, steps=20)
+
+    def fresh():
+        return H.Lattice([w["n"] + (w["bc"],)], H.make_params(tau=w["tau"], eps=w["eps"], gravity=w["gravity"],
+                                                            max_particles=len(w["particles"]["shape"])))
+    a = H.from_workload(w)
+    a.set_mea_mode("moments")
+    a.step(5)
+    snap = a.save()
+    pops = 3 * 45 * 48 * 19 * 32 * 4
+    counts = np.zeros(64, np.int32)
+    counts[3] = 2
+    old = b"HLBMCKP3" + snap[8:-pops] + counts.tobytes() + bytes(48) + snap[-pops:]
+    b = fresh()
+    b.load_snapshot(old)
+    a.step(4)
+    b.step(4)
+    assert np.array_equal(a.populations(), b.populations())
+    for cut in (pops + 40, pops + 200):
+        c = fresh()
+        with pytest.raises(H.HLBMError) as e:
+            c.load_snapshot(old[:-cut])
+        assert e.value.code == H.HLBM_ERR_ARG
+        c.close()
+    a.close()
+    b.close()
