@@ -293,7 +293,9 @@ struct ExchangeRows {
   int start[XCH_MAX_T];
   int xa[XCH_MAX_T], y[XCH_MAX_T], z[XCH_MAX_T];
   int wtot[XCH_MAX_T / 32];
+  unsigned found[XCH_MAX_T / 32][64];  // grid particles: a warp's interior cells, row << 8 | x - xa[row]
 };
+static_assert(MAX_PLANES <= 256 && XCH_MAX_T <= 1 << 24, "packing of ExchangeRows::found");
 
 // Calls cell(x, y, z, rr) for every interior cell of planes [q0, q0 + nq) of
 // the particle's bounding box (rr its offset from the centre), spread over
@@ -313,7 +315,11 @@ __device__ __forceinline__ void for_interior(const Rec& R, const BoxDesc& bd, in
   exchange_extent(R.xh[2], rc, bd.bc & 4, cutz ? bd.own_lo : 0, cutz ? bd.own_hi - 1 : bd.nz - 1, loz, extz);
   const int planes = min(nq, extz - q0);
   const int rows = planes > 0 ? planes * exty : 0;
-  const Capsule cap = capsule_of(R, 0.0f);
+  Capsule cap = capsule_of(R, 0.0f);
+  if (GRIDS && R.shape == 4 && gs.desc) {  // the interior only
+    cap.h = gs.desc[__float_as_int(R.in2)].out_h;
+    cap.r2 = gs.desc[__float_as_int(R.in2)].out_r2;
+  }
   for (int row0 = 0; row0 < rows; row0 += nt) {
     const int row = row0 + tid;
     int len = 0, xa = 0, y = 0, z = 0;
@@ -352,6 +358,52 @@ __device__ __forceinline__ void for_interior(const Rec& R, const BoxDesc& bd, in
     sh.y[tid] = y;
     sh.z[tid] = z;
     __syncthreads();
+    if (GRIDS && R.shape == 4) {
+      // Half the candidate cells or more lie outside: the warp collects the
+      // inside ones and takes 32 at a time (the sums depend on no order).
+      int held = 0;  // of found[warp], the same in every lane
+      auto take = [&](int n) {
+        __syncwarp();
+        if (lane < n) {
+          const unsigned e = sh.found[warp][lane];
+          const int r = (int)(e >> 8), xu = sh.xa[r] + (int)(e & 255u);
+          const int x = xu < 0 ? xu + bd.nx : (xu >= bd.nx ? xu - bd.nx : xu);
+          const float rr[3] = {offset_fp32(x, bd.nx, bd.bc & 1, R.xh[0], R.xl[0]),
+                               offset_fp32(sh.y[r], bd.ny, bd.bc & 2, R.xh[1], R.xl[1]),
+                               offset_fp32(sh.z[r], bd.nz, bd.bc & 4, R.xh[2], R.xl[2])};
+          cell(x, sh.y[r], sh.z[r], rr);
+        }
+        __syncwarp();
+      };
+      for (int q0w = 32 * warp; q0w < total; q0w += nt) {
+        const int q = q0w + lane;
+        bool in = false;
+        unsigned e = 0;
+        if (q < total) {
+          int r = 0;
+          for (int step = nt >> 1; step > 0; step >>= 1)
+            if (sh.start[r + step] <= q) r += step;
+          e = ((unsigned)r << 8) | (unsigned)(q - sh.start[r]);
+          const int xu = sh.xa[r] + (q - sh.start[r]);
+          const int x = xu < 0 ? xu + bd.nx : (xu >= bd.nx ? xu - bd.nx : xu);
+          float rr[3];
+          in = (unsigned)x < (unsigned)bd.nx && inside_fp32(R, bd, x, sh.y[r], sh.z[r], rr, gs);
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        if (in) sh.found[warp][held + __popc(m & ((1u << lane) - 1u))] = e;
+        held += __popc(m);
+        if (held >= 32) {
+          take(32);
+          const unsigned rest = lane + 32 < held ? sh.found[warp][lane + 32] : 0u;
+          held -= 32;
+          if (lane < held) sh.found[warp][lane] = rest;
+          __syncwarp();
+        }
+      }
+      if (held) take(held);
+      __syncthreads();
+      continue;
+    }
     for (int q = tid; q < total; q += nt) {
       int r = 0;  // the row holding flat index q: the last one starting at or before it
       for (int step = nt >> 1; step > 0; step >>= 1)

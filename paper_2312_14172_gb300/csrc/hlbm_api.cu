@@ -621,11 +621,14 @@ static int upload_fields(hlbm_ctx* h, int p0, int n, const std::vector<double>& 
   return HLBM_OK;
 }
 
-// Two capsules about the body z axis of a grid, each the best of 65
+// Three capsules about the body z axis of a grid, each the best of 65
 // half-lengths.  Enclosing (g.cap_h, g.cap_r): the smallest that holds every
 // grid cell with a corner below eps/2 (the blend is a convex combination of
 // the corners, so B > 0 and the inside lie in those cells, and a cell whose
-// corners are in the capsule is in it).  Inscribed (d.in_h, d.in_r2): the
+// corners are in the capsule is in it); (d.out_h, d.out_r2) likewise for the
+// cells with a corner below 0, the only ones whose blend can be negative (in
+// FP32 too: a + t (b - a) with a, b >= 0 and t <= 1 rounds to no less than 0).
+// Inscribed (d.in_h, d.in_r2): the
 // largest that meets only grid cells all of whose corners are below
 // -(eps/2 + 1e-3), kept 1e-3 cells off the others (a cell's distance from the
 // axis segment is bounded by its centre's minus its half-diagonal); there
@@ -642,8 +645,9 @@ static void grid_capsules(hlbm_ctx::HostGrid& g, double half_eps, GridDesc& d) {
     const double t = r[2] - std::min(std::max(r[2], -hh), hh);
     return r[0] * r[0] + r[1] * r[1] + t * t;
   };
-  std::vector<std::array<double, 3>> hold, avoid;  // corners to hold, centres of cells to avoid
-  std::vector<char> mark((size_t)nx * ny * nz, 0);
+  // corners to hold (B > 0; the inside), centres of cells to avoid
+  std::vector<std::array<double, 3>> hold[2], avoid;
+  std::vector<char> mark((size_t)nx * ny * nz, 0);  // bit 0, 1: in hold[0], hold[1]
   const double deep = -(half_eps + 1e-3);
   for (int k = 0; k + 1 < nz; ++k)
     for (int j = 0; j + 1 < ny; ++j)
@@ -655,7 +659,8 @@ static void grid_capsules(hlbm_ctx::HostGrid& g, double half_eps, GridDesc& d) {
           vmax = std::max(vmax, v);
         }
         if (vmin < half_eps)
-          for (int c = 0; c < 8; ++c) mark[((size_t)(k + (c >> 2)) * ny + j + ((c >> 1) & 1)) * nx + i + (c & 1)] = 1;
+          for (int c = 0; c < 8; ++c)
+            mark[((size_t)(k + (c >> 2)) * ny + j + ((c >> 1) & 1)) * nx + i + (c & 1)] |= vmin < 0.0 ? 3 : 1;
         if (!(vmax < deep)) {
           double r[3];
           pos(i + 0.5, j + 0.5, k + 0.5, r);
@@ -665,23 +670,33 @@ static void grid_capsules(hlbm_ctx::HostGrid& g, double half_eps, GridDesc& d) {
   double zmax = 0.0;
   for (int k = 0; k < nz; ++k)
     for (int j = 0; j < ny; ++j)
-      for (int i = 0; i < nx; ++i)
-        if (mark[((size_t)k * ny + j) * nx + i]) {
-          double r[3];
-          pos(i, j, k, r);
-          hold.push_back({r[0], r[1], r[2]});
-          zmax = std::max(zmax, std::fabs(r[2]));
-        }
+      for (int i = 0; i < nx; ++i) {
+        const char m = mark[((size_t)k * ny + j) * nx + i];
+        double r[3];
+        pos(i, j, k, r);
+        for (int s = 0; s < 2; ++s)
+          if ((m >> s) & 1) hold[s].push_back({r[0], r[1], r[2]});
+        if (m) zmax = std::max(zmax, std::fabs(r[2]));
+      }
+  double best;
+  auto enclose = [&](const std::vector<std::array<double, 3>>& pts, double& cap_h, double& cap_r) {
+    best = HUGE_VAL;
+    for (int t = 0; t <= 64; ++t) {
+      const double hh = zmax * t / 64.0;
+      double r2 = 0.0;
+      for (const auto& c : pts) r2 = std::max(r2, seg_d2(c.data(), hh));
+      const double r = std::sqrt(r2), vol = M_PI * r * r * 2.0 * hh + 4.0 / 3.0 * M_PI * r * r * r;
+      if (vol < best) { best = vol; cap_h = hh; cap_r = r; }
+    }
+  };
   g.cap_h = 0.0;
   g.cap_r = g.rinf;
-  double best = HUGE_VAL;
-  for (int t = 0; t <= 64; ++t) {
-    const double hh = zmax * t / 64.0;
-    double r2 = 0.0;
-    for (const auto& c : hold) r2 = std::max(r2, seg_d2(c.data(), hh));
-    const double r = std::sqrt(r2), vol = M_PI * r * r * 2.0 * hh + 4.0 / 3.0 * M_PI * r * r * r;
-    if (vol < best) { best = vol; g.cap_h = hh; g.cap_r = r; }
-  }
+  enclose(hold[0], g.cap_h, g.cap_r);
+  double out_h = g.cap_h, out_r = g.cap_r;
+  enclose(hold[1], out_h, out_r);
+  out_r = out_r * 1.001 + 0.01;
+  d.out_h = (float)out_h;
+  d.out_r2 = (float)(out_r * out_r);
   const double half_diag = 0.5 * std::sqrt(3.0) * g.h;
   double in_h = 0.0, in_r = -1.0;
   best = 0.0;

@@ -104,6 +104,10 @@ struct GridDesc {
   // -(eps/2 + 1e-3): there B = 1 and the centre is inside, and the coupling
   // takes the distance in_d (below -(eps/2 + 1e-3)) without blending
   float in_h, in_r2, in_d;
+  // the smallest such capsule that holds every grid cell with a corner below
+  // 0 (half-length, squared radius with a margin for the rounding of FP32):
+  // beyond it no blend is negative
+  float out_h, out_r2;
   long long off;
 };
 struct GridSet {
