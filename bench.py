@@ -548,10 +548,10 @@ def run_gpu(args, ws, rank, local):
            "steps": e2e_steps,
            "note": "per step: hlbm_set_particle_state (X, U, omega, q) + hlbm_step(1) + "
                    "hlbm_particle_state (X, U, omega, q, F, T), pinned host arrays; the state written back "
-                   "is the one just read, so the step keeps the momentum exchange from the recorded moments",
+                   "is the one just read, so the step keeps the moments form of the momentum exchange",
            "moved": {"value": whole_job_mlups(cells, e2e_steps, t_moved * 1e3, ws), "unit": "MLUPS",
                      "note": "the same loop with every position written back changed (by 1e-9 cells): "
-                             "each step takes the bounding-box momentum exchange; the figure for a caller "
+                             "each step takes the link sums for its momentum exchange; the figure for a caller "
                              "that moves its particles itself"}}
     # state after the runs, for the FP16 comparison
     fp32_state = lat.particle_state()
@@ -628,7 +628,10 @@ def run_gpu(args, ws, rank, local):
     capsules = capsules_leg(args, stream, peak, ws) if args.capsules else None
     grids = grid_shapes_leg(args, stream, peak, ws) if args.grid_shapes else None
 
-    launches_per_step = 3 if npart > 0 else 1
+    # exchange, update, collision; fewer than four particles per SM are moved
+    # by the exchange's own blocks
+    few = npart < 4 * torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+    launches_per_step = (2 if few else 3) if npart > 0 else 1
     line = {
         "metric": "MLUPS incl. particle coupling", "value": value, "unit": "MLUPS", "n_gpus": ws,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,
@@ -714,9 +717,7 @@ def coupling_and_step_roofline(lat, cells, npart, steps, ms, ws, prec, peak):
     momentum exchange sums over; the library counts them in the moments
     mode (the mode is switched for one step if another was in use).  Bytes
     of a step: the collision's 2 * 19 * s per cell plus, per interior cell,
-    the momentum exchange's 19 arrivals (19 * s) and, in the moments mode,
-    the 24-byte list entry written by the collision and read back (in the
-    bounding-box mode the 19 departures instead)."""
+    the momentum exchange's 19 arrivals and 19 departures (2 * 19 * s)."""
     mode = lat.get_mea_mode()
     n_int = 0
     if npart > 0:
@@ -727,7 +728,7 @@ def coupling_and_step_roofline(lat, cells, npart, steps, ms, ws, prec, peak):
         if mode != "moments":
             lat.set_mea_mode(mode)
     s = BYTES_PER_CELL[prec] // 38
-    per_int = 19 * s + (48 if mode == "moments" else 19 * s)
+    per_int = 2 * 19 * s
     bpc_mea = BYTES_PER_CELL[prec] + per_int * n_int / cells
     sec = ms / steps / 1e3
     coupling = {"interior_cells_per_step": n_int, "interior_fraction": n_int / cells,

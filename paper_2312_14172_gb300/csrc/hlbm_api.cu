@@ -3,13 +3,15 @@
 //
 // One time step (Algorithm 1 of arXiv:2312.14172, Sec. 4.2.5, without its
 // communication rows) is three launches on the handle's stream:
-//   1. momentum exchange per particle          (mea_kernel)
+//   1. momentum exchange per particle          (mea_kernel, mea_moments_kernel)
 //   2. contact forces, when switched on       (contact_kernel)
 //      external force, Newton-Euler, records,
-//      per-tile particle lists                 (update_kernel)
-//   3. EDM coupling, collision and streaming   (collide_stream_kernel)
-// Steps alternate between the two AA parities, so each parity is captured
-// once as a CUDA graph and the graphs are launched alternately.
+//      per-tile particle lists                 (update_kernel; with few
+//                                              particles the exchange's blocks)
+//   3. EDM coupling, collision and streaming   (collide_pair_kernel,
+//                                              collide_stream_kernel)
+// Runs of 8, 4, 2 and 1 steps are captured as CUDA graphs, per parity of the
+// first step and form of the exchange, when a run first asks for them.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -1004,11 +1006,10 @@ int hlbm_set_particle_state(hlbm_handle h, const double* X, const double* U, con
   // the staging rows may still feed the previous upload
   CK(cudaEventSynchronize(h->hstage_ev));
   double* S = h->hstage;  // row r holds component r of the state, n doubles
-  // The cells inside the particles (and so the list the last collision
-  // recorded) depend on positions and, for non-spheres, orientations only:
+  // The moments form needs a collision that knew the same interior cells,
+  // and those depend on positions and, for non-spheres, orientations only:
   // when both come back as the state downloaded after this very step, bit
-  // for bit, the next step may still take the momentum exchange from the
-  // recorded moments.
+  // for bit, the next step may still take it.
   const bool fresh = h->hst_valid && h->hst_steps == h->steps;
   bool moved = false;
   if (X)
@@ -1097,7 +1098,7 @@ int hlbm_set_owned_planes(hlbm_handle h, int box, int z_lo, int z_hi) {
   bd.own_hi = z_hi;
   CK(cudaMemcpyAsync(h->d_boxes + box, &bd, sizeof(BoxDesc), cudaMemcpyHostToDevice, h->stream));
   CK(cudaStreamSynchronize(h->stream));
-  h->moments_valid = false;  // the recorded interior cells may hold ghost planes
+  h->moments_valid = false;  // the next step takes the link sums, over the new owned planes
   return HLBM_OK;
 }
 
@@ -1516,8 +1517,8 @@ int hlbm_autotune(hlbm_handle h, int nsteps, int* tile_y, int* tile_z, int* cell
   if (cells_x) *cells_x = best.cx;
   if (ms_per_step) *ms_per_step = best.ms;
   if (rc != HLBM_OK) return rc;
-  // the restored state is the one before tuning: its recorded interior
-  // cells are valid for the mode in use then
+  // the restored state is the one before tuning: the form of its next
+  // exchange with it
   h->moments_valid = moments0 && best.mode == HLBM_MEA_MOMENTS && h->mea_mode == HLBM_MEA_MOMENTS;
   {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
