@@ -361,6 +361,8 @@ __device__ __forceinline__ void for_interior(const Rec& R, const BoxDesc& bd, in
     if (GRIDS && R.shape == 4) {
       // Half the candidate cells or more lie outside: the warp collects the
       // inside ones and takes 32 at a time (the sums depend on no order).
+      // 1300 rounded boxes in 224^3: exchange 117 -> 104 us FP32, 108 -> 89
+      // FP16, with the candidates from the interior's capsule.
       int held = 0;  // of found[warp], the same in every lane
       auto take = [&](int n) {
         __syncwarp();

@@ -95,6 +95,44 @@ def test_few_and_many_particles_of_all_shapes(H, O, mode, count):
     _steps_agree(lat, orc, 3)
 
 
+@pytest.mark.parametrize("bc", [0, 7])
+@pytest.mark.parametrize("kind", ["cell", "slab", "rod", "star", "large"])
+def test_grid_particles_of_few_and_many_inside_cells(H, O, kind, bc):
+    """The moments form collects a distance-grid particle's inside cells per
+    warp and takes 32 at a time: from a few cells in all to several hundred a
+    warp, shapes that fill little of the capsule the candidates come from,
+    walls and periodic faces; the cells counted exactly."""
+    from paper_2312_14172_gb300 import workloads
+    grid = {"cell": lambda: workloads.rounded_box_grid((0.8, 0.8, 0.8), 0.3),
+            "slab": lambda: workloads.rounded_box_grid((7.0, 1.2, 6.0), 0.4),
+            "rod": lambda: workloads.rounded_box_grid((1.3, 1.3, 11.0), 0.5),
+            "star": lambda: workloads.superellipsoid_grid((8.0, 8.0, 8.0), power=0.8),
+            "large": lambda: workloads.rounded_box_grid((12.0, 11.0, 13.0), 2.0)}[kind]()
+    n = (66, 63, 64)
+    X = np.array([[20.3, 19.4, 18.2], [49.1, 47.7, 46.6]])
+    if bc == 0 and kind != "large":
+        X = np.concatenate([X, [[0.4, 62.6, 33.2]]])  # across two faces
+    m = len(X)
+    rng = np.random.default_rng(11)
+    q = rng.standard_normal((m, 4))
+    q /= np.linalg.norm(q, axis=1)[:, None]
+    U, om = rng.uniform(-1e-3, 1e-3, (m, 3)), rng.uniform(-1e-3, 1e-3, (m, 3))
+    lat = H.Lattice([n + (bc,)], H.make_params(tau=0.7, eps=1.5, gravity=(1e-6, 0, -1e-5), max_particles=m,
+                                               grid_floats=grid[0].size))
+    orc = O.Oracle(n, 0.7, 1.5, bc, (1e-6, 0, -1e-5))
+    f = _pops(n, 12)
+    for s in (lat, orc):
+        s.add_grid(*grid)
+        s.add_particles([4] * m, [[0.0] * 3] * m, X, U, om, q, np.full(m, 2.0))
+        s.set_populations(f)
+    lat.set_mea_mode("moments")
+    lat.step(1)
+    orc.step(1)
+    want = sum(orc.mea(p)[2] for p in range(m))
+    assert want > 0 and lat.interior_cells() == want
+    _steps_agree(lat, orc, 2)
+
+
 def test_contacts_beyond_one_list_and_one_chunk(H, O):
     """A sphere with 90 neighbours in contact (a warp's list holds 64) among
     300 particles (256 are staged at a time); fluid and particles at rest, so
