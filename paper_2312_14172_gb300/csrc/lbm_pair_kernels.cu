@@ -64,10 +64,13 @@ template <> struct Two<__half> {
 };
 
 // v, which all lanes of the warp hold alike, as a value the compiler may keep
-// once per warp (uniform registers)
-__device__ __forceinline__ int uniform(int v) { return __shfl_sync(__activemask(), v, 0); }
-__device__ __forceinline__ long long uniform(long long v) {
-  return (long long)(((unsigned long long)(unsigned)uniform((int)(v >> 32)) << 32) | (unsigned)uniform((int)v));
+// once per warp (uniform registers).  `lanes` names every lane the warp has,
+// and all of them call it: the shuffle then brings the warp together and lane
+// 0 is there to read from, whatever divergent code came before.
+__device__ __forceinline__ int uniform(unsigned lanes, int v) { return __shfl_sync(lanes, v, 0); }
+__device__ __forceinline__ long long uniform(unsigned lanes, long long v) {
+  return (long long)(((unsigned long long)(unsigned)uniform(lanes, (int)(v >> 32)) << 32) |
+                     (unsigned)uniform(lanes, (int)v));
 }
 
 // mass and momentum of the two cells' values v_i (opposite directions taken
@@ -127,13 +130,15 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
   pdl_wait();
   if (COUPLE) load_candidates<(C > 1)>(a, k, srec, scap, s_rowmask);
 
-  const int z0 = uniform(k.z0), nz = uniform(bd.nz);
+  // a block is whole warps, or 16 threads (sub_y = 1); no thread has left yet
+  const unsigned lanes = blockDim.y == 1 ? 0xffffu : 0xffffffffu;
+  const int z0 = uniform(lanes, k.z0), nz = uniform(lanes, bd.nz);
   const int z1 = min(z0 + a.sub_z, nz);
-  const long long slice_bytes = uniform((long long)bd.ny * bd.ntx * (QVB * (int)sizeof(S)));
-  char* const base = reinterpret_cast<char*>(a.f) + uniform(bd.blk_off * (long long)(QVB * sizeof(S)));
+  const long long slice_bytes = uniform(lanes, (long long)bd.ny * bd.ntx * (QVB * (int)sizeof(S)));
+  char* const base = reinterpret_cast<char*>(a.f) + uniform(lanes, bd.blk_off * (long long)(QVB * sizeof(S)));
   const int x0 = k.x0 + 2 * threadIdx.x;
   const int y = k.y0 + threadIdx.y;
-  if (x0 >= bd.nx || y >= bd.ny) return;
+  const bool here = x0 < bd.nx && y < bd.ny;  // the other lanes leave below
   // an odd nx leaves one cell in a row's last pair: its second slot is the
   // row's padding, computed but never stored, and the cell's right
   // neighbour is x0 + 1 wrapped (rb.dr, rb.wr refer to x0 + 1 there)
@@ -146,7 +151,8 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
   // cell, but few warps hold such cells: they run the slice with the selects,
   // all others without (a warp runs one of the two).
   const bool special = single || (WALLS && (((bd.bc & 2) && (y == 0 || y == bd.ny - 1)) || rb.wl || rb.wr));
-  const bool plain_row = FAST && !__any_sync(__activemask(), special);
+  const bool plain_row = FAST && !__any_sync(lanes, here && special);
+  if (!here) return;
   // Byte offsets within a z slice (below 4 GB, the caller sees to it) of slot 0
   // of x0 in the rows y - 1, y, y + 1, and from there to x0 - 1 and x0 + 2:
   // they hold for every slice, and with the slices' base addresses, which are

@@ -1,0 +1,90 @@
+"""The collision's launch shapes and the handle's timing calls at the edges
+where their kernels or their steps change."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+W = [1 / 3] + [1 / 18] * 6 + [1 / 36] * 12
+
+
+@pytest.fixture(scope="module")
+def H():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_2312_14172_gb300 import build, hlbm
+    build.build()
+    hlbm.load()
+    return hlbm
+
+
+def _fluid(lat, precision):
+    """The handle's populations as stored, [blocks, 19, 32]."""
+    import torch
+    dt, size = (torch.float32, 4) if precision == "fp32" else (torch.float16, 2)
+    blocks = sum(-(-b[0] // 32) * b[1] * b[2] for b in lat.boxes)
+    return lat.buffer[: blocks * 19 * 32 * size].view(dt).view(blocks, 19, 32)
+
+
+def _worst(a, b, nx, precision):
+    """Largest difference of two such tensors of a box of rows of nx cells, in
+    units of the weights; the padding cells of a row's last block hold nothing."""
+    import torch
+    w = torch.tensor(W, device=a.device)[None, :, None] * (1.0 if precision == "fp32" else 2.0 ** 14)
+    last = (nx - 1) // 32
+    worst = 0.0
+    for k in range(last + 1):
+        cells = min(32, nx - 32 * k)
+        d = (a[k::last + 1, :, :cells].float() - b[k::last + 1, :, :cells].float()).abs() / w
+        worst = max(worst, float(d.max()))
+    return worst
+
+
+def _disturb(lat, precision, seed):
+    """Deviations of 1e-3 of the weights in every cell (padding included)."""
+    import torch
+    v = _fluid(lat, precision)
+    g = torch.Generator(device=v.device).manual_seed(seed)
+    w = torch.tensor(W, device=v.device)[None, :, None] * (1.0 if precision == "fp32" else 2.0 ** 14)
+    for part in v.split(1 << 20):
+        part.copy_(1e-3 * w * torch.randn(part.shape, generator=g, device=v.device))
+    torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("precision,n,bc,particles", [
+    ("fp32", (101, 29, 21), 7, 0),       # selects at every wall, a row's single last cell
+    ("fp32", (101, 45, 44), 6, 12),
+    ("fp16", (70, 33, 30), 0, 0),
+    ("fp16", (97, 50, 43), 0, 12),
+    ("fp16", (203, 190, 180), 2, 40),    # above twice the L2: blocks prefetch their rows
+])
+def test_blocks_of_every_height_take_the_same_step(H, precision, n, bc, particles):
+    """16 threads (half a warp) to 128 per block, both parities, particles or
+    none: the same step.  In FP32 the shapes may differ by rounding (1e-6 of
+    the weights); with half storage such a difference can turn a stored value
+    to its neighbour, 2^-10 of a deviation of up to 5e-3, here bounded over
+    the five steps by 2e-5."""
+    import torch
+    from paper_2312_14172_gb300 import workloads
+    rng = np.random.default_rng(5)
+    ref = None
+    for shape in ((8, 8, 2), (1, 2, 2), (1, 8, 2), (2, 4, 2), (4, 1, 2)):
+        lat = H.Lattice([n + (bc,)], H.make_params(tau=0.7, precision=precision, max_particles=max(1, particles)))
+        if particles:
+            if ref is None:
+                w = workloads.nonspherical(n=n, count=particles, tau=0.7, grid=True)
+                P = w["particles"]
+                P["U"] = rng.uniform(-1e-3, 1e-3, P["U"].shape)
+            lat.add_workload_particles(P)
+        _disturb(lat, precision, 7)
+        lat.set_launch(*shape)
+        lat.step(5)
+        lat.sync()
+        got = _fluid(lat, precision).clone()
+        lat.close()
+        if ref is None:
+            ref = got
+            continue
+        assert _worst(ref, got, n[0], precision) <= (1e-6 if precision == "fp32" else 2e-5), shape
+    torch.cuda.empty_cache()
