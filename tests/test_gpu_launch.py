@@ -88,3 +88,31 @@ def test_blocks_of_every_height_take_the_same_step(H, precision, n, bc, particle
             continue
         assert _worst(ref, got, n[0], precision) <= (1e-6 if precision == "fp32" else 2e-5), shape
     torch.cuda.empty_cache()
+
+
+def test_autotune_times_the_steps_alone(H):
+    """The time per step that the autotuner returns (of twelve steps here) is
+    that of the same steps taken again with their graphs there.  Capturing and
+    instantiating the two graphs takes longer than the twelve steps of this box
+    (44 us of host time against 35 us); a quarter is room for the clock."""
+    import torch
+    from paper_2312_14172_gb300 import workloads
+    w = workloads.single_sphere(n=26, radius=4.0)
+    w["particles"] = {k: v[:0] for k, v in w["particles"].items()}
+    lat = H.from_workload(w)
+    lat.step(8)
+    told = lat.autotune(nsteps=3)[3]
+    times = []
+    for _ in range(9):
+        lat.step(2)
+        lat.step(12)
+        torch.cuda.synchronize()
+        lat.step(2)
+        e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        e[0].record(lat.stream)
+        lat.step(12)
+        e[1].record(lat.stream)
+        torch.cuda.synchronize()
+        times.append(e[0].elapsed_time(e[1]) / 12)
+    lat.close()
+    assert told <= 1.25 * np.median(times)
