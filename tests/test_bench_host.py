@@ -129,3 +129,35 @@ def test_clock_sampler_keeps_the_samples_inside_the_timed_window():
     c = s.stop()
     assert c["samples"] == 2 and c["sm_mhz"] == 2035.0 and c["sm_max_mhz"] == 2070.0
     assert c["reasons"] == ["sw_power_cap"] and c["in_window"] and c["source"] == "nvml"
+
+
+def test_warm_up_captures_the_timed_runs_graphs():
+    """After bench.warm_up the run to be timed launches only graphs that were
+    launched before, whatever its length and the warm-up's parity: runs are
+    taken in graphs of 8, 4, 2 and 1 steps per parity of the first step and
+    form of the exchange (the link sums on the first step only)."""
+    class Lat:
+        def __init__(self):
+            self.done, self.seen, self.new = 0, set(), 0
+
+        def step(self, n):
+            self.new = 0
+            while n:
+                k = next(k for k in (8, 4, 2, 1) if k <= n)
+                g = (k, self.done > 0, self.done & 1)
+                self.new += g not in self.seen
+                self.seen.add(g)
+                self.done += k
+                n -= k
+
+        def sync(self):
+            pass
+    for warmup in (3, 4, 5, 10):
+        for steps in list(range(1, 45)) + [200, 999, 1000]:
+            lat = Lat()
+            lat.step(7)  # a tuned handle's steps
+            lat.seen.clear()
+            extra = bench.warm_up(lat, warmup, steps)
+            assert lat.done == 7 + warmup + extra
+            lat.step(steps)
+            assert lat.new == 0, (warmup, steps)
