@@ -281,10 +281,13 @@ int hlbm_get_mea_mode(hlbm_handle h);
  * without timing. */
 int hlbm_autotune(hlbm_handle h, int nsteps, int* tile_y, int* tile_z, int* cells_x, float* ms_per_step);
 
-/* Runs nsteps steps with each kernel launched on its own, bracketed by CUDA
- * events on the handle's stream, and writes the mean time per launch in ms:
- * ms[0] momentum exchange, ms[1] contact (when on), Newton-Euler and work
- * lists, ms[2] collision and streaming.  Synchronises. */
+/* Runs nsteps steps, the kernels of hlbm_step each launched on its own and
+ * bracketed by CUDA events on the handle's stream, and writes the mean times
+ * per step in ms: ms[0] momentum exchange, with the motion and the work lists
+ * where it moves the particles itself (fewer than four particles per SM);
+ * ms[1] contact (when on) and the update kernel (Newton-Euler and work lists,
+ * otherwise), 0 when neither is launched; ms[2] collision and streaming.
+ * Synchronises. */
 int hlbm_kernel_times(hlbm_handle h, int nsteps, float ms[3]);
 
 /* Writes to *n the number of (cell, particle) pairs whose cell centre lies

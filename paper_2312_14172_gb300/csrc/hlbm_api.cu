@@ -1551,33 +1551,38 @@ int hlbm_autotune(hlbm_handle h, int nsteps, int* tile_y, int* tile_z, int* cell
 int hlbm_kernel_times(hlbm_handle h, int nsteps, float ms[3]) {
   if (!h || !ms) return HLBM_ERR_ARG;
   if (nsteps < 1) return fail(h, HLBM_ERR_ARG, "nsteps < 1");
-  cudaEvent_t ev[4];
-  for (int k = 0; k < 4; ++k) CK(cudaEventCreate(&ev[k]));
+  // the launches of a step, an event before and after each: contact (when
+  // on), exchange, update (unless the exchange moves the particles), collision
+  constexpr int KINDS = 4, OF[KINDS] = {1, 0, 1, 2};  // their place in ms
+  cudaEvent_t ev[KINDS + 1];
+  for (cudaEvent_t& e : ev) CK(cudaEventCreate(&e));
   double acc[3] = {0, 0, 0};
   int rc = HLBM_OK;
   for (int s = 0; s < nsteps; ++s) {
     const int parity = (int)(h->steps & 1);
     const bool moments = h->moments_valid && h->np > 0;
     PartArgs pa = part_args(h, parity, moments);
+    pa.move = h->fused;
+    const bool on[KINDS] = {h->np > 0 && h->contact_k > 0.0, h->np > 0, h->np > 0 && !h->fused, true};
     cudaEventRecord(ev[0], h->stream);
-    if (h->np > 0) launch_mea(pa, h->prm.precision, parity, h->walls, moments, h->stream);
-    cudaEventRecord(ev[1], h->stream);
-    if (h->np > 0) launch_contact(pa, h->stream);
-    if (h->np > 0) launch_update(pa, h->stream);
-    cudaEventRecord(ev[2], h->stream);
-    launch_collide(lbm_args(h, parity), h->prm.precision, parity, h->walls, h->np > 0, h->stream);
-    cudaEventRecord(ev[3], h->stream);
-    const cudaError_t e = cudaEventSynchronize(ev[3]);
+    for (int k = 0; k < KINDS; ++k) {
+      if (on[k] && k == 0) launch_contact(pa, h->stream);
+      if (on[k] && k == 1) launch_mea(pa, h->prm.precision, parity, h->walls, moments, h->stream);
+      if (on[k] && k == 2) launch_update(pa, h->stream);
+      if (on[k] && k == 3) launch_collide(lbm_args(h, parity), h->prm.precision, parity, h->walls, h->np > 0, h->stream);
+      cudaEventRecord(ev[k + 1], h->stream);
+    }
+    const cudaError_t e = cudaEventSynchronize(ev[KINDS]);
     if (e != cudaSuccess) { rc = fail(h, HLBM_ERR_CUDA, std::string("kernel timing: ") + cudaGetErrorString(e)); break; }
-    for (int k = 0; k < 3; ++k) {
+    for (int k = 0; k < KINDS; ++k) {
       float t = 0.f;
-      cudaEventElapsedTime(&t, ev[k], ev[k + 1]);
-      acc[k] += t;
+      if (on[k]) cudaEventElapsedTime(&t, ev[k], ev[k + 1]);
+      acc[OF[k]] += t;
     }
     h->steps += 1;
     h->moments_valid = h->mea_mode == HLBM_MEA_MOMENTS;
   }
-  for (int k = 0; k < 4; ++k) cudaEventDestroy(ev[k]);
+  for (cudaEvent_t& e : ev) cudaEventDestroy(e);
   if (rc != HLBM_OK) return rc;
   for (int k = 0; k < 3; ++k) ms[k] = (float)(acc[k] / nsteps);
   return read_status(h);

@@ -116,3 +116,36 @@ def test_autotune_times_the_steps_alone(H):
         times.append(e[0].elapsed_time(e[1]) / 12)
     lat.close()
     assert told <= 1.25 * np.median(times)
+
+
+@pytest.mark.parametrize("contact", [False, True])
+@pytest.mark.parametrize("count", [12, 700])
+def test_kernel_times_are_those_of_a_steps_kernels(H, count, contact):
+    """hlbm_kernel_times launches what hlbm_step launches: the run it leaves
+    is that of as many steps, bit for bit, and where the exchange moves few
+    particles itself there is no update kernel to time."""
+    rng = np.random.default_rng(3)
+    n = (100, 90, 80)
+    site = rng.permutation(10 * 9 * 8)[:count]
+    X = np.stack([site % 10, site // 10 % 9, site // 90], 1) * 10.0 + rng.uniform(4.0, 6.0, (count, 3))
+    U = rng.uniform(-1e-3, 1e-3, (count, 3))
+    lats = []
+    for _ in range(2):
+        lat = H.Lattice([n + (0,)], H.make_params(tau=0.7, gravity=(0, 0, -1e-5), max_particles=count))
+        lat.add_particles(np.zeros(count, int), np.full((count, 1), 3.0), X, U, U, None, np.full(count, 2.0))
+        lat.set_mea_mode("moments")
+        if contact:
+            lat.set_contact(1e-3, 3.0)
+        lat.step(2)
+        lats.append(lat)
+    a, b = lats
+    t = a.kernel_times(3)
+    b.step(3)
+    sa, sb = a.particle_state(), b.particle_state()
+    for k in sa:
+        assert np.array_equal(sa[k], sb[k]), k
+    assert np.array_equal(a.populations(), b.populations())
+    assert t["mea"] > 0.0 and t["collide_stream"] > 0.0
+    assert (t["update"] > 0.0) == (contact or count == 700)
+    a.close()
+    b.close()
