@@ -224,13 +224,6 @@ static int fail(hlbm_ctx* h, int code, const std::string& msg) {
   return code;
 }
 
-// cells per thread as launched: with half storage or walls the two-cell
-// kernel addresses a z slice with 32-bit offsets, and lattices of larger
-// slices run the one-cell kernel
-static int run_cells_x(const hlbm_ctx* h) {
-  return h->wide_slices && (h->walls || h->prm.precision == HLBM_FP16) ? 1 : h->cells_x;
-}
-
 static LbmArgs lbm_args(const hlbm_ctx* h, int parity) {
   LbmArgs a{};
   a.nsm = h->nsm;
@@ -239,10 +232,11 @@ static LbmArgs lbm_args(const hlbm_ctx* h, int parity) {
   a.nboxes = (int)h->boxes.size();
   a.sub_y = h->sub_y;
   a.sub_z = h->sub_z;
-  a.cells_x = run_cells_x(h);
+  a.cells_x = h->cells_x;
   a.nsub = (TILE_Y / h->sub_y) * (TILE_Z / h->sub_z);
   a.nbricks = h->L.ntiles * a.nsub;
   a.reverse = parity && h->reverse_odd;
+  a.wide = h->wide_slices;
   a.prefetch = std::min(h->prefetch, h->sub_y * h->sub_z);
   a.omega = (float)(1.0 / h->prm.tau);
   for (int j = 0; j < 3; ++j) a.ff[j] = (float)h->prm.fluid_force[j];
@@ -280,7 +274,7 @@ static PartArgs part_args(const hlbm_ctx* h, int parity, bool moments = false) {
   a.nchunks = h->nchunks[moments];
   a.mea_threads = h->mea_threads[moments];
   a.mea_group = h->mea_group;
-  a.cells_x = run_cells_x(h);
+  a.cells_x = h->cells_x;
   a.partial = h->partial;
   a.done = h->done;
   a.acc = h->acc;

@@ -100,8 +100,8 @@ template <typename S>
 struct PairBlocks { static constexpr int value = sizeof(S) == 4 ? HLBM_CP_MINBLOCKS_F32 : HLBM_CP_MINBLOCKS_F16; };
 
 // C: 0 no particles, 1 particles of the analytic shapes, 2 with distance
-// grids among them
-template <typename S, int PAR, bool WALLS, int C>
+// grids among them.  WIDE: a z slice of some box takes 4 GB or more (odd steps)
+template <typename S, int PAR, bool WALLS, int C, bool WIDE>
 __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel(LbmArgs a) {
   constexpr bool COUPLE = C > 0;
   // Odd steps address the neighbour rows by 32-bit offsets (below): a tenth
@@ -110,8 +110,15 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
   // FP16 432 -> 388) and where walls add to them (128^3 FP32 61.5 -> 57.1).
   // FP32 without walls waits for HBM instead, and there the pointer form's
   // slower stream of requests is the faster one (non-spherical 256^3 FP32 452
-  // against 465); an even step touches its own cells only.
-  constexpr bool FAST = PAR == 1 && (sizeof(S) == 2 || WALLS);
+  // against 465); an even step touches its own cells only.  Offsets within a
+  // wider slice take 64 bits, and so the pointer form; as kernels of their own
+  // those cost the others nothing (a branch between the forms spills a hundred
+  // bytes of registers in the kernels without particles).  Boxes of rows of
+  // 8192 (FP32) or 16384 cells in 6 slices, ms a step, one cell per thread /
+  // pointers (6900 rows a slice, above 4 GB) / offsets (6898): FP32 with walls
+  // 8.82 / 7.83 / 7.74, FP16 12.12 / 10.50 / 10.73, with walls 15.28 / 11.82 /
+  // 11.12.
+  constexpr bool FAST = PAR == 1 && !WIDE && (sizeof(S) == 2 || WALLS);
   using T = Two<S>;
   __shared__ Rec srec[COUPLE ? MAX_CAND : 1];
   __shared__ Capsule scap[C == 1 ? MAX_CAND : 1];
@@ -151,9 +158,9 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
   // cell, but few warps hold such cells: they run the slice with the selects,
   // all others without (a warp runs one of the two).
   const bool special = single || (WALLS && (((bd.bc & 2) && (y == 0 || y == bd.ny - 1)) || rb.wl || rb.wr));
-  const bool plain_row = FAST && !__any_sync(lanes, here && special);
+  const bool plain_row = (FAST || (WIDE && WALLS)) && !__any_sync(lanes, here && special);
   if (!here) return;
-  // Byte offsets within a z slice (below 4 GB, the caller sees to it) of slot 0
+  // Byte offsets within a z slice (below 4 GB unless WIDE) of slot 0
   // of x0 in the rows y - 1, y, y + 1, and from there to x0 - 1 and x0 + 2:
   // they hold for every slice, and with the slices' base addresses, which are
   // the same for the whole warp, address the slots in few instructions.
@@ -161,9 +168,11 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
 #pragma unroll
   for (int j = 0; j < 3; ++j) ro[j] = ((unsigned)(max(rb.yb[j], 0) + rb.xb) * QVB + rb.xin) * (unsigned)sizeof(S);
   const unsigned dl = (unsigned)(rb.dl * (int)sizeof(S)), dr = (unsigned)(rb.dr * (int)sizeof(S));
-  auto slice = [&](auto ptag, int z) {
+  // PLAIN: by those offsets; otherwise by pointers, with the selects of walls
+  // where W
+  auto slice = [&](auto ptag, auto wtag, int z) {
     constexpr bool PLAIN = decltype(ptag)::value;
-    constexpr bool W = WALLS && !PLAIN;
+    constexpr bool W = decltype(wtag)::value;
     int zb[3];
     slice_blocks<W>(bd, z, zb);
     S* const own = cell_ptr(f, zb[1] + rb.yb[1] + rb.xb, rb.xin);  // slot 0 of cell x0
@@ -316,27 +325,29 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
   // one z slice at a time: an unrolled loop would hold two slices' arrivals
 #pragma unroll 1
   for (int z = z0; z < z1; ++z) {
-    if (FAST && (plain_row && !(WALLS && (bd.bc & 4) && (z == 0 || z == nz - 1))))
-      slice(std::integral_constant<bool, true>{}, z);
-    else
-      slice(std::integral_constant<bool, false>{}, z);
+    const bool plain = plain_row && !(WALLS && (bd.bc & 4) && (z == 0 || z == nz - 1));
+    if (FAST && plain) slice(std::true_type{}, std::false_type{}, z);
+    else if (WIDE && plain) slice(std::false_type{}, std::false_type{}, z);
+    else slice(std::false_type{}, std::integral_constant<bool, WALLS>{}, z);
   }
   if (!early) pdl_trigger();
 }
 
-template <typename S, int PAR, bool W, int C>
+template <typename S, int PAR, bool W, int C, bool WIDE = false>
 static cudaError_t launch_cp(const LbmArgs& a, cudaStream_t s) {
   dim3 block(TILE_X / 2, a.sub_y);
   LbmArgs b = a;
   // resident blocks per SM as the launch bounds provide for (registers)
   b.pdl_tail = a.nsm > 0 ? (long long)a.nsm * (PairBlocks<S>::value * 128 / (int)(block.x * block.y))
                          : a.nbricks;
-  return launch_k(collide_pair_kernel<S, PAR, W, C>, dim3((unsigned)a.nbricks), block, 0, s, a.pdl != 0, b);
+  return launch_k(collide_pair_kernel<S, PAR, W, C, WIDE>, dim3((unsigned)a.nbricks), block, 0, s, a.pdl != 0, b);
 }
 
 template <typename S, int C>
 static cudaError_t launch_cp_c(const LbmArgs& a, int parity, bool walls, cudaStream_t s) {
   if (parity == 0) return launch_cp<S, 0, false, C>(a, s);
+  if (a.wide && walls) return launch_cp<S, 1, true, C, true>(a, s);
+  if (a.wide && sizeof(S) == 2) return launch_cp<S, 1, false, C, sizeof(S) == 2>(a, s);
   return walls ? launch_cp<S, 1, true, C>(a, s) : launch_cp<S, 1, false, C>(a, s);
 }
 

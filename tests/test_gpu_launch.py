@@ -149,3 +149,33 @@ def test_kernel_times_are_those_of_a_steps_kernels(H, count, contact):
     assert (t["update"] > 0.0) == (contact or count == 700)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("precision,nx,bc", [("fp32", 8192, 6), ("fp16", 16384, 0), ("fp16", 16384, 7)])
+@pytest.mark.parametrize("ny,nz,particles", [(6898, 3, 0), (6900, 3, 0), (6898, 7, 2), (6900, 7, 2)])
+def test_slices_on_both_sides_of_four_gigabytes(H, precision, nx, bc, ny, nz, particles):
+    """A z slice of 6898 such rows ends just below 2^32 bytes, one of 6900 just
+    above: odd steps address the one by 32-bit offsets, the other by pointers.
+    Both take the step of the one-cell kernel up to rounding (as above, three
+    steps) and not its very bits, which would mean that it ran instead.  Without
+    particles, and with one at either end of the slices."""
+    import torch
+    assert (ny * (nx // 32) * 19 * 32 * (4 if precision == "fp32" else 2) > 2 ** 32) == (ny == 6900)
+    got = []
+    for cells_x in (2, 1):
+        lat = H.Lattice([(nx, ny, nz, bc)], H.make_params(tau=0.7, precision=precision, max_particles=2))
+        _disturb(lat, precision, 9)
+        if particles:
+            lat.add_particles([0, 0], [[1.0] * 3] * 2, [[4.3, 2.2, 3.1], [nx - 5.4, ny - 3.3, 3.4]],
+                              U=[[1e-3, 2e-3, -1e-3]] * 2, omega=[[1e-3, 0.0, 2e-3]] * 2, rho_p=[2.0, 2.0])
+        lat.set_launch(4, 2, cells_x)
+        assert lat.get_launch() == (4, 2, cells_x)
+        lat.step(3)
+        lat.sync()
+        got.append(_fluid(lat, precision).clone())
+        lat.close()
+        del lat
+    assert _worst(*got, nx, precision) <= (1e-6 if precision == "fp32" else 2e-5)
+    assert not torch.equal(*got)
+    del got
+    torch.cuda.empty_cache()
