@@ -211,3 +211,40 @@ def test_snapshot_of_the_version_before_loads(H):
         c.close()
     a.close()
     b.close()
+
+
+def test_particles_added_one_at_a_time(H):
+    """The run is that of particles added at once, bit for bit, and adding one
+    costs the same in a lattice of half a million bin tiles as in one of 64
+    (copies and a synchronisation, about 95 us): at most twice, the shortest
+    call of each."""
+    import time
+    n, count = (96, 80, 72), 60
+    rng = np.random.default_rng(8)
+    site = rng.permutation(8 * 7 * 6)[:count]
+    X = np.stack([site % 8, site // 8 % 7, site // 56], 1) * 11.0 + rng.uniform(5.0, 7.0, (count, 3))
+    a = rng.uniform(1.5, 4.0, (count, 1))
+    params = H.make_params(tau=0.7, gravity=(0, 0, -1e-5), max_particles=count)
+    one, all_ = H.Lattice([n + (0,)], params), H.Lattice([n + (0,)], params)
+    all_.add_particles([0] * count, a, X, rho_p=[2.0] * count)
+    for k in range(count):
+        one.add_particles([0], a[k:k + 1], X[k:k + 1], rho_p=[2.0])
+    one.step(4)
+    all_.step(4)
+    assert np.array_equal(one.populations(), all_.populations())
+    s1, s2 = one.particle_state(), all_.particle_state()
+    for k in s1:
+        assert np.array_equal(s1[k], s2[k]), k
+    one.close()
+    all_.close()
+    shortest = []
+    for n in ((128, 64, 32), (1024, 1024, 1024)):
+        lat = H.Lattice([n + (0,)], H.make_params(tau=0.7, precision="fp16", max_particles=count))
+        took = []
+        for k in range(count):
+            t0 = time.perf_counter()
+            lat.add_particles([0], [[2.0] * 3], [[2.0 * k, 9.0, 9.0]], rho_p=[2.0])
+            took.append(time.perf_counter() - t0)
+        shortest.append(min(took))
+        lat.close()
+    assert shortest[1] <= 2.0 * shortest[0]
