@@ -1776,8 +1776,11 @@ int hlbm_load(hlbm_handle h, const void* buf, size_t bytes) {
   if (hd.moments_valid && std::memcmp(hd.magic, CK_MAGIC_OLD, 8) == 0) {
     int32_t cnt[OLD_STRIPES];
     if (!get(cnt, sizeof(cnt))) return fail(h, HLBM_ERR_ARG, "truncated snapshot");
+    // a stripe held 1/64 of half the cells, or two entries per cell of a tile
+    const long long room = std::max((h->L.ncell / 2 + OLD_STRIPES - 1) / OLD_STRIPES, 2LL * TILE_X * TILE_Y * TILE_Z);
     for (int k = 0; k < OLD_STRIPES; ++k) {
-      if (cnt[k] < 0 || h->L.cap == 0) return fail(h, HLBM_ERR_ARG, "snapshot's interior-cell list does not fit this handle");
+      if (cnt[k] < 0 || cnt[k] > room || h->L.cap == 0)
+        return fail(h, HLBM_ERR_ARG, "snapshot's interior-cell list does not fit this handle");
       const size_t nb = (sizeof(int2) + sizeof(float4)) * (size_t)cnt[k];
       if ((size_t)(end - i) < nb) return fail(h, HLBM_ERR_ARG, "truncated snapshot");
       i += nb;

@@ -131,3 +131,34 @@ def test_snapshots_that_do_not_fit_are_refused(H):
     assert np.max(np.abs(a.populations() - b.populations()) / a.populations()) <= 1e-6
     a.close()
     b.close()
+
+
+def test_earlier_snapshots_with_an_impossible_list_are_refused(H):
+    """HLBMCKP3: a stripe of its list of interior cells held 1/64 of half the
+    cells, at least 4096; a larger count was refused then and is refused now."""
+    n = (40, 30, 33)
+
+    def fresh():
+        return H.Lattice([n + (0,)], H.make_params(tau=0.7, max_particles=1))
+    a = fresh()
+    a.add_particles([0], [[3.0] * 3], [[20.0, 15.0, 16.0]], rho_p=[2.0])
+    a.set_mea_mode("moments")
+    a.step(2)
+    snap = a.save()
+    pops = 33 * 30 * 2 * 19 * 32 * 4
+    for entries in (4096, 4097):
+        counts = np.zeros(64, np.int32)
+        counts[5] = entries
+        old = b"HLBMCKP3" + snap[8:-pops] + counts.tobytes() + bytes(24 * entries) + snap[-pops:]
+        b = fresh()
+        if entries == 4096:
+            b.load_snapshot(old)
+            b.step(1)
+            a.step(1)
+            assert np.array_equal(a.populations(), b.populations())
+        else:
+            with pytest.raises(H.HLBMError) as e:
+                b.load_snapshot(old)
+            assert e.value.code == H.HLBM_ERR_ARG
+        b.close()
+    a.close()
