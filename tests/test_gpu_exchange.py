@@ -248,3 +248,80 @@ def test_particles_added_one_at_a_time(H):
         shortest.append(min(took))
         lat.close()
     assert shortest[1] <= 2.0 * shortest[0]
+
+
+def _all_shapes(count, n, contact_gap):
+    """Spheres, ellipsoids, cuboids, capsules and grid particles on displaced
+    sites of a box, spinning, with uneven principal moments."""
+    rng = np.random.default_rng(count + contact_gap)
+    pitch = 8
+    k = [v // pitch for v in n]
+    site = rng.permutation(k[0] * k[1] * k[2])[:count]
+    X = np.stack([site % k[0], site // k[0] % k[1], site // (k[0] * k[1])], 1) * float(pitch) + \
+        rng.uniform(3.6, 4.4, (count, 3))
+    shape = np.arange(count) % 5
+    a = rng.uniform(1.4, 2.6, (count, 3))
+    a[shape == 2] *= 0.8
+    a[shape == 3] = (1.4, 1.4, 1.2)
+    a[shape == 4] = 0.0  # names grid 0
+    q = rng.standard_normal((count, 4))
+    q /= np.linalg.norm(q, axis=1)[:, None]
+    return shape, a, X, rng.uniform(-2e-3, 2e-3, (count, 3)), rng.uniform(-4e-3, 4e-3, (count, 3)), q
+
+
+@pytest.mark.parametrize("mode", ["kernel", "moments"])
+@pytest.mark.parametrize("bc,contact", [(0, False), (7, True)])
+@pytest.mark.parametrize("count", [45, 700])
+def test_both_movers_take_the_same_step(H, O, count, bc, contact, mode):
+    """Few particles are moved by the exchange's blocks, many (and those of a
+    split step) by the update kernel: bit for bit the same motion, for every
+    shape, between walls and in contact.  Against the oracle: a force within
+    1e-5 of the largest (as above) leaves U of a particle within that over its
+    mass after each step, omega within the same of the torque over its least
+    principal moment (at least 2/5 m a_min^2); X and the quaternion add up
+    three such errors."""
+    from paper_2312_14172_gb300 import workloads
+    n = (88, 80, 72)
+    grid = workloads.rounded_box_grid((1.6, 1.2, 2.0), 0.4)
+    shape, a, X, U, om, q = _all_shapes(count, n, contact)
+    lats = []
+    for _ in range(2):
+        lat = H.Lattice([n + (bc,)], H.make_params(tau=0.7, gravity=(1e-6, 0, -1e-5), max_particles=count,
+                                                   grid_floats=grid[0].size))
+        lats.append(lat)
+    orc = O.Oracle(n, 0.7, 0.5, bc, (1e-6, 0, -1e-5))
+    f = _pops(n, 21)
+    for s in lats + [orc]:
+        s.add_grid(*grid)
+        s.add_particles(shape, a, X, U, om, q, np.full(count, 2.0))
+        s.set_populations(f)
+        if contact:
+            s.set_contact(1e-3, 1.5)
+    for lat in lats:
+        lat.set_mea_mode(mode)
+    one, split = lats
+    largest = {"F": 0.0, "T": 0.0}
+    for _ in range(3):
+        one.step(1)
+        split.step_with_forces(*split.step_forces())
+        orc.step(1)
+        st = orc.particle_state()
+        largest = {k: max(v, np.abs(st[k]).max()) for k, v in largest.items()}
+    s1, s2, so = one.particle_state(), split.particle_state(), orc.particle_state()
+    for k in s1:
+        assert np.array_equal(s1[k], s2[k]), k
+    assert np.array_equal(one.populations(), split.populations())
+    box = {k: v[shape != 4] for k, v in (("shape", shape), ("a", a))}
+    mass, amin = np.full(count, 2.0 * 8 * 1.6 * 1.2 * 2.0 * 0.8), np.full(count, 1.2)
+    mass[shape != 4] = 2.0 * workloads.particle_volumes(box)
+    amin[shape != 4] = box["a"].min(axis=1)
+    dU = 3e-5 * largest["F"] / mass[:, None]
+    dW = 3e-5 * largest["T"] / (0.4 * mass * amin ** 2)[:, None]
+    L = np.array(n, float)
+    for k, bound in (("U", dU), ("omega", dW), ("X", 3 * dU), ("quat", 3 * dW)):
+        d = s1[k] - so[k]
+        if k == "X":
+            d -= L * np.round(d / L)
+        assert np.all(np.abs(d) <= bound + 1e-14), k
+    one.close()
+    split.close()
