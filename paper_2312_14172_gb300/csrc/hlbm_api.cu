@@ -180,8 +180,7 @@ struct hlbm_ctx {
   long long steps = 0;
   int sub_y = 4, sub_z = 2;  // bricks of the collision (default_launch, until hlbm_set_launch)
   bool launch_set = false;
-  int cells_x = 1;       // cells per thread along x
-  bool pair_ok = false;  // the two-cell kernel may run
+  int cells_x = 2;       // cells per thread along x
   bool wide_slices = false;  // a z slice of some box takes 4 GB or more
   // captured steps [steps per graph][moments form in the first][parity], built
   // when a run first asks for them
@@ -189,7 +188,7 @@ struct hlbm_ctx {
   // the last collision knew this particle state, so in the moments mode the
   // momentum exchange takes the moments form
   bool moments_valid = false;
-  int split = 0;  // a split step is open: 1 after its bounding-box exchange, 2 after its moments one
+  bool split = false;  // a split step is open
   // hstage holds the device's particle rows X .. T as downloaded by
   // hlbm_particle_state after step hst_steps (until an upload reuses it)
   bool hst_valid = false;
@@ -443,13 +442,11 @@ int hlbm_init_batch(hlbm_handle* out, int nboxes, const hlbm_box* boxes, const h
   h->prm = *prm;
   if (h->prm.bin_capacity == 0) h->prm.bin_capacity = DEFAULT_BIN_CAP;
   h->stream = (cudaStream_t)cuda_stream;
-  h->pair_ok = true;  // any nx: an odd nx leaves one cell in a row's last pair
   for (int b = 0; b < nboxes; ++b) {
     h->walls |= boxes[b].bc_flags != 0;
     const BoxDesc& d = h->boxes[b];
     h->wide_slices |= (unsigned long long)d.ny * d.ntx * QVB * (prm->precision == HLBM_FP32 ? 4 : 2) > 0xffffffffULL;
   }
-  h->cells_x = 2;
   cudaError_t e;
   if (device_buf) {
     if (((uintptr_t)device_buf % ALIGN) || device_buf_bytes < h->L.total) {
@@ -1148,7 +1145,7 @@ int hlbm_step_forces(hlbm_handle h, double* F, double* T) {
   if (n > 0 && (!F || !T)) return fail(h, HLBM_ERR_ARG, "NULL force or torque array");
   const int parity = (int)(h->steps & 1);
   if (n == 0) {
-    h->split = 1;
+    h->split = true;
     return HLBM_OK;
   }
   const bool moments = h->moments_valid;
@@ -1165,7 +1162,7 @@ int hlbm_step_forces(hlbm_handle h, double* F, double* T) {
         T[3 * k + j] = rows[(size_t)(3 + j) * n + k];
       }
   }
-  h->split = moments ? 2 : 1;
+  h->split = true;
   return HLBM_OK;
 }
 
@@ -1192,7 +1189,7 @@ int hlbm_step_with_forces(hlbm_handle h, const double* F, const double* T) {
   }
   CK(launch_collide(lbm_args(h, parity), h->prm.precision, parity, h->walls, n > 0, h->stream));
   CK(cudaStreamSynchronize(h->stream));  // the host rows above are released
-  h->split = 0;
+  h->split = false;
   h->steps += 1;
   h->moments_valid = h->mea_mode == HLBM_MEA_MOMENTS;
   h->hst_valid = false;
@@ -1333,7 +1330,6 @@ int hlbm_set_launch(hlbm_handle h, int tile_y, int tile_z, int cells_x) {
   auto ok = [](int v) { return v == 1 || v == 2 || v == 4 || v == 8; };
   if (!ok(tile_y) || !ok(tile_z)) return fail(h, HLBM_ERR_ARG, "tile_y and tile_z must be 1, 2, 4 or 8");
   if (cells_x != 1 && cells_x != 2) return fail(h, HLBM_ERR_ARG, "cells_x must be 1 or 2");
-  if (cells_x == 2 && !h->pair_ok) return fail(h, HLBM_ERR_ARG, "cells_x = 2 is not available");
   h->launch_set = true;
   if (tile_y != h->sub_y || tile_z != h->sub_z || cells_x != h->cells_x) {
     h->sub_y = tile_y;
@@ -1397,7 +1393,7 @@ int hlbm_get_launch(hlbm_handle h, int* tile_y, int* tile_z, int* cells_x) {
 namespace {
 // choices of hlbm_autotune per (device, boxes, precision, particle count),
 // kept for the life of the process
-struct TuneChoice { int ty, tz, cx, mode; float ms; };
+struct TuneChoice { int ty, tz, cx; float ms; };
 std::mutex g_tune_mutex;
 std::map<std::string, TuneChoice> g_tune_cache;
 
@@ -1422,13 +1418,19 @@ int hlbm_autotune(hlbm_handle h, int nsteps, int* tile_y, int* tile_z, int* cell
   if (!h) return HLBM_ERR_ARG;
   if (nsteps < 1) return fail(h, HLBM_ERR_ARG, "nsteps < 1");
   if (h->split) return fail(h, HLBM_ERR_STATE, "a split step is open");
+  // the moments form of the exchange walks the same cells as the link sums
+  // without their fixed order: it is the faster mode at every size (us a step,
+  // moments / link sums: one sphere in 48^3 14.5 / 15.7, 200 spheres in 128^3
+  // FP16 57.9 / 68.0, 230 ellipsoids and cuboids there 73.2 / 88.5, 12 grid
+  // particles in 72^3 33.2 / 33.4, 1300 in 224^3 456 / 530)
+  const int mode = h->np > 0 ? HLBM_MEA_MOMENTS : HLBM_MEA_KERNEL;
   const std::string key = tune_key(h);
   {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     auto it = g_tune_cache.find(key);
     if (it != g_tune_cache.end()) {
       const TuneChoice c = it->second;
-      int r = hlbm_set_mea_mode(h, c.mode);
+      int r = hlbm_set_mea_mode(h, mode);
       if (r == HLBM_OK) r = hlbm_set_launch(h, c.ty, c.tz, c.cx);
       if (r != HLBM_OK) return r;
       if (tile_y) *tile_y = c.ty;
@@ -1472,25 +1474,20 @@ int hlbm_autotune(hlbm_handle h, int nsteps, int* tile_y, int* tile_z, int* cell
     restore();
     return fail(h, HLBM_ERR_CUDA, "autotune: cudaEventCreate failed");
   }
-  struct Cand { int ty, tz, cx, mode; float ms; };
+  struct Cand { int ty, tz, cx; float ms; };
   std::vector<Cand> cand;
   const int vals[4] = {1, 2, 4, 8};
-  // the moments form of the exchange walks the same cells as the link sums
-  // without their fixed order: it is the faster mode at every size (us: one
-  // sphere 9.7 / 11.7, 200 spheres FP16 21.5 / 31.5, 50 000 958 / 1484)
-  const int mode = h->np > 0 ? HLBM_MEA_MOMENTS : HLBM_MEA_KERNEL;
-  const int nkinds = h->pair_ok ? 2 : 1;
-  for (int im = 0; im < nkinds * 16; ++im) {
+  for (int im = 0; im < 2 * 16; ++im) {
     const int kind = im / 16, iy = (im / 4) % 4, iz = im % 4;
     if (kind == 1 && vals[iy] == 1) continue;  // 16-thread blocks leave half of each warp idle
-    cand.push_back({vals[iy], vals[iz], kind + 1, mode, 0.f});
+    cand.push_back({vals[iy], vals[iz], kind + 1, 0.f});
   }
   int rc = HLBM_OK;
   // steps per timing: about 20 ms, between nsteps and 4 nsteps (tuning
   // advances the state; long runs would let particles settle and overlap)
   int n = nsteps;
   auto time_one = [&](Cand& c) -> int {
-    int r = hlbm_set_mea_mode(h, c.mode);
+    int r = hlbm_set_mea_mode(h, mode);
     if (r == HLBM_OK) r = hlbm_set_launch(h, c.ty, c.tz, c.cx);
     if (r == HLBM_OK) r = hlbm_step(h, 2);  // warm-up
     // the graphs of the timed steps are captured and uploaded before, not
@@ -1540,7 +1537,7 @@ int hlbm_autotune(hlbm_handle h, int nsteps, int* tile_y, int* tile_z, int* cell
   if (rrc != HLBM_OK) return rrc;
   const Cand best = *std::min_element(cand.begin(), cand.end(),
                                       [](const Cand& x, const Cand& y) { return x.ms < y.ms; });
-  rc = hlbm_set_mea_mode(h, best.mode);
+  rc = hlbm_set_mea_mode(h, mode);
   if (rc == HLBM_OK) rc = hlbm_set_launch(h, best.ty, best.tz, best.cx);
   if (tile_y) *tile_y = best.ty;
   if (tile_z) *tile_z = best.tz;
@@ -1549,10 +1546,10 @@ int hlbm_autotune(hlbm_handle h, int nsteps, int* tile_y, int* tile_z, int* cell
   if (rc != HLBM_OK) return rc;
   // the restored state is the one before tuning: the form of its next
   // exchange with it
-  h->moments_valid = moments0 && best.mode == HLBM_MEA_MOMENTS && h->mea_mode == HLBM_MEA_MOMENTS;
+  h->moments_valid = moments0 && h->mea_mode == HLBM_MEA_MOMENTS;
   {
     std::lock_guard<std::mutex> lock(g_tune_mutex);
-    g_tune_cache[key] = TuneChoice{best.ty, best.tz, best.cx, best.mode, best.ms};
+    g_tune_cache[key] = TuneChoice{best.ty, best.tz, best.cx, best.ms};
   }
   return HLBM_OK;
 }

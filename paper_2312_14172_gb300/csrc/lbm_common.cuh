@@ -17,9 +17,6 @@ template <> struct Pop<float> {
   static __device__ __forceinline__ void st(float* p, float v, float) { *p = v; }
   static __device__ __forceinline__ float ld_raw(const float* p) { return *p; }
   static __device__ __forceinline__ void st_raw(float* p, float v) { *p = v; }
-  // two adjacent cells (8-byte aligned)
-  static __device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
-  static __device__ __forceinline__ void st2(float* p, float2 v) { *reinterpret_cast<float2*>(p) = v; }
 };
 template <> struct Pop<__half> {
   static __device__ __forceinline__ float ld(const __half* p, float inv_s) {
@@ -30,14 +27,8 @@ template <> struct Pop<__half> {
   static constexpr bool SCALED = true;
   static __device__ __forceinline__ float ld_raw(const __half* p) { return __half2float(*p); }
   static __device__ __forceinline__ void st_raw(__half* p, float v) { *p = __float2half_rn(v); }
-  // two adjacent cells (4-byte aligned)
-  static __device__ __forceinline__ float2 ld2(const __half* p) {
-    return __half22float2(*reinterpret_cast<const __half2*>(p));
-  }
-  static __device__ __forceinline__ void st2(__half* p, float2 v) {
-    *reinterpret_cast<__half2*>(p) = __float22half2_rn(v);
-  }
 };
+
 // Addressing of a thread's cells x .. x + n - 1 (one row, one storage block)
 // for the collide-and-stream: the rows y - 1, y, y + 1 as block offsets, and
 // the x neighbours left of the first and right of the last cell as element
