@@ -170,12 +170,12 @@ int hlbm_add_particles(hlbm_handle h, int n, const int* box_id, const int* shape
  * NULL to keep that field).  Arrays as in hlbm_add_particles.  The values are
  * checked and staged on the host, the upload is queued on the stream and the
  * call returns without waiting for it: the arrays may be reused at once.
- * A new position or orientation changes the cells inside the particles, so
- * the next step takes the link sums of the momentum exchange; positions (and the
+ * After a new position or orientation the next step takes the link sums of
+ * the momentum exchange, as after every change of state; positions (and the
  * orientations of non-spheres) that are not given, or that equal bit for bit
- * the state hlbm_particle_state returned after the current step, keep the
- * moments form of the momentum exchange.  HLBM_ERR_ARG (nothing
- * changed) for a non-finite position or a zero or non-finite quaternion. */
+ * the state hlbm_particle_state returned after the current step, are none.
+ * HLBM_ERR_ARG (nothing changed) for a non-finite position or a zero or
+ * non-finite quaternion. */
 int hlbm_set_particle_state(hlbm_handle h, const double* X, const double* U, const double* omega,
                             const double* quat);
 
@@ -210,8 +210,11 @@ int hlbm_set_contact(hlbm_handle h, double k, double zeta);
 
 /* Queues nsteps >= 0 time steps (Algorithm 1: momentum exchange, external
  * force, Newton-Euler update, particle work lists, EDM coupling, collision
- * and streaming) on the stream and returns without waiting.  Errors found by
- * the GPU are reported by the next call that synchronises. */
+ * and streaming) on the stream and returns without waiting.  A run is taken
+ * in captured graphs of 8, 4, 2 and 1 steps, each built when a run first
+ * asks for it after a change of parameters (20 to 60 us of host time
+ * each).  Errors found by the GPU are reported by the next call that
+ * synchronises. */
 int hlbm_step(hlbm_handle h, int nsteps);
 
 /* Waits for the stream and returns HLBM_OK or the error the GPU flagged
@@ -246,8 +249,8 @@ long long hlbm_steps_done(hlbm_handle h);
  * 32 x tile_y x tile_z cells, tile_y and tile_z in {1, 2, 4, 8}, with
  * cells_x = 1 or 2 x-adjacent cells per thread (32 x tile_y or 16 x tile_y
  * threads); cells_x = 2 is the default, with tile_y = 4 and a tile_z that
- * follows the lattice's size until this call or hlbm_autotune.  Both compute the same step; their
- * results differ by FP32 rounding order only. */
+ * follows the lattice's size until this call or hlbm_autotune.  Both compute
+ * the same step; their results differ by FP32 rounding order only. */
 int hlbm_set_launch(hlbm_handle h, int tile_y, int tile_z, int cells_x);
 int hlbm_get_launch(hlbm_handle h, int* tile_y, int* tile_z, int* cells_x);
 
@@ -257,9 +260,9 @@ int hlbm_get_launch(hlbm_handle h, int* tile_y, int* tile_z, int* cells_x);
  *   HLBM_MEA_MOMENTS  per interior cell, the momentum the cell gained by the last
  *                     streaming minus u_p times the mass it gained, from the
  *                     moments of what arrived and of what the collision sent
- *                     out, added in fixed point (no order).  The link sums still
- *                     run on the first step after any change of state.  Needs
- *                     max_particles > 0.
+ *                     out, added in fixed point (no order).  The link sums
+ *                     run on the first step after any change of state.
+ *                     Needs max_particles > 0.
  * Both walk the cells of each particle and read the populations alone.
  * Both give the same force and torque up to FP32 summation order. */
 #define HLBM_MEA_KERNEL 0
@@ -307,8 +310,9 @@ int hlbm_interior_cells(hlbm_handle h, long long* n);
  * particle table with shapes and box ids, the step count (hence the AA
  * parity), the fluid force, the momentum-exchange mode and whether the next
  * step takes the moments form.  Launch shape and tuning are not part of it.
- * Snapshots of the version that kept a list of interior cells load as well.  The layout is host byte order with fixed-width fields; it is
- * meant for the same library on machines of the same byte order.
+ * Snapshots of the version that kept a list of interior cells load as well.
+ * The layout is host byte order with fixed-width fields; it is meant for the
+ * same library on machines of the same byte order.
  *
  * hlbm_checkpoint_bytes: *bytes = the size of a snapshot of the current
  * state.  Synchronises; returns the error the GPU flagged, if any (no

@@ -4,13 +4,13 @@
 // One time step (Algorithm 1 of arXiv:2312.14172, Sec. 4.2.5, without its
 // communication rows) is three launches on the handle's stream:
 //   1. momentum exchange per particle          (mea_kernel, mea_moments_kernel)
-//   2. contact forces, when switched on       (contact_kernel)
-//      external force, Newton-Euler, records,
+//   2. external force, Newton-Euler, records,
 //      per-tile particle lists                 (update_kernel; with few
 //                                              particles the exchange's blocks)
 //   3. EDM coupling, collision and streaming   (collide_pair_kernel,
 //                                              collide_stream_kernel)
-// Runs of 8, 4, 2 and 1 steps are captured as CUDA graphs, per parity of the
+// and one more, of contact forces, before them when contact is switched on
+// (contact_kernel).  Runs of 8, 4, 2 and 1 steps are captured as CUDA graphs, per parity of the
 // first step and form of the exchange, when a run first asks for them.
 #include <algorithm>
 #include <cmath>
@@ -185,8 +185,11 @@ struct hlbm_ctx {
   // captured steps [steps per graph][moments form in the first][parity], built
   // when a run first asks for them
   cudaGraphExec_t exec[GRAPH_KINDS][2][2] = {};
-  // the last collision knew this particle state, so in the moments mode the
-  // momentum exchange takes the moments form
+  // the next step's momentum exchange takes the moments form: in the moments
+  // mode, unless the particles or populations were set since the last step.
+  // The form reads the present populations and records alone and holds after
+  // such a change too; the link sums there keep the bits of runs that begin
+  // with or contain one
   bool moments_valid = false;
   bool split = false;  // a split step is open
   // hstage holds the device's particle rows X .. T as downloaded by
@@ -292,9 +295,8 @@ static PartArgs part_args(const hlbm_ctx* h, int parity, bool moments = false) {
   return a;
 }
 
-// moments: the momentum exchange of this step takes the moments form (the
-// collision of the previous step knew the particle state); otherwise the link
-// sums (always on the first step after a change of state).
+// moments: the momentum exchange of this step takes the moments form,
+// otherwise the link sums (always on the first step after a change of state).
 // Kernels captured into a step's graph use programmatic dependent launch.
 static cudaError_t enqueue_step(hlbm_ctx* h, int parity, bool moments, cudaStream_t s) {
   cudaError_t e;
@@ -1034,10 +1036,10 @@ int hlbm_set_particle_state(hlbm_handle h, const double* X, const double* U, con
   // the staging rows may still feed the previous upload
   CK(cudaEventSynchronize(h->hstage_ev));
   double* S = h->hstage;  // row r holds component r of the state, n doubles
-  // The moments form needs a collision that knew the same interior cells,
-  // and those depend on positions and, for non-spheres, orientations only:
-  // when both come back as the state downloaded after this very step, bit
-  // for bit, the next step may still take it.
+  // A state that comes back as downloaded after this very step, bit for bit,
+  // is no change of state: the next step keeps its form of the exchange.
+  // (Positions and, for non-spheres, orientations count; with them the cells
+  // inside the particles are the same.)
   const bool fresh = h->hst_valid && h->hst_steps == h->steps;
   bool moved = false;
   if (X)
@@ -1116,7 +1118,7 @@ int hlbm_set_owned_planes(hlbm_handle h, int box, int z_lo, int z_hi) {
   bd.own_hi = z_hi;
   CK(cudaMemcpyAsync(h->d_boxes + box, &bd, sizeof(BoxDesc), cudaMemcpyHostToDevice, h->stream));
   CK(cudaStreamSynchronize(h->stream));
-  h->moments_valid = false;  // the next step takes the link sums, over the new owned planes
+  h->moments_valid = false;  // a change of state: other cells enter the exchange
   return HLBM_OK;
 }
 

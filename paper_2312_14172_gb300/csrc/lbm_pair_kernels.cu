@@ -110,7 +110,8 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
   // FP16 432 -> 388) and where walls add to them (128^3 FP32 61.5 -> 57.1).
   // FP32 without walls waits for HBM instead, and there the pointer form's
   // slower stream of requests is the faster one (non-spherical 256^3 FP32 452
-  // against 465); an even step touches its own cells only.  Offsets within a
+  // against 465; boxes within L2 were not compared and take it too); an even
+  // step touches its own cells only.  Offsets within a
   // wider slice take 64 bits, and so the pointer form; as kernels of their own
   // those cost the others nothing (a branch between the forms spills a hundred
   // bytes of registers in the kernels without particles).  Boxes of rows of
@@ -147,7 +148,7 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
   const int y = k.y0 + threadIdx.y;
   const bool here = x0 < bd.nx && y < bd.ny;  // the other lanes leave below
   // an odd nx leaves one cell in a row's last pair: its second slot is the
-  // row's padding, computed but never stored, and the cell's right
+  // row's padding, which takes values that no cell reads, and the cell's right
   // neighbour is x0 + 1 wrapped (rb.dr, rb.wr refer to x0 + 1 there)
   const bool single = x0 + 1 == bd.nx;
   const RowBlocks rb = row_blocks<WALLS>(bd, x0, y, single ? 1 : 2);

@@ -392,9 +392,8 @@ __global__ void __launch_bounds__(XCH_MAX_T, 2) mea_kernel(PartArgs a) {
   move_particle(a, p, bd, R, mv);
 }
 
-// Momentum exchange of every particle in the moments form (after a collision
-// that knew the same particle state): same blocks of planes, sums in fixed
-// point.  It took the place of a list of interior cells that the collision
+// Momentum exchange of every particle in the moments form: blocks of whole
+// planes as above, sums in fixed point.  It took the place of a list of interior cells that the collision
 // wrote (cell, particle and departing moments, 24 bytes a cell) and a kernel
 // that walked it: the populations hold the departures too, the particle's
 // geometry gives the cells, and the collision is rid of the appends (us,
