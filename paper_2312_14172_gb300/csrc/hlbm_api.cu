@@ -10,8 +10,9 @@
 //   3. EDM coupling, collision and streaming   (collide_pair_kernel,
 //                                              collide_stream_kernel)
 // and one more, of contact forces, before them when contact is switched on
-// (contact_kernel).  Runs of 8, 4, 2 and 1 steps are captured as CUDA graphs, per parity of the
-// first step and form of the exchange, when a run first asks for them.
+// (contact_kernel).  Runs of 8, 4, 2 and 1 steps are captured as CUDA graphs,
+// per parity of the first step and form of the exchange, when a run first asks
+// for them.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
