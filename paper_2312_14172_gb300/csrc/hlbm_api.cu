@@ -156,6 +156,7 @@ struct hlbm_ctx {
   // with, still in L2); larger lattices gain nothing and keep one order
   bool reverse_odd = false;
   int prefetch = 0;  // rows a collision block prefetches at most
+  double touched = 0.0;         // about the tiles that each particle is a candidate of, summed
   std::vector<int> h_planes;    // bounding-box planes per particle
   int mea_group = 1;            // planes whose cells are summed together
   bool fused = false;           // the momentum exchange moves the particles too
@@ -371,20 +372,34 @@ static int need_run(hlbm_ctx* h, int nsteps) {
 // The bricks of the collision until the caller or the autotuner sets them:
 // 32 x 4 x 2 cells, or taller ones as long as they leave two and a half
 // resident waves of blocks (8 blocks of 64 threads per SM in FP32, 10 in
-// FP16).  A taller brick stages its candidates for more cells: 32x4x4 against
-// 32x4x2, collision in us: 128^3 FP16 45.3 / 47.8, non-spherical 256^3 FP32
-// 422 / 470; FP16, with its lighter slices, gains up to 32x4x8 (non-spherical
-// 256^3 387 / 398 / 445, dense 512x512x1024 4280 / 4549 / 5237), FP32 does not
-// (470 / 422).  Small lattices want the blocks (duct 101x67x83 18.1 / 15.3 us
-// a step), and so do distance grids, whose cells cost unevenly (128^3 FP16
-// 91 / 85).
+// FP16; duct 101x67x83 15.3 us a step with 4x2, 18.1 with 4x4).  A taller
+// brick stages its candidates for more cells, so what it gains grows with the
+// candidates of a tile; without any it loses in FP32 and gains a little, up to
+// 4x4, in FP16 with its lighter slices.  us a step, 4x2 / 4x4 / 4x8:
+//   candidates per tile    FP32                 FP16
+//   none, 128^3            40.3 / 41.5 / 42.9   30.6 / 30.1 / 32.8
+//   none, 256^3             369 /  374 /  425    250 /  244 /  252
+//   0.2, 128^3             55.3 / 54.3 / 55.2   43.5 / 41.0 / 43.4
+//   0.5, 256^3              411 /  419 /  484    310 /  274 /  275
+//   1.2, 512x512x256       1745 / 1787 / 2011   1340 / 1177 / 1132
+//   2.3, 256^3              497 /  491 /  560    415 /  371 /  352
+//   4.2, 160^3              152 /  146 /  164    132 /  124 /  126
+//   6, 256^3                659 /  602 /  641    600 /  548 /  525
+// Populations within twice the L2 (128^3, and 160^3 in FP16) do not wait for
+// HBM: any particles there make 4x4 the better one in FP32, and 4x8 none in
+// FP16.  Distance grids, whose cells cost unevenly, want the blocks (128^3
+// FP16 91 with 4x4, 85 with 4x2).
 static void default_launch(hlbm_ctx* h) {
   if (h->launch_set) return;
-  const bool half = h->prm.precision == HLBM_FP16;
+  const bool half = h->prm.precision == HLBM_FP16, in_l2 = h->reverse_odd;
   const long long resident = (long long)(h->nsm > 0 ? h->nsm : 152) * (half ? 10 : 8);
+  const double cand = h->touched / (double)h->L.ntiles;
   h->sub_z = 2;
   if (!h->grids.empty()) return;
-  for (int z = half ? 8 : 4; z > 2; z /= 2)
+  int tallest = 2;
+  if (half) tallest = !in_l2 && cand >= 0.5 ? 8 : 4;
+  else if (cand >= 2.0 || (in_l2 && cand > 0.0)) tallest = 4;
+  for (int z = tallest; z > 2; z /= 2)
     if (2 * h->L.ntiles * (TILE_Y / h->sub_y) * (TILE_Z / z) >= 5 * resident) {
       h->sub_z = z;
       break;
@@ -912,6 +927,7 @@ int hlbm_add_particles(hlbm_handle h, int n, const int* box_id, const int* shape
   std::vector<int> sh(n), bx(n), nch(n);
   std::vector<double> cells(n);
   std::vector<int> tile(n);
+  double touched = 0.0;
   auto T = [&](int fld, int k) -> double& { return tab[(size_t)fld * n + k]; };
   for (int k = 0; k < n; ++k) {
     const int b = box_id ? box_id[k] : 0;
@@ -998,6 +1014,7 @@ int hlbm_add_particles(hlbm_handle h, int n, const int* box_id, const int* shape
     bx[k] = b;
     nch[k] = (int)std::ceil(2.0 * rc) + 2;  // bounding-box planes, at most MAX_PLANES
     cells[k] = 1.3 * V;  // about the cells its momentum exchange walks
+    touched += (1.0 + 2.0 * rinf / TILE_X) * (1.0 + 2.0 * rinf / TILE_Y) * (1.0 + 2.0 * rinf / TILE_Z);
   }
   const int p0 = h->np;
   int rc = upload_fields(h, p0, n, tab);
@@ -1012,6 +1029,8 @@ int hlbm_add_particles(hlbm_handle h, int n, const int* box_id, const int* shape
   h->h_planes.insert(h->h_planes.end(), nch.begin(), nch.end());
   h->h_cells.insert(h->h_cells.end(), cells.begin(), cells.end());
   h->h_tile.insert(h->h_tile.end(), tile.begin(), tile.end());
+  h->touched += touched;
+  default_launch(h);
   rc = plan_exchange(h, p0);
   if (rc != HLBM_OK) return rc;
   CK(launch_records(part_args(h, 0), h->stream));

@@ -179,3 +179,35 @@ def test_slices_on_both_sides_of_four_gigabytes(H, precision, nx, bc, ny, nz, pa
     assert not torch.equal(*got)
     del got
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("precision,n,count,r,tile_z", [
+    ("fp32", (96, 96, 96), 0, 0.0, 2),      # too few blocks for taller bricks
+    ("fp16", (96, 96, 96), 50, 5.0, 2),
+    ("fp32", (128, 128, 128), 0, 0.0, 2),   # fluid alone
+    ("fp32", (128, 128, 128), 20, 6.0, 4),  # particles within twice the L2
+    ("fp16", (128, 128, 128), 0, 0.0, 4),
+    ("fp16", (160, 160, 160), 1200, 5.0, 4),
+    ("fp32", (256, 256, 256), 400, 6.0, 2),   # few candidates, streaming
+    ("fp32", (256, 256, 256), 2000, 6.0, 4),  # many
+    ("fp16", (256, 256, 256), 0, 0.0, 4),
+    ("fp16", (256, 256, 256), 2000, 6.0, 8),
+])
+def test_default_bricks_follow_size_and_particles(H, precision, n, count, r, tile_z):
+    """The default's tile_z is the fastest of 2, 4 and 8 as measured for such
+    handles, whether the particles come at once or in two calls; a launch
+    shape that was set stays."""
+    k = [int(v // (2 * r + 2)) if count else 1 for v in n]
+    site = np.arange(count)
+    X = (np.stack([site % k[0], site // k[0] % k[1], site // (k[0] * k[1])], 1) + 0.5) * (np.array(n) / k)
+    for calls in (1, 2):
+        for fixed in (False, True):
+            lat = H.Lattice([n + (0,)], H.make_params(precision=precision, max_particles=max(1, count)))
+            if fixed:
+                lat.set_launch(2, 1, 2)
+            for part in np.array_split(site, calls):
+                if len(part):
+                    lat.add_particles(np.zeros(len(part), int), np.full((len(part), 1), r), X[part],
+                                      rho_p=np.full(len(part), 2.0))
+            assert lat.get_launch() == ((2, 1, 2) if fixed else (4, tile_z, 2))
+            lat.close()
