@@ -184,6 +184,9 @@ struct hlbm_ctx {
   bool launch_set = false;
   int cells_x = 2;       // cells per thread along x
   bool wide_slices = false;  // a z slice of some box takes 4 GB or more
+  // half of the cells or more lie in boxes whose rows, of at most six storage
+  // blocks, end in a single cell with no wall in x
+  bool single_ends = false;
   // captured steps [steps per graph][moments form in the first][parity], built
   // when a run first asks for them
   cudaGraphExec_t exec[GRAPH_KINDS][2][2] = {};
@@ -243,6 +246,7 @@ static LbmArgs lbm_args(const hlbm_ctx* h, int parity) {
   a.nbricks = h->L.ntiles * a.nsub;
   a.reverse = parity && h->reverse_odd;
   a.wide = h->wide_slices;
+  a.single_ends = h->single_ends;
   a.prefetch = std::min(h->prefetch, h->sub_y * h->sub_z);
   a.omega = (float)(1.0 / h->prm.tau);
   for (int j = 0; j < 3; ++j) a.ff[j] = (float)h->prm.fluid_force[j];
@@ -460,11 +464,14 @@ int hlbm_init_batch(hlbm_handle* out, int nboxes, const hlbm_box* boxes, const h
   h->prm = *prm;
   if (h->prm.bin_capacity == 0) h->prm.bin_capacity = DEFAULT_BIN_CAP;
   h->stream = (cudaStream_t)cuda_stream;
+  long long ends = 0;  // cells of such boxes
   for (int b = 0; b < nboxes; ++b) {
     h->walls |= boxes[b].bc_flags != 0;
     const BoxDesc& d = h->boxes[b];
+    if ((d.nx & 1) && !(d.bc & 1) && d.ntx <= 6) ends += (long long)d.nx * d.ny * d.nz;
     h->wide_slices |= (unsigned long long)d.ny * d.ntx * QVB * (prm->precision == HLBM_FP32 ? 4 : 2) > 0xffffffffULL;
   }
+  h->single_ends = 2 * ends >= h->L.ncell;
   cudaError_t e;
   if (device_buf) {
     if (((uintptr_t)device_buf % ALIGN) || device_buf_bytes < h->L.total) {

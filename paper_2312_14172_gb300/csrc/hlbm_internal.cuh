@@ -285,6 +285,7 @@ struct LbmArgs {
   // bricks the step before ended with, whose populations L2 still holds
   int reverse;
   int wide;                 // a z slice of some box takes 4 GB or more
+  int single_ends;          // most cells lie in short rows that end in a single cell
   int prefetch;             // rows of its brick a block asks L2 for before its loads (0: none)
   float omega;              // 1 / tau
   float ff[3];              // fluid force density

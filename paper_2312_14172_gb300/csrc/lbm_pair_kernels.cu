@@ -100,8 +100,8 @@ template <typename S>
 struct PairBlocks { static constexpr int value = sizeof(S) == 4 ? HLBM_CP_MINBLOCKS_F32 : HLBM_CP_MINBLOCKS_F16; };
 
 // C: 0 no particles, 1 particles of the analytic shapes, 2 with distance
-// grids among them.  WIDE: a z slice of some box takes 4 GB or more (odd steps)
-template <typename S, int PAR, bool WALLS, int C, bool WIDE>
+// grids among them.  POINTERS: no 32-bit offsets (odd steps)
+template <typename S, int PAR, bool WALLS, int C, bool POINTERS>
 __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel(LbmArgs a) {
   constexpr bool COUPLE = C > 0;
   // Odd steps address the neighbour rows by 32-bit offsets (below): a tenth
@@ -111,15 +111,21 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
   // FP32 without walls waits for HBM instead, and there the pointer form's
   // slower stream of requests is the faster one (non-spherical 256^3 FP32 452
   // against 465; boxes within L2 were not compared and take it too); an even
-  // step touches its own cells only.  Offsets within a
-  // wider slice take 64 bits, and so the pointer form; as kernels of their own
-  // those cost the others nothing (a branch between the forms spills a hundred
-  // bytes of registers in the kernels without particles).  Boxes of rows of
-  // 8192 (FP32) or 16384 cells in 6 slices, ms a step, one cell per thread /
-  // pointers (6900 rows a slice, above 4 GB) / offsets (6898): FP32 with walls
-  // 8.82 / 7.83 / 7.74, FP16 12.12 / 10.50 / 10.73, with walls 15.28 / 11.82 /
-  // 11.12.
-  constexpr bool FAST = PAR == 1 && !WIDE && (sizeof(S) == 2 || WALLS);
+  // step touches its own cells only.
+  // POINTERS: the same by pointers, in kernels of their own (a branch between
+  // the forms spills a hundred bytes of registers in those without particles).
+  // For slices above 4 GB, whose offsets take 64 bits: rows of 8192 (FP32) or
+  // 16384 cells in 6 slices, ms a step, one cell per thread / pointers (6900
+  // rows a slice) / offsets (6898): FP32 with walls 8.82 / 7.83 / 7.74, FP16
+  // 12.12 / 10.50 / 10.73, with walls 15.28 / 11.82 / 11.12.  And for rows of up
+  // to 6 blocks that end in a single cell, between walls in y or z: the warps
+  // of a row's last block take its single end without the selects of walls
+  // here.  us a step, offsets / pointers, walls in z: fluid 33x300x300 FP32
+  // 116.8 / 110.5, FP16 83.7 / 76.7, 101x150x150 58.4 / 55.6, 42.2 / 40.2,
+  // 161x128x128 62.9 / 61.8, 43.8 / 42.9, there with 200 spheres 91.5 / 89.8,
+  // 74.1 / 70.8; longer rows gain less or lose (257x200x200 FP16 158.1 / 158.4,
+  // walls in y too 158.6 / 159.9).
+  constexpr bool FAST = PAR == 1 && !POINTERS && (sizeof(S) == 2 || WALLS);
   using T = Two<S>;
   __shared__ Rec srec[COUPLE ? MAX_CAND : 1];
   __shared__ Capsule scap[C == 1 ? MAX_CAND : 1];
@@ -156,12 +162,13 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
   const float sc = Pop<S>::SCALED ? a.scale : 1.0f, isc = Pop<S>::SCALED ? a.inv_scale : 1.0f;
 
   // Walls need selects in every direction, and so does a row's single last
-  // cell, but few warps hold such cells: they run the slice with the selects,
-  // all others without (a warp runs one of the two).
-  const bool special = single || (WALLS && (((bd.bc & 2) && (y == 0 || y == bd.ny - 1)) || rb.wl || rb.wr));
-  const bool plain_row = (FAST || (WIDE && WALLS)) && !__any_sync(lanes, here && special);
+  // cell by offsets, but few warps hold such cells: they run the slice with
+  // the selects, all others without (a warp runs one of the two).
+  const bool special = (!POINTERS && single) ||
+                       (WALLS && (((bd.bc & 2) && (y == 0 || y == bd.ny - 1)) || rb.wl || rb.wr));
+  const bool plain_row = (FAST || (POINTERS && WALLS)) && !__any_sync(lanes, here && special);
   if (!here) return;
-  // Byte offsets within a z slice (below 4 GB unless WIDE) of slot 0
+  // Byte offsets within a z slice (below 4 GB unless POINTERS) of slot 0
   // of x0 in the rows y - 1, y, y + 1, and from there to x0 - 1 and x0 + 2:
   // they hold for every slice, and with the slices' base addresses, which are
   // the same for the whole warp, address the slots in few instructions.
@@ -328,26 +335,26 @@ __global__ void __launch_bounds__(128, PairBlocks<S>::value) collide_pair_kernel
   for (int z = z0; z < z1; ++z) {
     const bool plain = plain_row && !(WALLS && (bd.bc & 4) && (z == 0 || z == nz - 1));
     if (FAST && plain) slice(std::true_type{}, std::false_type{}, z);
-    else if (WIDE && plain) slice(std::false_type{}, std::false_type{}, z);
+    else if (POINTERS && plain) slice(std::false_type{}, std::false_type{}, z);
     else slice(std::false_type{}, std::integral_constant<bool, WALLS>{}, z);
   }
   if (!early) pdl_trigger();
 }
 
-template <typename S, int PAR, bool W, int C, bool WIDE = false>
+template <typename S, int PAR, bool W, int C, bool POINTERS = false>
 static cudaError_t launch_cp(const LbmArgs& a, cudaStream_t s) {
   dim3 block(TILE_X / 2, a.sub_y);
   LbmArgs b = a;
   // resident blocks per SM as the launch bounds provide for (registers)
   b.pdl_tail = a.nsm > 0 ? (long long)a.nsm * (PairBlocks<S>::value * 128 / (int)(block.x * block.y))
                          : a.nbricks;
-  return launch_k(collide_pair_kernel<S, PAR, W, C, WIDE>, dim3((unsigned)a.nbricks), block, 0, s, a.pdl != 0, b);
+  return launch_k(collide_pair_kernel<S, PAR, W, C, POINTERS>, dim3((unsigned)a.nbricks), block, 0, s, a.pdl != 0, b);
 }
 
 template <typename S, int C>
 static cudaError_t launch_cp_c(const LbmArgs& a, int parity, bool walls, cudaStream_t s) {
   if (parity == 0) return launch_cp<S, 0, false, C>(a, s);
-  if (a.wide && walls) return launch_cp<S, 1, true, C, true>(a, s);
+  if ((a.wide || a.single_ends) && walls) return launch_cp<S, 1, true, C, true>(a, s);
   if (a.wide && sizeof(S) == 2) return launch_cp<S, 1, false, C, sizeof(S) == 2>(a, s);
   return walls ? launch_cp<S, 1, true, C>(a, s) : launch_cp<S, 1, false, C>(a, s);
 }

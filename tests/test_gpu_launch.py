@@ -211,3 +211,54 @@ def test_default_bricks_follow_size_and_particles(H, precision, n, count, r, til
                                       rho_p=np.full(len(part), 2.0))
             assert lat.get_launch() == ((2, 1, 2) if fixed else (4, tile_z, 2))
             lat.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp16"])
+@pytest.mark.parametrize("n,bc,particles", [
+    ((1, 20, 18), 2, 0), ((3, 9, 11), 6, 0), ((31, 18, 17), 4, 0), ((33, 40, 38), 2, 6), ((65, 37, 41), 6, 10),
+    ((191, 34, 36), 4, 20), ((193, 34, 36), 4, 20),  # the longest such rows, and longer ones
+])
+def test_single_ends_between_walls(H, precision, n, bc, particles):
+    """Rows that end in a single cell, between walls in y or z: alone such a
+    box takes its odd steps by pointers, beside a larger box of even rows by
+    32-bit offsets; the same step either way, within rounding as above."""
+    rng = np.random.default_rng(n[0])
+    k = [max(1, v // 12) for v in n]  # sites 12 cells apart or more, off the walls
+    site = rng.permutation(k[0] * k[1] * k[2])[:particles]
+    X = (np.stack([site % k[0], site // k[0] % k[1], site // (k[0] * k[1])], 1) + 0.5) * (np.array(n) / k)
+    r, U = rng.uniform(3.0, 5.5, (len(site), 1)), rng.uniform(-1e-3, 1e-3, (len(site), 3))
+    blocks = -(-n[0] // 32) * n[1] * n[2]
+    got = []
+    for beside in ([], [(n[0] + 1, n[1] + 1, n[2] + 1, bc)]):
+        lat = H.Lattice([n + (bc,)] + beside, H.make_params(tau=0.7, precision=precision, max_particles=max(1, particles)))
+        if particles:
+            lat.add_particles(np.zeros(len(site), int), r, X, U, U, None, np.full(len(site), 2.0))
+        _disturb(lat, precision, 13)
+        lat.set_launch(4, 2, 2)
+        lat.step(5)
+        lat.sync()
+        got.append(_fluid(lat, precision)[:blocks].clone())
+        lat.close()
+    assert _worst(*got, n[0], precision) <= (1e-6 if precision == "fp32" else 2e-5)
+
+
+def test_a_single_end_costs_little_more_than_a_pair(H):
+    """Rows of 33 and of 34 cells take the same blocks, rows and bytes: the
+    step of the odd ones, between walls, at most a tenth more."""
+    import torch
+    took = []
+    for nx in (33, 34):
+        lat = H.Lattice([(nx, 300, 300, 4)], H.make_params(tau=0.6, precision="fp16", fluid_force=(1e-7, 0, 0)))
+        times = []
+        for _ in range(7):
+            lat.step(16)
+            torch.cuda.synchronize()
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record(lat.stream)
+            lat.step(16)
+            e[1].record(lat.stream)
+            torch.cuda.synchronize()
+            times.append(e[0].elapsed_time(e[1]))
+        took.append(min(times))
+        lat.close()
+    assert took[0] <= 1.1 * took[1]
