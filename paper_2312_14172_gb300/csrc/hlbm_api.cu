@@ -43,7 +43,8 @@ const double PI_D = 3.14159265358979323846;
 size_t align_up(size_t v) { return (v + ALIGN - 1) / ALIGN * ALIGN; }
 
 struct Layout {
-  long long nblocks = 0, ncell = 0, ntiles = 0, stage_cells = 0;
+  long long nblocks = 0, ncell = 0, ntiles = 0;
+  long long stage_cells = 0, stage_f64 = 0;  // cells whose Q values the staging area holds, FP32 and FP64
   int cap = 0, bin_cap = 0;
   size_t off_f, off_boxes, off_P, off_shape, off_box, off_rec, off_part, off_acc, off_chunk[2], off_done,
       off_count, off_cnt[2], off_ids[2], off_status, off_stage, off_gdesc, off_gvals, total;
@@ -91,7 +92,8 @@ bool make_layout(int nb, const hlbm_box* boxes, const hlbm_params* prm, Layout& 
   L.nblocks = blocks;
   L.ncell = cells;
   L.ntiles = tiles;
-  L.stage_cells = maxbox < STAGE_CELLS ? maxbox : STAGE_CELLS;
+  L.stage_cells = std::min(maxbox, STAGE_CELLS);
+  L.stage_f64 = std::min(maxbox, STAGE_CELLS / 2);  // a box of up to 2^17 cells in one run
   L.cap = prm->max_particles;
   L.bin_cap = prm->bin_capacity ? prm->bin_capacity : DEFAULT_BIN_CAP;
   const size_t s = prm->precision == HLBM_FP32 ? 4 : 2;
@@ -112,7 +114,8 @@ bool make_layout(int nb, const hlbm_box* boxes, const hlbm_params* prm, Layout& 
     L.off_ids[k] = o; o = align_up(o + sizeof(int) * (size_t)L.ntiles * L.bin_cap);
   }
   L.off_status = o; o = align_up(o + sizeof(int));
-  L.off_stage = o; o = align_up(o + sizeof(float) * Q * (size_t)std::max(2LL, L.stage_cells));
+  L.off_stage = o;
+  o = align_up(o + Q * std::max(sizeof(float) * (size_t)L.stage_cells, sizeof(double) * (size_t)L.stage_f64));
   L.grid_floats = prm->grid_floats;
   L.off_gdesc = o; o = align_up(o + (L.grid_floats > 0 ? sizeof(GridDesc) * MAX_GRIDS : 0));
   L.off_gvals = o; o = align_up(o + sizeof(float) * (size_t)L.grid_floats);
@@ -1260,11 +1263,15 @@ int hlbm_particle_state(hlbm_handle h, double* X, double* U, double* omega, doub
 }  // extern "C"
 
 // n doubles of each of the Q rows of a host array of N per row, from cell c0
-// on, to or from the packed staging area: one strided copy where the rows
-// are within the runtime's largest pitch (2^31 - 1 bytes)
+// on, to or from the packed staging area: one copy where that is the whole
+// array, one strided copy where the rows are within the runtime's largest
+// pitch (2^31 - 1 bytes)
 static cudaError_t copy_rows(double* host, long long N, long long c0, double* stage, long long n, bool put,
                              cudaStream_t s) {
   const size_t w = sizeof(double) * n, pitch = sizeof(double) * N;
+  if (n == N)
+    return put ? cudaMemcpyAsync(stage, host, Q * w, cudaMemcpyHostToDevice, s)
+               : cudaMemcpyAsync(host, stage, Q * w, cudaMemcpyDeviceToHost, s);
   if (pitch <= 0x7fffffffULL)
     return put ? cudaMemcpy2DAsync(stage, w, host + c0, pitch, w, Q, cudaMemcpyHostToDevice, s)
                : cudaMemcpy2DAsync(host + c0, pitch, stage, w, w, Q, cudaMemcpyDeviceToHost, s);
@@ -1306,7 +1313,7 @@ int hlbm_get_populations(hlbm_handle h, int box, double* host_f) {
   if (!h) return HLBM_ERR_ARG;
   if (box < 0 || box >= (int)h->boxes.size() || !host_f) return fail(h, HLBM_ERR_ARG, "bad box or NULL array");
   const BoxDesc& bd = h->boxes[box];
-  const long long N = (long long)bd.nx * bd.ny * bd.nz, run = std::max(1LL, h->L.stage_cells / 2);
+  const long long N = (long long)bd.nx * bd.ny * bd.nz, run = h->L.stage_f64;
   double* stage = reinterpret_cast<double*>(h->stage);
   touch_pages(host_f, sizeof(double) * Q * N);
   for (long long c0 = 0; c0 < N; c0 += run) {
@@ -1322,7 +1329,7 @@ int hlbm_set_populations(hlbm_handle h, int box, const double* host_f) {
   if (!h) return HLBM_ERR_ARG;
   if (box < 0 || box >= (int)h->boxes.size() || !host_f) return fail(h, HLBM_ERR_ARG, "bad box or NULL array");
   const BoxDesc& bd = h->boxes[box];
-  const long long N = (long long)bd.nx * bd.ny * bd.nz, run = std::max(1LL, h->L.stage_cells / 2);
+  const long long N = (long long)bd.nx * bd.ny * bd.nz, run = h->L.stage_f64;
   double* stage = reinterpret_cast<double*>(h->stage);
   for (long long c0 = 0; c0 < N; c0 += run) {
     const long long n = std::min(run, N - c0);
