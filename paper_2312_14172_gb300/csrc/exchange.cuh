@@ -297,13 +297,14 @@ struct ExchangeRows {
 };
 static_assert(MAX_PLANES <= 256 && XCH_MAX_T <= 1 << 24, "packing of ExchangeRows::found");
 
-// Calls cell(x, y, z, rr) for every interior cell of planes [q0, q0 + nq) of
-// the particle's bounding box (rr its offset from the centre), spread over
-// the block's threads (blockDim.x a power of two; all of them call, it
-// synchronises).  One thread finds the x-range of one row; the rows' cells
-// are then flattened, so that lanes stay busy whatever the shape.
+// Calls cell(x, y, z, rr) for every interior cell of the planes of the
+// particle's bounding box from q0 on, and of the rows of each, that a block
+// takes (part is .z of its entry of PartArgs::chunks; rr the cell's offset from
+// the centre), spread over the block's threads (blockDim.x a power of two; all
+// of them call, it synchronises).  One thread finds the x-range of one row; the
+// rows' cells are then flattened, so that lanes stay busy whatever the shape.
 template <bool GRIDS, typename Cell>
-__device__ __forceinline__ void for_interior(const Rec& R, const BoxDesc& bd, int q0, int nq, GridSet grids,
+__device__ __forceinline__ void for_interior(const Rec& R, const BoxDesc& bd, int q0, int part, GridSet grids,
                                              ExchangeRows& sh, Cell cell) {
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const GridSet gs = GRIDS ? grids : GridSet{};
@@ -313,7 +314,9 @@ __device__ __forceinline__ void for_interior(const Rec& R, const BoxDesc& bd, in
   exchange_extent(R.xh[0], rc, bd.bc & 1, 0, bd.nx - 1, lox, extx);
   exchange_extent(R.xh[1], rc, bd.bc & 2, 0, bd.ny - 1, loy, exty);
   exchange_extent(R.xh[2], rc, bd.bc & 4, cutz ? bd.own_lo : 0, cutz ? bd.own_hi - 1 : bd.nz - 1, loz, extz);
-  const int planes = min(nq, extz - q0);
+  loy += (part >> 8) & 0xff;
+  exty = max(min(exty - ((part >> 8) & 0xff), part >> 16), 0);
+  const int planes = min(part & 0xff, extz - q0);
   const int rows = planes > 0 ? planes * exty : 0;
   Capsule cap = capsule_of(R, 0.0f);
   if (GRIDS && R.shape == 4 && gs.desc) {  // the interior only

@@ -38,6 +38,7 @@ namespace {
 constexpr size_t ALIGN = 256;
 constexpr int DEFAULT_BIN_CAP = 64;
 constexpr long long STAGE_CELLS = 1 << 18;
+constexpr int MORE_CHUNKS = 112;  // blocks of the moments form beyond MAX_PLANES per particle, in all
 const double PI_D = 3.14159265358979323846;
 
 size_t align_up(size_t v) { return (v + ALIGN - 1) / ALIGN * ALIGN; }
@@ -106,7 +107,10 @@ bool make_layout(int nb, const hlbm_box* boxes, const hlbm_params* prm, Layout& 
   L.off_rec = o; o = align_up(o + sizeof(Rec) * (size_t)L.cap);
   L.off_part = o; o = align_up(o + sizeof(double) * 6 * MAX_PLANES * (size_t)L.cap);
   L.off_acc = o; o = align_up(o + sizeof(double) * 6 * (size_t)L.cap);
-  for (int k = 0; k < 2; ++k) { L.off_chunk[k] = o; o = align_up(o + sizeof(int4) * MAX_PLANES * (size_t)L.cap); }
+  for (int k = 0; k < 2; ++k) {
+    L.off_chunk[k] = o;
+    o = align_up(o + sizeof(int4) * (MAX_PLANES * (size_t)L.cap + (L.cap ? MORE_CHUNKS : 0)));
+  }
   L.off_done = o; o = align_up(o + sizeof(int) * (size_t)L.cap);
   L.off_count = o; o = align_up(o + sizeof(unsigned long long));
   for (int k = 0; k < 2; ++k) {
@@ -866,7 +870,11 @@ int hlbm_add_grid(hlbm_handle h, int nx, int ny, int nz, double spacing, const f
 // 200 spheres FP32 35 / 38 / 57, 495 spheres 64 / 50 / 51, 2000 ellipsoids
 // and cuboids 249 / 174 / 170, 50 000 spheres FP16 2869 / 1813 / 1470).
 // In the moments form neither is: there a block takes about as many cells
-// as its threads walk in six (few particles) or twenty (many) rounds.
+// as its threads walk in six (few particles) or twenty (many) rounds, or, where
+// that leaves SMs without a block, at least one and a half: in whole planes
+// or, beyond a block a plane, in bands of their rows (one sphere in 80^3 FP16,
+// us a step with planes / bands: radius 15 22.3 / 20.6, 20 25.5 / 22.1, 25 30.3
+// / 25.1, 29 35.0 / 28.6).
 static int plan_exchange(hlbm_ctx* h, int p0) {
   const int nsm = h->nsm > 0 ? h->nsm : 152;
   long long planes = 0;
@@ -908,13 +916,21 @@ static int plan_exchange(hlbm_ctx* h, int p0) {
     h->mea_threads[form] = t;
     ck[form].reserve(h->np);
     for (int p : order) {
-      // whole groups of planes per block
-      const int g = form ? 1 : G, groups = (h->h_planes[p] + g - 1) / g;
-      int want = form ? (int)std::ceil(h->h_cells[p] / ((few ? 6.0 : 20.0) * t)) : (h->h_planes[p] + 23) / 24;
-      // at least a block (three) per SM
-      want = std::max(1, std::max(want, (form ? 1 : 3) * nsm / h->np));
-      const int per = (groups + want - 1) / want, parts = (groups + per - 1) / per;
-      for (int k = 0; k < parts; ++k) ck[form].push_back(make_int4(p, k * per * g, per * g, parts));
+      const int E = h->h_planes[p];
+      if (form == 0) {  // whole groups of planes per block, at least three blocks per SM
+        const int groups = (E + G - 1) / G, want = std::max(1, std::max((E + 23) / 24, 3 * nsm / h->np));
+        const int per = (groups + want - 1) / want, parts = (groups + per - 1) / per;
+        for (int k = 0; k < parts; ++k) ck[0].push_back(make_int4(p, k * per * G, per * G, parts));
+        continue;
+      }
+      const double cells = h->h_cells[p] / t;
+      int want = std::max(1, (int)std::ceil(cells / (few ? 6.0 : 20.0)));
+      want = std::max(want, std::min(nsm / h->np, std::max(E, (int)std::ceil(cells / 1.5))));
+      const int bands = std::min((want + E - 1) / E, (MAX_PLANES + MORE_CHUNKS / h->np) / E);  // per plane
+      const int per = bands > 1 ? 1 : (E + want - 1) / want, planes = (E + per - 1) / per;
+      const int rows = (E + bands - 1) / bands, parts = planes * ((E + rows - 1) / rows);
+      for (int k = 0; k < planes; ++k)
+        for (int y = 0; y < E; y += rows) ck[1].push_back(make_int4(p, k * per, per | y << 8 | rows << 16, parts));
     }
     h->nchunks[form] = (int)ck[form].size();
     CK(cudaMemcpyAsync(h->chunks[form], ck[form].data(), sizeof(int4) * ck[form].size(), cudaMemcpyHostToDevice,

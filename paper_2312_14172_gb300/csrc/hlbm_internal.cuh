@@ -313,8 +313,10 @@ struct PartArgs {
   // momentum exchange input
   const void* f;            // populations, blocked layout
   float scale, inv_scale;
-  // momentum exchange: block k walks part of particle chunks[k].x, from plane
-  // chunks[k].y on chunks[k].z planes; the particle has chunks[k].w blocks
+  // momentum exchange: block k walks part of particle chunks[k].x, which has
+  // chunks[k].w blocks, from plane chunks[k].y on: chunks[k].z planes (link
+  // sums); chunks[k].z & 0xff planes, of each the rows from chunks[k].z >> 8 & 0xff
+  // on, chunks[k].z >> 16 of them (moments form)
   const int4* chunks;
   int nchunks;
   int mea_group;            // planes whose cells are summed together

@@ -352,3 +352,46 @@ def test_a_small_box_exchanges_its_populations_in_one_run(H, what):
         took.append(np.median(times))
         lat.close()
     assert took[0] <= 7 / 6 * took[1]
+
+
+@pytest.mark.parametrize("bc", [0, 7])
+@pytest.mark.parametrize("shape,a", [(0, (16.0, 16.0, 16.0)), (0, (20.0, 20.0, 20.0)), (0, (25.0, 25.0, 25.0)),
+                                     (1, (12.0, 18.0, 26.0)), (2, (13.0, 17.0, 15.0))])
+def test_large_particles_in_bands_of_rows(H, O, shape, a, bc):
+    """One large particle is walked by several blocks a plane, each a band of
+    its rows: every interior cell once, force and torque within 1e-5."""
+    n = (73, 70, 71)
+    X = [(36.4, 34.7, 36.1)] if bc else [(2.3, 69.2, 35.6)]  # inside; across two faces
+    q = np.array([[0.8, 0.3, -0.4, 0.33]])
+    lat, orc = _pair(H, O, n, bc, ([shape], [a], X, q / np.linalg.norm(q)), "moments")
+    lat.step(1)
+    orc.step(1)
+    assert lat.interior_cells() == orc.mea(0)[2] > 0
+    _steps_agree(lat, orc, 2)
+
+
+def test_a_large_particles_exchange_fills_the_gpu(H):
+    """The cells of a sphere of radius 25, 4.6 times those of radius 15, spread
+    over the SMs: a step of the same box at most 1.28 times as long (two of the
+    seven rounds of 256 threads that a whole plane takes stay on the critical
+    path instead of all)."""
+    import torch
+    took = []
+    for r in (15.0, 25.0):
+        lat = H.Lattice([(80, 80, 80, 0)], H.make_params(tau=0.6, max_particles=1))
+        lat.add_particles([0], [[r] * 3], [[40.0, 40.0, 40.0]], rho_p=[2.0])
+        lat.set_mea_mode("moments")
+        lat.step(1)
+        times = []
+        for _ in range(9):
+            lat.step(40)
+            torch.cuda.synchronize()
+            e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            e[0].record(lat.stream)
+            lat.step(40)
+            e[1].record(lat.stream)
+            torch.cuda.synchronize()
+            times.append(e[0].elapsed_time(e[1]))
+        took.append(min(times))
+        lat.close()
+    assert took[1] <= 1.28 * took[0]
