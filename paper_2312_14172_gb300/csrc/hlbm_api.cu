@@ -396,10 +396,15 @@ static int need_run(hlbm_ctx* h, int nsteps) {
 //   2.3, 256^3              497 /  491 /  560    415 /  371 /  352
 //   4.2, 160^3              152 /  146 /  164    132 /  124 /  126
 //   6, 256^3                659 /  602 /  641    600 /  548 /  525
-// Populations within twice the L2 (128^3, and 160^3 in FP16) do not wait for
-// HBM: any particles there make 4x4 the better one in FP32, and 4x8 none in
-// FP16.  Distance grids, whose cells cost unevenly, want the blocks (128^3
-// FP16 91 with 4x4, 85 with 4x2).
+// So boxes of a million cells that fill their bricks in y and z take the lower
+// of two heights while they have few candidates; elongated ones, whose capsules
+// a block computes, count more (100 capsules between walls in 192^3, 0.6 a
+// tile, FP32 4x2 207, 4x4 197, FP16 4x4 162, 4x8 155).  Batches of small boxes,
+// whose blocks look up their box, and thin boxes take the taller ones (200 boxes
+// of 32^3 FP32 173 / 167, 8 of 128^3 382 / 392; 2000x3x2000 302 / 273).  Populations within twice the L2 (128^3, and 160^3 in
+// FP16) do not wait for HBM: any particles there make 4x4 the better one in
+// FP32, and 4x8 gains with elongated ones alone in FP16.  Distance grids, whose
+// cells cost unevenly, want the blocks (128^3 FP16 91 with 4x4, 85 with 4x2).
 static void default_launch(hlbm_ctx* h) {
   if (h->launch_set) return;
   const bool half = h->prm.precision == HLBM_FP16, in_l2 = h->reverse_odd;
@@ -407,9 +412,15 @@ static void default_launch(hlbm_ctx* h) {
   const double cand = h->touched / (double)h->L.ntiles;
   h->sub_z = 2;
   if (!h->grids.empty()) return;
-  int tallest = 2;
-  if (half) tallest = !in_l2 && cand >= 0.5 ? 8 : 4;
-  else if (cand >= 2.0 || (in_l2 && cand > 0.0)) tallest = 4;
+  long long yz = 0, padded = 0;
+  for (const BoxDesc& d : h->boxes) {
+    yz += (long long)d.ny * d.nz;
+    padded += (long long)d.nty * TILE_Y * d.ntz * TILE_Z;
+  }
+  const bool full = (h->boxes.size() == 1 || h->L.ncell >= (long long)h->boxes.size() << 20) && 10 * yz >= 7 * padded;
+  const bool few = half ? cand < 0.5 || (in_l2 && !h->elongated)
+                        : cand < (h->elongated ? 0.5 : 2.0) && !(in_l2 && cand > 0.0);
+  const int tallest = (half ? 8 : 4) / (full && few ? 2 : 1);
   for (int z = tallest; z > 2; z /= 2)
     if (2 * h->L.ntiles * (TILE_Y / h->sub_y) * (TILE_Z / z) >= 5 * resident) {
       h->sub_z = z;

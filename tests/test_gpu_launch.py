@@ -262,3 +262,30 @@ def test_a_single_end_costs_little_more_than_a_pair(H):
         took.append(min(times))
         lat.close()
     assert took[0] <= 1.1 * took[1]
+
+
+@pytest.mark.parametrize("precision,boxes,tile_z", [
+    ("fp32", [(32, 32, 32)] * 200, 4), ("fp16", [(32, 32, 32)] * 200, 8),    # many small boxes
+    ("fp32", [(128, 128, 128)] * 8, 2), ("fp16", [(128, 128, 128)] * 8, 4),  # few large ones
+    ("fp32", [(2000, 3, 2000)], 4), ("fp16", [(2000, 3, 2000)], 8),          # bricks mostly empty in y
+])
+def test_default_bricks_of_batches_and_thin_boxes(H, precision, boxes, tile_z):
+    """As above, fluid alone: the height measured as the fastest of 2, 4 and 8,
+    or within 4 % of it and the one that such handles took before."""
+    lat = H.Lattice([b + (0,) for b in boxes], H.make_params(precision=precision))
+    assert lat.get_launch() == (4, tile_z, 2)
+    lat.close()
+
+
+@pytest.mark.parametrize("precision,few,many", [("fp32", 2, 4), ("fp16", 4, 8)])
+def test_default_bricks_with_elongated_particles(H, precision, few, many):
+    """Capsules count from half a candidate per tile on."""
+    n = (256, 256, 256)
+    lat = H.Lattice([n + (0,)], H.make_params(precision=precision, max_particles=400))
+    g = np.arange(400)
+    X = np.stack([g % 8, g // 8 % 8, g // 64], 1) * 30.0 + 20.0
+    lat.add_particles([3] * 100, [[4.0, 4.0, 6.0]] * 100, X[:100], rho_p=[2.0] * 100)
+    assert lat.get_launch() == (4, few, 2)
+    lat.add_particles([3] * 300, [[4.0, 4.0, 6.0]] * 300, X[100:], rho_p=[2.0] * 300)
+    assert lat.get_launch() == (4, many, 2)
+    lat.close()
