@@ -417,7 +417,8 @@ static void default_launch(hlbm_ctx* h) {
     yz += (long long)d.ny * d.nz;
     padded += (long long)d.nty * TILE_Y * d.ntz * TILE_Z;
   }
-  const bool full = (h->boxes.size() == 1 || h->L.ncell >= (long long)h->boxes.size() << 20) && 10 * yz >= 7 * padded;
+  const bool large = h->boxes.size() == 1 || h->L.ncell >= (long long)h->boxes.size() << 20;
+  const bool full = large && 10 * yz >= 7 * padded;
   const bool few = half ? cand < 0.5 || (in_l2 && !h->elongated)
                         : cand < (h->elongated ? 0.5 : 2.0) && !(in_l2 && cand > 0.0);
   const int tallest = (half ? 8 : 4) / (full && few ? 2 : 1);
